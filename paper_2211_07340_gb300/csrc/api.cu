@@ -75,6 +75,8 @@ haru::LaunchCfg haru_ctx::launch_cfg() const {
 haru::RefView haru_ctx::ref_view() const {
   haru::RefView r;
   r.img16 = img16;
+  r.imgh = imgh;
+  r.max_code = max_code;
   r.img32 = img32;
   r.N = static_cast<long>(N);
   r.scale_log2 = scale_log2;
@@ -85,14 +87,11 @@ namespace haru {
 
 // Reference and launch settings of a context, for haru_sdtw_batch_noalloc
 // (noalloc.cu). Reads state only; allocates nothing.
-int ctx_reference(haru_ctx *ctx, int precision, const void **img, long *N, int *scale_log2, int *device,
-                  cudaStream_t *stream, int *warps, int *tile, unsigned long long *wait, int *per_sm, int *sms) {
+int ctx_reference(haru_ctx *ctx, RefView *ref, int *device, cudaStream_t *stream, int *warps, int *tile, unsigned long long *wait, int *per_sm, int *sms) {
   std::lock_guard<std::mutex> lk(ctx->mu);
   if (ctx->sticky) return ctx->sticky;
   if (ctx->N == 0) return HARU_ENOREF;
-  *img = precision != HARU_FP32 ? static_cast<const void *>(ctx->img16) : static_cast<const void *>(ctx->img32);
-  *N = static_cast<long>(ctx->N);
-  *scale_log2 = ctx->scale_log2;
+  *ref = ctx->ref_view();
   *device = ctx->device;
   *stream = ctx->stream;
   *warps = pick_warps(ctx->cfg);
@@ -207,6 +206,7 @@ void haru_destroy(haru_ctx *ctx) {
   for (void *p : ptrs)
     if (p) cudaFree(p);
   free_ref_image(ctx->img16);
+  free_ref_image(ctx->imgh);
   free_ref_image(ctx->img32);
   haru::ws_free(ctx->ws);
   for (auto e : ctx->ev)
@@ -225,41 +225,48 @@ static int ref_install(haru_ctx *ctx, const float *x_dev, size_t n, int normaliz
   const size_t img_len = n + haru::kRefPad;
   const size_t all = static_cast<size_t>(haru::kRefFront) + img_len;
   float *z = nullptr, *i32b = nullptr;
-  uint32_t *i16b = nullptr;
+  uint32_t *i16b = nullptr, *ihb = nullptr;
   cudaError_t e = cudaMalloc(&z, n * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&i16b, all * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&ihb, all * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&i32b, all * sizeof(float));
   if (e != cudaSuccess) {
-    cudaFree(z); cudaFree(i16b); cudaFree(i32b);
+    cudaFree(z); cudaFree(i16b); cudaFree(ihb); cudaFree(i32b);
     cudaGetLastError();
     return HARU_ENOMEM;
   }
-  uint32_t *i16 = i16b + haru::kRefFront;
+  uint32_t *i16 = i16b + haru::kRefFront, *ih = ihb + haru::kRefFront;
   float *i32 = i32b + haru::kRefFront;
   const size_t nb = (n + 4095) / 4096;
-  int st = 0;
+  // status, and the largest |code| in the words after it
+  int st[2] = {0, 0};
   e = grow(&ctx->partials, &ctx->partials_cap, nb);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws.ints, 0, sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws.ints, 0, sizeof(st), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(i16b, 0, all * sizeof(uint32_t), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ihb, 0, all * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(i32b, 0, all * sizeof(float), s);
   if (e == cudaSuccess && normalize)
     e = haru::launch_zscore_stats(x_dev, n, ctx->partials, ctx->stats, ctx->ws.ints, s);
   if (e == cudaSuccess)
-    e = haru::launch_ref_finish(x_dev, n, ctx->stats, normalize, scale_log2, z, i16, i32, img_len, ctx->ws.ints, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&st, ctx->ws.ints, sizeof(int), cudaMemcpyDeviceToHost, s);
+    e = haru::launch_ref_finish(x_dev, n, ctx->stats, normalize, scale_log2, z, i16, ih, i32, ctx->ws.ints,
+                                ctx->ws.ints + 1, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(st, ctx->ws.ints, sizeof(st), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess || st != HARU_OK) {  // the previous reference stays in place
-    const int rc = e != cudaSuccess ? cuda_fail(ctx, e) : st;
+  if (e != cudaSuccess || st[0] != HARU_OK) {  // the previous reference stays in place
+    const int rc = e != cudaSuccess ? cuda_fail(ctx, e) : st[0];
     cudaStreamSynchronize(s);
-    cudaFree(z); cudaFree(i16b); cudaFree(i32b);
+    cudaFree(z); cudaFree(i16b); cudaFree(ihb); cudaFree(i32b);
     return rc;
   }
   cudaFree(ctx->ref_z);
   free_ref_image(ctx->img16);
+  free_ref_image(ctx->imgh);
   free_ref_image(ctx->img32);
   ctx->ref_z = z;
   ctx->img16 = i16;
+  ctx->imgh = ih;
   ctx->img32 = i32;
+  ctx->max_code = st[1];
   ctx->N = n;
   ctx->scale_log2 = scale_log2;
   return HARU_OK;

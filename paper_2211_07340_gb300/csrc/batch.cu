@@ -148,7 +148,11 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
 
   SdtwArgs sa;
   const bool fp_ref = precision == HARU_FP32 || precision == kPrecF32Span;
-  sa.ref_img = fp_ref ? static_cast<const void *>(ref.img32) : static_cast<const void *>(ref.img16);
+  sa.ref_img = fp_ref ? static_cast<const void *>(ref.img32)
+                      : static_cast<const void *>(precision == HARU_INT16 ? ref.imgh : ref.img16);
+  sa.ref_large = ref.img16;
+  sa.half_max = kHalfSpan - ref.max_code;
+  sa.large_possible = precision == HARU_INT16 && large_codes_possible(ref, raw);
   sa.N = ref.N;
   sa.img = ws.img;
   sa.items = ws.items;

@@ -64,11 +64,24 @@ inline size_t items_bound(int mode, size_t nq) {
 
 // The reference as the kernels read it.
 struct RefView {
-  const uint32_t *img16 = nullptr;
+  const uint32_t *img16 = nullptr;  // (r | r << 16), two's complement codes
+  const uint32_t *imgh = nullptr;   // (h | h << 16), half codes
   const float *img32 = nullptr;
   long N = 0;
   int scale_log2 = 6;
+  int max_code = 0;  // largest |r|
 };
+
+// Whether an int16 batch can hold a query code too large for the half-code
+// cell (|q| > kHalfSpan - the reference's largest code). Raw queries are
+// z-scored over their own m events, so |z| <= sqrt(m - 1) < 22.7 for m <= 512
+// (the largest deviation of m values with population sigma 1); 22.7 * 2^k + 1
+// covers the roundings. With a 2^6 scale and a reference within 9 sigma that
+// bound clears every raw batch, and the large-code sweep is not launched.
+inline int large_codes_possible(const RefView &r, int raw) {
+  const double bound = raw ? 22.7 * static_cast<double>(1 << r.scale_log2) + 1.0 : static_cast<double>(kQmax);
+  return bound > static_cast<double>(kHalfSpan - r.max_code) && kQmax > kHalfSpan - r.max_code ? 1 : 0;
+}
 
 // Device scratch of one batch in flight: status/counter words, planner
 // output, packed query images, segment states and per-unit minima.
@@ -147,6 +160,8 @@ struct haru_ctx {
   int scale_log2 = 6;
   float *ref_z = nullptr;       // N
   uint32_t *img16 = nullptr;    // N + kRefPad, packed (q, q)
+  uint32_t *imgh = nullptr;     // N + kRefPad, packed half codes
+  int max_code = 0;             // largest |q|
   float *img32 = nullptr;       // N + kRefPad
   double *stats = nullptr;      // mean, sigma
   double *partials = nullptr;

@@ -16,7 +16,6 @@ namespace haru {
 // 16-bit halves of every register (INT16 pair), or one query whose int16
 // codes are computed exactly in FP32 (wide accumulation). qb < 0 when a pair
 // is short. Its steps are cut into nseg segments (work units).
-constexpr int kItemF32 = 0, kItemPair = 1, kItemExact = 2;
 // A stacked item holds two strips one above the other in the warp's PE
 // chain: lanes 0..15 sweep qa (and qb, INT16), lanes 16..31 sweep qc (and
 // qd), each 16 * S rows high; lane 16 starts its stack from the free-start
@@ -26,7 +25,7 @@ struct Item {
   int qb;
   int S;        // rows per lane of the warp strip: 32 * S (16 * S if stacked) >= longest query
   int nseg;     // segments of its sweep
-  int kind;     // kItemF32, kItemPair or kItemExact
+  int qmax;     // INT16: largest |code| of its queries (written by the packing kernel)
   int qc;       // stacked: lower stack's queries (-1: none)
   int qd;
   int stacked;  // 1: two stacks of 16 lanes
@@ -57,9 +56,10 @@ struct Best {
   int64_t ca, cb;
 };
 
-// Per-item register image: [2][S][32] 32-bit words (INT16: packed query
-// codes q and their negations -q, both -4095 on pad rows; FP32: query
-// samples (0 on pad rows) and row weights, -1 on real rows and 0 on pad rows).
+// Per-item register image: [2][S][32] 32-bit words (INT16: the packed query
+// codes as sign-magnitude halves, kPadHalf on pad rows, then as two's
+// complement, kPadCode on pad rows; FP32: query samples (0 on pad rows) and
+// row weights, -1 on real rows and 0 on pad rows).
 constexpr int kImgStride = 2 * 16 * 32;
 // A saved strip state: the last two oblique columns, [2][S][32] words (the
 // start-column forms follow them with their start columns, as many words).
@@ -67,6 +67,17 @@ constexpr int kStateStride = 2 * 16 * 32;
 constexpr int kMaxS = 16;
 constexpr int kMaxSeg = 64;
 constexpr int kQmax = HARU_INT16_QMAX;
+// An int16 code as a sign-magnitude half is the fp16 number code * 2^-24 (a
+// subnormal up to 1023, then the first normal binade, whose spacing is the
+// same): differences of two codes are exact in fp16 up to 2^11, and the
+// result's low 11 bits are the distance |q - r| itself. A pad row holds
+// 2^15 (0x7800): minus any code it stays 2^15, whose low 11 bits are 0.
+constexpr int kHalfSpan = 2047;      // largest |q| + |r| the 11 bits hold
+constexpr uint32_t kPadHalf = 0x7800u;
+constexpr int kPadCode = -4095;      // two's complement image: distance 0 through the relu
+__host__ __device__ constexpr uint32_t half_code(int q) {
+  return q < 0 ? 0x8000u | static_cast<uint32_t>(-q) : static_cast<uint32_t>(q);
+}
 constexpr int kCap = HARU_INT16_CAP;
 // Extra reference columns past N that the tile stream may read: the lane
 // skew of the tallest strip (32 * 16) plus one whole tile.
@@ -83,6 +94,9 @@ static_assert(kRefFront >= 31 * kMaxS && kRefFront % 16 == 0, "front pad: the la
 // HARU_INT16 and HARU_INT16_ACC32: the FP32 and wide forms that also carry
 // each alignment's start column (haru_sdtw_batch_span).
 constexpr int kPrecF32Span = 3, kPrecWideSpan = 4;
+// and the int16 form for groups whose codes are too large for the half-code
+// cell (kHalfSpan).
+constexpr int kPrecI16Large = 5;
 __host__ __device__ constexpr bool prec_span(int p) { return p == kPrecF32Span || p == kPrecWideSpan; }
 // Tracking-ring words per warp: costs (and start columns, +128, for the span forms).
 // Words of one flush buffer of a warp's last-row tracking ring: a whole
@@ -91,7 +105,7 @@ __host__ __device__ constexpr bool prec_span(int p) { return p == kPrecF32Span |
 // columns keep two more for the starts. Measured per form on GB300: 64 words
 // for the int16 strips, 128 for the FP32-unit ones (fewer scans; the int16
 // kernel ran 0.5% slower with 128, FP32 2.9% faster).
-__host__ __device__ constexpr int flush_words(int p) { return p == HARU_INT16 ? 64 : 128; }
+__host__ __device__ constexpr int flush_words(int p) { return p == HARU_INT16 || p == kPrecI16Large ? 64 : 128; }
 __host__ __device__ constexpr int ring_words(int p) { return (prec_span(p) ? 4 : 2) * flush_words(p); }
 // Words of one saved strip state: costs, and start columns for the span forms.
 __host__ __device__ constexpr int state_words(int p) { return prec_span(p) ? 2 * kStateStride : kStateStride; }
@@ -123,9 +137,10 @@ inline cudaError_t opt_in_smem(K kernel, SmemOptIn &rec, size_t bytes) {
 
 // Layout of the small integer block every batch uses: the status word, the
 // planner's group and item counts, the fix-up count, the sweep kernel's work
-// queue counter and the most segments any item was cut into.
+// queue counter, the most segments any item was cut into and the queue
+// counter of the large-code int16 sweep.
 constexpr int kIntStatus = 0, kIntGroups = 1, kIntItems = 2, kIntFixups = 3, kIntQueue = 4, kIntMaxSeg = 5,
-              kIntWords = 6;
+              kIntQueueLarge = 6, kIntWords = 7;
 
 __host__ __device__ inline int steps_per_chunk(int S) { return (S % 2 == 0) ? S : 2 * S; }
 
@@ -165,8 +180,11 @@ __host__ __device__ inline void seg_bounds(int S, int nseg, int seg, long N, lon
 }
 
 struct SdtwArgs {
-  const void *ref_img;     // INT16: uint32 (r | r << 16); FP32: float. Column 0 of N + kRefPad words,
-                           // kRefFront zero words before it
+  const void *ref_img;     // INT16: uint32 (h | h << 16), h the half code; integer forms in FP32: (r | r << 16);
+                           // FP32: float. Column 0 of N + kRefPad words, kRefFront zero words before it
+  const void *ref_large;   // INT16: uint32 (r | r << 16), for the large-code groups
+  int half_max;            // INT16: largest query |code| the half-code cell takes (kHalfSpan - the reference's)
+  int large_possible;      // INT16: a group may hold larger codes (its sweep is launched too)
   long N;                  // reference length (columns)
   const uint32_t *img;     // item images, kImgStride words each
   const Item *items;
@@ -204,7 +222,7 @@ struct PlanArgs {
 struct PackArgs {
   const float *events;
   const uint32_t *offsets;
-  const Item *items;
+  Item *items;              // read; INT16: qmax is written
   const int *n_items;
   uint32_t *img;
   int raw;                  // z-score each query first
@@ -238,7 +256,7 @@ cudaError_t launch_ref_levels(const uint8_t *bases, size_t n, const float *model
 cudaError_t launch_zscore_stats(const float *x, size_t n, double *partials, double *stats, int *status,
                                 cudaStream_t s);
 cudaError_t launch_ref_finish(const float *x, size_t n, const double *stats, int normalize, int scale_log2,
-                              float *z, uint32_t *img16, float *img32, size_t img_len, int *status,
+                              float *z, uint32_t *img16, uint32_t *imgh, float *img32, int *status, int *max_code,
                               cudaStream_t s);
 
 // Set *status to code if it is still 0 (device side).

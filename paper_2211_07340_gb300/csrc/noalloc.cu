@@ -64,8 +64,7 @@ cudaError_t scratch_on(int device, unsigned char **out) {
 }  // namespace
 
 // Reference access and sticky CUDA errors for the no-allocation path (defined in api.cu).
-int ctx_reference(haru_ctx *ctx, int precision, const void **img, long *N, int *scale_log2, int *device,
-                  cudaStream_t *stream, int *warps, int *tile, unsigned long long *wait, int *per_sm, int *sms);
+int ctx_reference(haru_ctx *ctx, RefView *ref, int *device, cudaStream_t *stream, int *warps, int *tile, unsigned long long *wait, int *per_sm, int *sms);
 int ctx_cuda_fail(haru_ctx *ctx, cudaError_t e);
 
 }  // namespace haru
@@ -80,12 +79,11 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   if (flags & ~static_cast<uint32_t>(HARU_RAW)) return HARU_EINVAL;
   if (nq == 0) return HARU_OK;
   if (!events || !offsets || !out_cost || !out_col) return HARU_EINVAL;
-  const void *img = nullptr;
-  long N = 0;
-  int scale = 0, device = 0, warps = 0, tile = 0, per_sm = 0, sms = 0;
+  RefView ref;
+  int device = 0, warps = 0, tile = 0, per_sm = 0, sms = 0;
   unsigned long long wait = 0;
   cudaStream_t own = nullptr;
-  int rc = ctx_reference(ctx, precision, &img, &N, &scale, &device, &own, &warps, &tile, &wait, &per_sm, &sms);
+  int rc = ctx_reference(ctx, &ref, &device, &own, &warps, &tile, &wait, &per_sm, &sms);
   if (rc != HARU_OK) return rc;
   cudaError_t e = cudaSetDevice(device);
   if (e != cudaSuccess) return ctx_cuda_fail(ctx, e);
@@ -107,7 +105,7 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   PlanArgs pa;
   pa.offsets = offsets;
   pa.nq = nq;
-  pa.N = N;
+  pa.N = ref.N;
   pa.pair = precision == HARU_INT16;
   pa.warps = warps;
   pa.units_target = 1;
@@ -129,12 +127,16 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   ka.raw = (flags & HARU_RAW) ? 1 : 0;
   ka.qstats = qstats;
   ka.pair = pa.pair;
-  ka.scale_log2 = scale;
+  ka.scale_log2 = ref.scale_log2;
   ka.status = status + kIntStatus;
   if ((e = launch_pack(ka, static_cast<uint32_t>(max_items), s)) != cudaSuccess) return ctx_cuda_fail(ctx, e);
   SdtwArgs sa;
-  sa.ref_img = img;
-  sa.N = N;
+  const int raw = (flags & HARU_RAW) ? 1 : 0;
+  sa.ref_img = precision == HARU_INT16 ? static_cast<const void *>(ref.imgh) : static_cast<const void *>(ref.img32);
+  sa.ref_large = ref.img16;
+  sa.half_max = kHalfSpan - ref.max_code;
+  sa.large_possible = precision == HARU_INT16 && large_codes_possible(ref, raw);
+  sa.N = ref.N;
   sa.img = imgs;
   sa.items = items;
   sa.groups = groups;
@@ -145,7 +147,7 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   sa.nseg_cap = 1;
   sa.out_cost = out_cost;
   sa.out_col = out_col;
-  sa.inv_scale = 1.0f / static_cast<float>(1 << scale);
+  sa.inv_scale = 1.0f / static_cast<float>(1 << ref.scale_log2);
   sa.tile_cols = tile;
   sa.warps = warps;
   sa.wait_ns = wait;

@@ -87,7 +87,9 @@ __global__ void finish_sums_kernel(const double *partials, size_t nblocks, size_
 }
 
 __global__ void ref_finish_kernel(const float *x, size_t n, const double *stats, int normalize, float s,
-                                  float *z, uint32_t *img16, float *img32, int *status) {
+                                  float *z, uint32_t *img16, uint32_t *imgh, float *img32, int *status,
+                                  int *max_code) {
+  int most = 0;
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
     float v = x[i];
@@ -99,8 +101,12 @@ __global__ void ref_finish_kernel(const float *x, size_t n, const double *stats,
     const int q = quantise(v, s);
     z[i] = v;
     img16[i] = (static_cast<uint32_t>(q) & 0xffffu) | (static_cast<uint32_t>(q) << 16);
+    imgh[i] = half_code(q) * 0x10001u;
     img32[i] = v;
+    most = max(most, abs(q));
   }
+  most = __reduce_max_sync(0xffffffffu, most);
+  if ((threadIdx.x & 31) == 0) atomicMax(max_code, most);
 }
 
 // --------------------------------------------------------------- planner --
@@ -234,7 +240,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
   for (int i = tid; i < n_items; i += blockDim.x) {
     Item it;
     it.qa = -1; it.qb = -1; it.S = 0; it.nseg = 1;
-    it.kind = a.pair == 0 ? kItemF32 : (a.pair == 3 ? kItemExact : kItemPair);
+    it.qmax = 0;
     it.qc = -1; it.qd = -1; it.stacked = 0;
     a.items[i] = it;
   }
@@ -264,7 +270,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
       } else {
         Item it;
         it.qa = static_cast<int>(q); it.qb = -1; it.S = b; it.nseg = nseg_of[b];
-        it.kind = a.pair == 3 ? kItemExact : kItemF32;
+        it.qmax = 0;
         it.qc = -1; it.qd = -1; it.stacked = 0;
         a.items[ibase[b] + pos] = it;
       }
@@ -343,8 +349,9 @@ __global__ void pack_kernel(PackArgs a) {
   int m[2] = {0, 0};
   uint32_t base[2] = {0, 0};
   double mean[2] = {0.0, 0.0}, sigma[2] = {1.0, 1.0};
-  const bool packed = it.kind == kItemPair;   // two int16 queries per word
-  const bool codes = it.kind != kItemF32;     // int16 codes (packed, or as floats)
+  const bool packed = a.pair == 1;  // two int16 queries per word
+  const bool codes = a.pair != 0;   // int16 codes (packed, or as floats)
+  int most = 0;
   const int halves = packed ? 2 : 1;
   for (int h = 0; h < halves; ++h) {
     if (qs[h] >= 0) {
@@ -378,11 +385,10 @@ __global__ void pack_kernel(PackArgs a) {
         if (!isfinite(z) || fabsf(z) > 1.0e20f) report(a.status, HARU_EINVAL);
       }
       if (packed) {
-        // real row: (q, -q); pad row: (-4095, -4095), read by the sweep as distance 0
-        const int qv = real ? quantise(z, s) : -4095;
-        const int nv = real ? -qv : -4095;
-        w0 |= (static_cast<uint32_t>(qv) & 0xffffu) << (16 * h);
-        w1 |= (static_cast<uint32_t>(nv) & 0xffffu) << (16 * h);
+        const int qv = real ? quantise(z, s) : kPadCode;
+        if (real) most = max(most, abs(qv));
+        w0 |= (real ? half_code(qv) : kPadHalf) << (16 * h);
+        w1 |= (static_cast<uint32_t>(qv) & 0xffffu) << (16 * h);
       } else {
         // FP32: the z-value; exact form: the int16 code as a float; the row
         // weight the sweep multiplies the reference sample by: -1 on real
@@ -394,6 +400,10 @@ __global__ void pack_kernel(PackArgs a) {
     }
     img[k * 32 + lane] = w0;
     img[(S + k) * 32 + lane] = w1;
+  }
+  if (packed) {  // warp-uniform
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) a.items[item].qmax = most;
   }
 }
 
@@ -450,15 +460,14 @@ cudaError_t launch_zscore_stats(const float *x, size_t n, double *partials, doub
 }
 
 cudaError_t launch_ref_finish(const float *x, size_t n, const double *stats, int normalize, int scale_log2,
-                              float *z, uint32_t *img16, float *img32, size_t img_len, int *status,
+                              float *z, uint32_t *img16, uint32_t *imgh, float *img32, int *status, int *max_code,
                               cudaStream_t s) {
-  (void)img_len;
   const int th = 256;
   size_t blocks = (n + th - 1) / th;
   if (blocks > 65535) blocks = 65535;
   ref_finish_kernel<<<static_cast<unsigned>(blocks), th, 0, s>>>(x, n, stats, normalize,
                                                                  static_cast<float>(1 << scale_log2), z, img16,
-                                                                 img32, status);
+                                                                 imgh, img32, status, max_code);
   return cudaGetLastError();
 }
 

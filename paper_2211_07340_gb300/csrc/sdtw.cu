@@ -23,6 +23,7 @@ HARU_SDTW_DECLARE(1)
 HARU_SDTW_DECLARE(2)
 HARU_SDTW_DECLARE(3)
 HARU_SDTW_DECLARE(4)
+HARU_SDTW_DECLARE(5)
 
 size_t sdtw_smem_bytes(int precision, int tile_cols, int warps) {
   // Shared header, per-warp tracking rings, two tile slots (each with the
@@ -70,7 +71,9 @@ cudaError_t load_sdtw(int precision) {
   if ((e = sdtw_sweep_load_##P()) != cudaSuccess) return e;      \
   return sdtw_fixup_load_##P();
   switch (precision) {
-    case HARU_INT16: HARU_SDTW_LOAD(1)
+    case HARU_INT16:
+      if ((e = sdtw_sweep_load_5()) != cudaSuccess) return e;
+      HARU_SDTW_LOAD(1)
     case HARU_INT16_ACC32: HARU_SDTW_LOAD(2)
     case kPrecF32Span: HARU_SDTW_LOAD(3)
     case kPrecWideSpan: HARU_SDTW_LOAD(4)
@@ -90,7 +93,9 @@ cudaError_t launch_sdtw(int precision, const SdtwArgs &a, int grid, int fix_item
   if (ev_fix && (e = record_event(ev_fix, s)) != cudaSuccess) return e;         \
   return sdtw_fixup_##P(a, fix_items, s);
   switch (precision) {
-    case HARU_INT16: HARU_SDTW_BOTH(1)
+    case HARU_INT16:
+      if (a.large_possible && (e = sdtw_sweep_5(a, grid, s)) != cudaSuccess) return e;
+      HARU_SDTW_BOTH(1)
     case HARU_INT16_ACC32: HARU_SDTW_BOTH(2)
     case kPrecF32Span: HARU_SDTW_BOTH(3)
     case kPrecWideSpan: HARU_SDTW_BOTH(4)

@@ -177,38 +177,40 @@ struct Geo {
 };
 
 // ---------------------------------------------------------------- INT16 --
-// Pad rows carry the code -4095 in both Q and NQ: |q - r| is then taken as
-// relu(max(r + NQ, Q - r)) = relu(negative) = 0, so a pad row stays 0 (the
-// free-start row) without a per-row cap, and real rows (|q|, |r| <= 2047)
-// get max(r - q, q - r) unchanged.
-constexpr uint32_t kPadQ2 = 0xf001f001u;  // -4095 in both halves
 constexpr uint32_t kCap2 = (static_cast<uint32_t>(kCap) << 16) | static_cast<uint32_t>(kCap);
 
 // Sparse saturation. Costs are held as unsigned 16-bit halves and only rows
-// k = S-1, S-1-kCapRun, ... of each lane take min(CAP, .); the rows between
+// k = S-1, S-1-RUN, ... of each lane take min(CAP, .); the rows between
 // add without a cap: a plain 32-bit add of the two packed words, which is the
 // per-half add exactly because no half's sum reaches 2^16 (see below), and
-// keeps those rows off the DPX min/max pipe. Every cell lies between min(CAP, exact)
-// and the exact cost, and a min3 is at most its `up` input, so the j-th
-// uncapped row after a capped one holds at most CAP + j * 4094. Runs are at
-// most kCapRun - 1 = 8 rows (also across lanes: row S-1 is capped), so every
-// value and every sum before a cap stays below 2^16 (28673 + 9 * 4094 =
-// 65519), and each capped row -- the query's last row among them -- equals
-// min(CAP, exact), the value of the all-saturating recurrence.
-constexpr int kCapRun = 9;
+// keeps those rows off the half-rate pipe. Every cell lies between min(CAP,
+// exact) and the exact cost, and a min3 is at most its `up` input, so the
+// j-th uncapped row after a capped one holds at most CAP + j * D for
+// distances of at most D. Row S-1 is capped, so runs never cross lanes:
+// every value and every sum before a cap stays below 2^16, and each capped
+// row -- the query's last row among them -- equals min(CAP, exact), the
+// value of the all-saturating recurrence.
+//   half codes:  D = kHalfSpan, RUN = 16: only row S-1 is capped
+//                (28673 + 16 * 2047 = 61425);
+//   large codes: D = 4094, RUN = 9 (28673 + 9 * 4094 = 65519).
+constexpr int kCapRunHalf = kMaxS, kCapRunLarge = 9;
+static_assert(kCap + kCapRunHalf * kHalfSpan < 65536 && kCap + kCapRunLarge * 2 * kQmax < 65536, "no carry");
 
+// q - r per half, on half codes (exact: see kHalfSpan).
+__device__ __forceinline__ uint32_t half_diff(uint32_t q, uint32_t r) {
+  uint32_t d;
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(q), "r"(r));
+  return d;
+}
+
+// State shared by the int16 strips: the last two oblique columns, the
+// reference samples moving down the lane's rows, and the two oblique columns
+// of the row above the lane.
 template <int S>
-struct StripI16 {
-  uint32_t Q[S], NQ[S], G[2][S], Rr[S];
+struct StateI16 {
+  uint32_t G[2][S], Rr[S];
   uint32_t gprev;
 
-  __device__ __forceinline__ void load(const uint32_t *img, int lane) {
-#pragma unroll
-    for (int k = 0; k < S; ++k) {
-      Q[k] = img[k * 32 + lane];
-      NQ[k] = img[(S + k) * 32 + lane];
-    }
-  }
   // As if the reference began at the current step: every row, pad rows
   // included, holds CAP (infinity), and the row above a stack's top row held
   // the free-start 0 one step back (gprev). The top row then turns 0 at
@@ -246,8 +248,15 @@ struct StripI16 {
     }
   }
 
-  __device__ __forceinline__ void chunk(const uint32_t *ref, int lane, uint32_t *ring, int e0, uint32_t ng,
-                                        bool tracked, int, int) {
+  // One chunk of U steps; dist(k, r) is row k's distance to the sample r.
+  // A step's distances, minima and sums are three passes over the rows, and
+  // neighbouring rows name the value they share (G[a][k - 1]: `up` of row k,
+  // `left` of row k - 1) in the same operand place: the cell is bound by
+  // register operand reads (about 1.7 a clock and scheduler over all mixes
+  // measured), and this order lets a minimum reuse one of its operands.
+  template <int RUN, class Dist>
+  __device__ __forceinline__ void steps(const uint32_t *ref, uint32_t *ring, int e0, uint32_t ng, bool tracked,
+                                        const Dist &dist) {
     constexpr int U = Geo<S>::U;
     LaneWindow<S> win;
 #pragma unroll
@@ -263,22 +272,66 @@ struct StripI16 {
       // put the zero in.
       if constexpr (S == kMaxS) gup = imad(gup, ng, 0u);
       Rr[p] = win.get(ref, u);  // row 0's reference: column t - lane * S
+      uint32_t d[S], m[S];
+#pragma unroll
+      for (int k = S - 1; k >= 0; --k) d[k] = dist(k, Rr[(p + k) % S]);
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) {
-        const uint32_t r = Rr[(p + k) % S];
-        const uint32_t d = __viaddmax_s16x2_relu(r, NQ[k], __vsub2(Q[k], r));  // |q - r| per half
         const uint32_t up = k ? G[a][k - 1] : gup;
         const uint32_t dg = k ? G[b][k - 1] : gprev;
-        const uint32_t m = __vimin3_u16x2(up, dg, G[a][k]);
-        // rows between caps: one 32-bit add, exact per half (no carry leaves a half: every sum is below 2^16)
-        G[b][k] = (S - 1 - k) % kCapRun == 0 ? __viaddmin_u16x2(d, m, kCap2) : m + d;
+        m[k] = (k & 1) ? __vimin3_u16x2(up, dg, G[a][k]) : __vimin3_u16x2(G[a][k], dg, up);
       }
+#pragma unroll
+      for (int k = S - 1; k >= 0; --k)
+        G[b][k] = (S - 1 - k) % RUN == 0 ? __viaddmin_u16x2(d[k], m[k], kCap2) : m[k] + d[k];
       gprev = gup;
       // The last row's values of steps u - 1 and u sit in G[0] and G[1]: one
       // 8-byte store every two steps (U is even, the ring 16-byte aligned).
       if ((u & 1) && tracked)
         *reinterpret_cast<uint2 *>(ring + e0 + u - 1) = make_uint2(G[0][S - 1], G[1][S - 1]);
     }
+  }
+};
+
+// The int16 strip on half codes: the distance is one fp16x2 subtraction and
+// a mask, 8 register operands a cell pair with the minimum and the sum,
+// where the integer form below reads 10 and holds a second query array.
+template <int S>
+struct StripI16 : StateI16<S> {
+  uint32_t Q[S];
+  __device__ __forceinline__ void load(const uint32_t *img, int lane) {
+#pragma unroll
+    for (int k = 0; k < S; ++k) Q[k] = img[k * 32 + lane];
+  }
+  __device__ __forceinline__ void chunk(const uint32_t *ref, int, uint32_t *ring, int e0, uint32_t ng, bool tracked,
+                                        int, int) {
+    this->template steps<kCapRunHalf>(ref, ring, e0, ng, tracked, [this](int k, uint32_t r) {
+      return half_diff(Q[k], r) & 0x07ff07ffu;  // the low 11 bits: |q - r|; pad rows (2^15 - r = 2^15): 0
+    });
+  }
+};
+
+// The int16 strip on two's complement codes of any size (|q|, |r| <= 2047).
+// Pad rows carry the code -4095 in both Q and NQ: |q - r| is taken as
+// relu(max(r + NQ, Q - r)) = relu(negative) = 0, so a pad row stays 0 (the
+// free-start row), and real rows get max(r - q, q - r).
+template <int S>
+struct StripI16Large : StateI16<S> {
+  uint32_t Q[S], NQ[S];
+  __device__ __forceinline__ void load(const uint32_t *img, int lane) {
+    constexpr uint32_t kPad2 = (static_cast<uint32_t>(kPadCode) & 0xffffu) * 0x10001u;
+#pragma unroll
+    for (int k = 0; k < S; ++k) {
+      Q[k] = img[(S + k) * 32 + lane];
+      const uint32_t pad = __vcmpeq2(Q[k], kPad2);
+      NQ[k] = (__vneg2(Q[k]) & ~pad) | (kPad2 & pad);
+    }
+  }
+  __device__ __forceinline__ void chunk(const uint32_t *ref, int, uint32_t *ring, int e0, uint32_t ng, bool tracked,
+                                        int, int) {
+    this->template steps<kCapRunLarge>(ref, ring, e0, ng, tracked, [this](int k, uint32_t r) {
+      return __viaddmax_s16x2_relu(r, NQ[k], __vsub2(Q[k], r));  // |q - r| per half
+    });
   }
 };
 
@@ -387,7 +440,8 @@ struct StripF32 {
         const float d = __fmaf_rn(r, W[k], Q[k]);
         const float up = k ? G[a][k - 1] : gup;
         const float dg = k ? G[b][k - 1] : gprev;
-        const float m = fmin3f(up, dg, G[a][k]);
+        // the value shared with the row above in the same operand place, as in the int16 strips
+        const float m = (k & 1) ? fmin3f(up, dg, G[a][k]) : fmin3f(G[a][k], dg, up);
         G[b][k] = __fadd_rn(fabsf(d), m);
       }
       gprev = gup;
@@ -563,7 +617,8 @@ struct TrackF32Span {
 // codes computed exactly without saturation: wide accumulation (every cost
 // of a query of <= 512 events is an integer below 512 * 4094 < 2^24, so FP32
 // holds it exactly).
-constexpr int kFormF32 = 0, kFormI16 = 1, kFormExactWide = 3;
+constexpr int kFormF32 = 0, kFormI16 = 1, kFormI16Large = 2, kFormExactWide = 3;
+constexpr bool form_i16(int form) { return form == kFormI16 || form == kFormI16Large; }
 // and the FP32 and wide forms carrying the start column
 constexpr int kFormF32Span = 4, kFormWideSpan = 5;
 // Rows of 32 words in a saved strip state, per strip row: two oblique
@@ -576,6 +631,11 @@ struct FormOf;
 template <int S>
 struct FormOf<kFormI16, S> {
   using Strip = StripI16<S>;
+  using Track = TrackI16;
+};
+template <int S>
+struct FormOf<kFormI16Large, S> {
+  using Strip = StripI16Large<S>;
   using Track = TrackI16;
 };
 template <int S>
@@ -694,7 +754,7 @@ __device__ bool run_steps(typename FormOf<FORM, S>::Strip &st, typename FormOf<F
                           int TS, long t_start, long t_own, long t_end, bool fresh, long N, uint32_t *save_start,
                           uint32_t *save_final, uint32_t *ring, int lane, bool stk) {
   constexpr int U = Geo<S>::U;
-  constexpr int W = flush_words(FORM == kFormI16 ? HARU_INT16 : HARU_FP32);
+  constexpr int W = flush_words(form_i16(FORM) ? HARU_INT16 : HARU_FP32);
   // chunks between two flushes: a stack's entries fill its share of a buffer
   constexpr int kWhole = W / U > 0 ? W / U : 1;
   constexpr int kHalf = W / 2 / U > 0 ? W / 2 / U : 1;
@@ -786,6 +846,8 @@ __device__ __forceinline__ void sweep_any(const SdtwArgs &A, TileStream &ts, con
     sweep_unit<kFormF32Span, S>(A, ts, g, item, ring, lane);
   } else if constexpr (PREC == kPrecWideSpan) {
     sweep_unit<kFormWideSpan, S>(A, ts, g, item, ring, lane);
+  } else if constexpr (PREC == kPrecI16Large) {
+    sweep_unit<kFormI16Large, S>(A, ts, g, item, ring, lane);
   } else {
     sweep_unit<kFormI16, S>(A, ts, g, item, ring, lane);
   }
@@ -826,13 +888,26 @@ __global__ void __launch_bounds__(prec_span(PREC) ? 256 : 384, 1) sdtw_kernel(Sd
   }
   __syncthreads();
   const int count = A.ints[kIntGroups];
-  int *queue = A.ints + kIntQueue;
+  int *queue = A.ints + (PREC == kPrecI16Large ? kIntQueueLarge : kIntQueue);
   for (;;) {
     if (threadIdx.x == 0) sh->group = atomicAdd(queue, 1);
     __syncthreads();
     const int gi = sh->group;
     if (gi >= count || sh->abort) break;
     const Group grp = A.groups[gi];
+    if constexpr (PREC == HARU_INT16 || PREC == kPrecI16Large) {
+      // A group with a code too large for the half-code cell belongs to the
+      // large-code sweep, every other one to this form's.
+      bool large = false;
+      if (A.large_possible) {
+        const int it = lane < grp.count ? lane : 0;
+        large = __any_sync(kFull, A.items[grp.first + it].qmax > A.half_max);
+      }
+      if (large != (PREC == kPrecI16Large)) {
+        __syncthreads();  // every thread has read sh->group
+        continue;
+      }
+    }
     const int S = grp.S;
     const int TS = tile_width(S, A.tile_cols);
     long t_start, t_own, t_end;
@@ -840,7 +915,7 @@ __global__ void __launch_bounds__(prec_span(PREC) ? 256 : 384, 1) sdtw_kernel(Sd
     TileStream ts;
     ts.sh = sh;
     ts.slots = slots;
-    ts.src = reinterpret_cast<const char *>(A.ref_img);
+    ts.src = reinterpret_cast<const char *>(PREC == kPrecI16Large ? A.ref_large : A.ref_img);
     ts.tile_cols = TS;
     ts.k_first = static_cast<int>(t_start / TS);
     ts.K = static_cast<int>((t_end + TS - 1) / TS - t_start / TS);
@@ -874,7 +949,7 @@ __global__ void __launch_bounds__(prec_span(PREC) ? 256 : 384, 1) sdtw_kernel(Sd
 // tie the earlier segment's (smaller) column stays.
 template <int FORM>
 __device__ __forceinline__ void combine(Best &b, const Best &o) {
-  if (FORM == kFormI16) {
+  if (form_i16(FORM)) {
     if (o.ia < b.ia) { b.ia = o.ia; b.ca = o.ca; }
     if (o.ib < b.ib) { b.ib = o.ib; b.cb = o.cb; }
   } else {
@@ -885,7 +960,7 @@ __device__ __forceinline__ void combine(Best &b, const Best &o) {
 template <int FORM>
 __device__ __forceinline__ void write_out(const SdtwArgs &A, const Best &b, int qa, int qb) {
   if (qa < 0) return;
-  if (FORM == kFormI16) {
+  if (form_i16(FORM)) {
     A.out_cost[qa] = static_cast<float>(b.ia) * A.inv_scale;
     A.out_col[qa] = b.ca;
     if (qb >= 0) {
@@ -907,6 +982,7 @@ __device__ void fixup_item(const SdtwArgs &A, int item, uint32_t *ring, int lane
   const Item it = A.items[item];
   const int nseg = it.nseg;
   const bool stk = it.stacked != 0;
+  const uint32_t *ref = static_cast<const uint32_t *>(FORM == kFormI16Large ? A.ref_large : A.ref_img);
   const size_t base = static_cast<size_t>(item) * A.nseg_cap;
   Best b = A.bests[base];
   Best b2 = stk ? A.bests2[base] : b;
@@ -926,14 +1002,14 @@ __device__ void fixup_item(const SdtwArgs &A, int item, uint32_t *ring, int lane
       bool eq = true;
       for (int k = 0; k < kRows * S; ++k) {
         const uint32_t x = exact[k * 32 + lane], y = spec[k * 32 + lane];
-        eq = eq && (FORM == kFormI16 ? __vminu2(x, kCap2) == __vminu2(y, kCap2) : x == y);
+        eq = eq && (form_i16(FORM) ? __vminu2(x, kCap2) == __vminu2(y, kCap2) : x == y);
       }
       if (!__all_sync(kFull, eq)) {
         long t_start, t_own, t_end;
         seg_bounds(S, nseg, s, A.N, &t_start, &t_own, &t_end);
-        st.restore(exact, reinterpret_cast<const uint32_t *>(A.ref_img), t_own, lane, ng);
+        st.restore(exact, ref, t_own, lane, ng);
         typename FormOf<FORM, S>::Track tr;
-        GlobalTiles src{reinterpret_cast<const uint32_t *>(A.ref_img), TS, t_own / TS};
+        GlobalTiles src{ref, TS, t_own / TS};
         uint32_t *sf = s + 1 < nseg ? A.states + ((base + s) * 2 + 1) * kWords : nullptr;
         run_steps<FORM, S>(st, tr, src, TS, t_own, t_own, t_end, false, A.N, nullptr, sf, ring, lane, stk);
         tr.reduce(stk ? 16 : 32);
@@ -964,6 +1040,8 @@ __device__ __forceinline__ void fixup_any(const SdtwArgs &A, int item, uint32_t 
     fixup_item<kFormF32Span, S>(A, item, ring, lane);
   } else if constexpr (PREC == kPrecWideSpan) {
     fixup_item<kFormWideSpan, S>(A, item, ring, lane);
+  } else if (A.items[item].qmax > A.half_max) {
+    fixup_item<kFormI16Large, S>(A, item, ring, lane);
   } else {
     fixup_item<kFormI16, S>(A, item, ring, lane);
   }
