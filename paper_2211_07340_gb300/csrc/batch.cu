@@ -18,7 +18,7 @@ cudaError_t record_event(cudaEvent_t e, cudaStream_t s) {
 }
 
 void ws_free(Workspace &ws) {
-  void *p[] = {ws.ints, ws.items, ws.groups, ws.img, ws.states, ws.bests, ws.qstats};
+  void *p[] = {ws.ints, ws.items, ws.arrived, ws.groups, ws.img, ws.states, ws.bests, ws.qstats};
   for (void *q : p)
     if (q) cudaFree(q);
   ws = Workspace();
@@ -59,14 +59,17 @@ cudaError_t ws_alloc(Workspace &ws, size_t max_items, size_t units, size_t qstat
   if ((e = grow(&ws.ints, &c, kIntWords)) != cudaSuccess) return e;
   if (ws.cap_items < max_items) {
     cudaFree(ws.items);
+    cudaFree(ws.arrived);
     cudaFree(ws.groups);
     cudaFree(ws.img);
     ws.items = nullptr;
+    ws.arrived = nullptr;
     ws.groups = nullptr;
     ws.img = nullptr;
     ws.cap_items = 0;
-    size_t c0 = 0, c1 = 0, c2 = 0;
+    size_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;
     if ((e = grow(&ws.items, &c0, max_items)) != cudaSuccess) return e;
+    if ((e = grow(&ws.arrived, &c3, max_items)) != cudaSuccess) return e;
     if ((e = grow(&ws.groups, &c1, (max_items + kMaxS) * kMaxSeg)) != cudaSuccess) return e;
     if ((e = grow(&ws.img, &c2, max_items * kImgStride)) != cudaSuccess) return e;
     ws.cap_items = max_items;
@@ -127,6 +130,7 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
   pa.stack = lc.stack_short > 0 || (lc.stack_short == 0 && fills) ? 1 : 0;
   pa.nseg_cap = ws.nseg_cap;
   pa.items = ws.items;
+  pa.arrived = ws.arrived;
   pa.groups = ws.groups;
   pa.ints = ws.ints;
   if ((e = launch_plan(pa, s)) != cudaSuccess) return e;
@@ -161,6 +165,7 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
   sa.states = ws.states;
   sa.bests = ws.bests;
   sa.bests2 = ws.bests + ws.max_items * static_cast<size_t>(ws.nseg_cap);
+  sa.arrived = ws.arrived;
   sa.out_start = d_start;
   sa.nseg_cap = ws.nseg_cap;
   sa.out_cost = d_cost;

@@ -88,6 +88,7 @@ inline int large_codes_possible(const RefView &r, int raw) {
 struct Workspace {
   int *ints = nullptr;
   Item *items = nullptr;
+  int *arrived = nullptr;  // per item
   Group *groups = nullptr;
   uint32_t *img = nullptr;
   size_t cap_items = 0;

@@ -193,6 +193,7 @@ struct SdtwArgs {
   uint32_t *states;        // [item][nseg_cap][2] saved states (start, final), kStateStride words each
   Best *bests;             // [item][nseg_cap]: the strip's (upper stack's) last-row minimum
   Best *bests2;            // [item][nseg_cap]: the lower stack's, for stacked items
+  int *arrived;            // [item]: CTAs of the fix-up kernel that verified their segments (zeroed by the planner)
   int64_t *out_start;      // span forms: the alignment start column per query
   int nseg_cap;
   float *out_cost;
@@ -215,6 +216,7 @@ struct PlanArgs {
   int stack;                // 1: stack queries of <= kStackMax events two to a strip
   int nseg_cap;             // most segments per item (state storage is sized for it)
   Item *items;
+  int *arrived;             // zeroed, one word per item (nullptr: not used)
   Group *groups;
   int *ints;                // kIntWords counters (status, counts, queues, class ranges)
 };

@@ -112,6 +112,7 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   pa.stack = 0;  // at most HARU_NOALLOC_MAX_QUERIES queries: latency over throughput
   pa.nseg_cap = 1;
   pa.items = items;
+  pa.arrived = nullptr;  // one segment per item
   pa.groups = groups;
   pa.ints = status;
   if ((e = launch_plan(pa, s)) != cudaSuccess) return ctx_cuda_fail(ctx, e);
@@ -144,6 +145,7 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   sa.states = nullptr;
   sa.bests = bests;
   sa.bests2 = bests + kNaItems;
+  sa.arrived = nullptr;
   sa.nseg_cap = 1;
   sa.out_cost = out_cost;
   sa.out_col = out_col;

@@ -243,6 +243,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
     it.qmax = 0;
     it.qc = -1; it.qd = -1; it.stacked = 0;
     a.items[i] = it;
+    if (a.arrived) a.arrived[i] = 0;
   }
   __syncthreads();
   const unsigned lt = (1u << lane) - 1u;

@@ -941,22 +941,15 @@ __global__ void __launch_bounds__(prec_span(PREC) ? 256 : 384, 1) sdtw_kernel(Sd
 }
 
 // --------------------------------------------------------------- fix-up --
-// One warp per item: verify every segment boundary, recompute segments whose
-// speculative start state differs from the exact one, combine the segments'
-// last-row minima (smallest cost, then smallest column) and write the
-// outputs.
-// Segment minima combine in segment order: the smaller cost wins, and on a
-// tie the earlier segment's (smaller) column stays.
-template <int FORM>
-__device__ __forceinline__ void combine(Best &b, const Best &o) {
-  if (form_i16(FORM)) {
-    if (o.ia < b.ia) { b.ia = o.ia; b.ca = o.ca; }
-    if (o.ib < b.ib) { b.ib = o.ib; b.cb = o.cb; }
-  } else {
-    if (o.f < b.f) { b.f = o.f; b.ca = o.ca; b.cb = o.cb; }  // cb: the start column of the span forms
-  }
-}
-
+// Verifies every segment boundary, recomputes segments whose speculative
+// start state differs from the exact one, combines the segments' last-row
+// minima (smallest cost, then smallest column) and writes the outputs.
+//
+// One CTA per item and kFixWarps segments: each warp compares one boundary
+// (latency bound: 4S independent 128-byte loads), the item's last CTA to
+// finish reads the verdicts, and its first warp does the rest. One warp per
+// item that walked the boundaries in turn took 89 us where this takes 9 (51
+// int16 items of up to 29 segments) and 734 us where this takes 36 (128 items of 57).
 template <int FORM>
 __device__ __forceinline__ void write_out(const SdtwArgs &A, const Best &b, int qa, int qb) {
   if (qa < 0) return;
@@ -977,96 +970,189 @@ __device__ __forceinline__ void write_out(const SdtwArgs &A, const Best &b, int 
   if (FORM == kFormF32Span || FORM == kFormWideSpan) A.out_start[qa] = b.cb;
 }
 
+// Whether segment s of an item started from the state the segment before it
+// ended in (whole warp): costs, and start columns in the span forms; int16
+// equal modulo min(CAP, .), which fixes every later capped value.
+template <int FORM>
+__device__ __forceinline__ bool boundary_exact(const SdtwArgs &A, size_t base, int s, int S, int lane) {
+  constexpr int kRows = state_rows_per_s<FORM>();
+  constexpr size_t kWords = kRows * 16 * 32;
+  const uint32_t *exact = A.states + ((base + s - 1) * 2 + 1) * kWords + lane;
+  const uint32_t *spec = A.states + ((base + s) * 2 + 0) * kWords + lane;
+  unsigned diff = 0;
+#pragma unroll 8
+  for (int k = 0; k < kRows * S; ++k) {
+    const uint32_t x = exact[k * 32], y = spec[k * 32];
+    diff |= form_i16(FORM) ? __vminu2(x, kCap2) ^ __vminu2(y, kCap2) : x ^ y;
+  }
+  return __all_sync(kFull, diff == 0);
+}
+
+// Recompute, in order, every segment whose start state is not the exact one
+// (one warp): those marked, and those after a recomputed segment that the
+// new final state does not reach either.
 template <int FORM, int S>
-__device__ void fixup_item(const SdtwArgs &A, int item, uint32_t *ring, int lane) {
+__device__ void recompute_segments(const SdtwArgs &A, int item, uint32_t *ring, int lane) {
   const Item it = A.items[item];
   const int nseg = it.nseg;
   const bool stk = it.stacked != 0;
   const uint32_t *ref = static_cast<const uint32_t *>(FORM == kFormI16Large ? A.ref_large : A.ref_img);
   const size_t base = static_cast<size_t>(item) * A.nseg_cap;
-  Best b = A.bests[base];
-  Best b2 = stk ? A.bests2[base] : b;
-  if (nseg > 1) {
-    typename FormOf<FORM, S>::Strip st;
-    st.load(A.img + static_cast<size_t>(item) * kImgStride, lane);
-    const int TS = tile_width(S, A.tile_cols);
-    const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
-    constexpr int kRows = state_rows_per_s<FORM>();
-    constexpr size_t kWords = kRows * 16 * 32;
-    for (int s = 1; s < nseg; ++s) {
-      // The segment is exact iff its speculative start state (costs, and
-      // start columns in the span forms) equals the previous segment's final one.
-      const uint32_t *exact = A.states + ((base + s - 1) * 2 + 1) * kWords;
-      const uint32_t *spec = A.states + ((base + s) * 2 + 0) * kWords;
-      // (int16: equal modulo min(CAP, .), which fixes every later capped value)
-      bool eq = true;
-      for (int k = 0; k < kRows * S; ++k) {
-        const uint32_t x = exact[k * 32 + lane], y = spec[k * 32 + lane];
-        eq = eq && (form_i16(FORM) ? __vminu2(x, kCap2) == __vminu2(y, kCap2) : x == y);
-      }
-      if (!__all_sync(kFull, eq)) {
-        long t_start, t_own, t_end;
-        seg_bounds(S, nseg, s, A.N, &t_start, &t_own, &t_end);
-        st.restore(exact, ref, t_own, lane, ng);
-        typename FormOf<FORM, S>::Track tr;
-        GlobalTiles src{ref, TS, t_own / TS};
-        uint32_t *sf = s + 1 < nseg ? A.states + ((base + s) * 2 + 1) * kWords : nullptr;
-        run_steps<FORM, S>(st, tr, src, TS, t_own, t_own, t_end, false, A.N, nullptr, sf, ring, lane, stk);
-        tr.reduce(stk ? 16 : 32);
-        if (lane == 0) {
-          tr.store(A.bests + base + s);
-          atomicAdd(A.ints + kIntFixups, 1);
-        }
-        if (stk && lane == 16) tr.store(A.bests2 + base + s);
-        __syncwarp();
-      }
-      combine<FORM>(b, A.bests[base + s]);
-      if (stk) combine<FORM>(b2, A.bests2[base + s]);
+  const int TS = tile_width(S, A.tile_cols);
+  const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
+  constexpr size_t kWords = state_rows_per_s<FORM>() * 16 * 32;
+  typename FormOf<FORM, S>::Strip st;
+  st.load(A.img + static_cast<size_t>(item) * kImgStride, lane);
+  bool moved = false;  // the segment before was recomputed: its final state is new
+  for (int s = 1; s < nseg; ++s) {
+    const bool bad = moved ? !boundary_exact<FORM>(A, base, s, S, lane) : __ldcg(&A.bests[base + s].pad) != 0;
+    moved = bad;
+    if (!bad) continue;
+    long t_start, t_own, t_end;
+    seg_bounds(S, nseg, s, A.N, &t_start, &t_own, &t_end);
+    st.restore(A.states + ((base + s - 1) * 2 + 1) * kWords, ref, t_own, lane, ng);
+    typename FormOf<FORM, S>::Track tr;
+    GlobalTiles src{ref, TS, t_own / TS};
+    uint32_t *sf = s + 1 < nseg ? A.states + ((base + s) * 2 + 1) * kWords : nullptr;
+    run_steps<FORM, S>(st, tr, src, TS, t_own, t_own, t_end, false, A.N, nullptr, sf, ring, lane, stk);
+    tr.reduce(stk ? 16 : 32);
+    if (lane == 0) {
+      tr.store(A.bests + base + s);
+      atomicAdd(A.ints + kIntFixups, 1);
+    }
+    if (stk && lane == 16) tr.store(A.bests2 + base + s);
+    __syncwarp();
+  }
+}
+
+// Segment minima combine by smaller cost, then by smaller segment (its
+// columns are the smaller ones).
+struct Pick {
+  float c = __builtin_huge_valf();
+  int s = 0x7fffffff;
+  int64_t col = -1, start = -1;
+  __device__ __forceinline__ void take(float oc, int os, int64_t ocol, int64_t ostart) {
+    if (oc < c || (oc == c && os < s)) { c = oc; s = os; col = ocol; start = ostart; }
+  }
+  __device__ __forceinline__ void reduce() {
+    for (int o = 16; o > 0; o >>= 1) {
+      const float oc = __shfl_xor_sync(kFull, c, o);
+      const int os = __shfl_xor_sync(kFull, s, o);
+      const int64_t ocol = __shfl_xor_sync(kFull, col, o), ostart = __shfl_xor_sync(kFull, start, o);
+      take(oc, os, ocol, ostart);
     }
   }
-  if (lane == 0) {
-    write_out<FORM>(A, b, it.qa, it.qb);
-    if (stk) write_out<FORM>(A, b2, it.qc, it.qd);
-  }
-}
+};
 
-template <int PREC, int S>
-__device__ __forceinline__ void fixup_any(const SdtwArgs &A, int item, uint32_t *ring, int lane) {
-  if constexpr (PREC == HARU_FP32) {
-    fixup_item<kFormF32, S>(A, item, ring, lane);
-  } else if constexpr (PREC == HARU_INT16_ACC32) {
-    fixup_item<kFormExactWide, S>(A, item, ring, lane);
-  } else if constexpr (PREC == kPrecF32Span) {
-    fixup_item<kFormF32Span, S>(A, item, ring, lane);
-  } else if constexpr (PREC == kPrecWideSpan) {
-    fixup_item<kFormWideSpan, S>(A, item, ring, lane);
-  } else if (A.items[item].qmax > A.half_max) {
-    fixup_item<kFormI16Large, S>(A, item, ring, lane);
+// The item's result over its segments (whole warp; valid on every lane).
+template <int FORM>
+__device__ __forceinline__ Best combine(const Best *bests, int nseg, int lane) {
+  Pick a, b;
+  for (int s = lane; s < nseg; s += 32) {
+    const Best o = bests[s];
+    if (form_i16(FORM)) {  // costs up to CAP: exact as floats
+      a.take(static_cast<float>(o.ia), s, o.ca, -1);
+      b.take(static_cast<float>(o.ib), s, o.cb, -1);
+    } else {
+      a.take(o.f, s, o.ca, o.cb);  // cb: the start column of the span forms
+    }
+  }
+  a.reduce();
+  Best r{};
+  if (form_i16(FORM)) {
+    b.reduce();
+    r.ia = static_cast<int>(a.c);
+    r.ib = static_cast<int>(b.c);
+    r.cb = b.col;
   } else {
-    fixup_item<kFormI16, S>(A, item, ring, lane);
+    r.f = a.c;
+    r.cb = a.start;
   }
+  r.ca = a.col;
+  return r;
 }
 
-template <int PREC, int S = 1>
-__device__ __forceinline__ void dispatch_fixup(int s, const SdtwArgs &A, int item, uint32_t *ring, int lane) {
+template <int FORM, int S = 1>
+__device__ __forceinline__ void dispatch_recompute(int s, const SdtwArgs &A, int item, uint32_t *ring, int lane) {
   if constexpr (S <= kMaxS) {
     if (s == S)
-      fixup_any<PREC, S>(A, item, ring, lane);
+      recompute_segments<FORM, S>(A, item, ring, lane);
     else
-      dispatch_fixup<PREC, S + 1>(s, A, item, ring, lane);
+      dispatch_recompute<FORM, S + 1>(s, A, item, ring, lane);
   }
 }
 
-constexpr int kFixWarps = 4;
+// Batches cut into at most kFixSolo segments (thousands of items) give each
+// warp an item of its own: a CTA per item ran 137 us on 6,571 items, this 20.
+constexpr int kFixWarps = 8, kFixSolo = 8;
+
+// part: which kFixWarps of the item's segments this CTA verifies, one to a
+// warp; -1: this warp alone has the item.
+template <int FORM>
+__device__ void fixup_item(const SdtwArgs &A, int item, int part, uint32_t *ring, int *last) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const Item it = A.items[item];
+  const int nseg = it.nseg;
+  const int parts = part < 0 ? 1 : (nseg + kFixWarps - 1) / kFixWarps;
+  if (part >= parts) return;
+  const size_t base = static_cast<size_t>(item) * A.nseg_cap;
+  const int s_lo = part < 0 ? 1 : part * kFixWarps + warp;
+  const int s_hi = part < 0 ? nseg : (s_lo < nseg ? s_lo + 1 : s_lo);
+  for (int s = s_lo; s < s_hi; ++s) {
+    if (s == 0) continue;
+    const bool exact = boundary_exact<FORM>(A, base, s, it.S, lane);
+    if (lane == 0) A.bests[base + s].pad = exact ? 0 : 1;
+  }
+  if (part >= 0) {
+    __syncthreads();
+    if (parts > 1) {
+      if (threadIdx.x == 0) {
+        __threadfence();
+        *last = atomicAdd(A.arrived + item, 1) == parts - 1;
+        __threadfence();
+      }
+      __syncthreads();
+      if (!*last) return;
+    }
+    if (warp != 0) return;
+  }
+  __syncwarp();
+  if (nseg > 1) {
+    bool bad = false;
+    for (int s = 1 + lane; s < nseg; s += 32) bad = bad || __ldcg(&A.bests[base + s].pad) != 0;
+    if (__any_sync(kFull, bad)) dispatch_recompute<FORM>(it.S, A, item, ring, lane);
+  }
+  const Best b = combine<FORM>(A.bests + base, nseg, lane);
+  if (lane == 0) write_out<FORM>(A, b, it.qa, it.qb);
+  if (it.stacked) {
+    const Best b2 = combine<FORM>(A.bests2 + base, nseg, lane);
+    if (lane == 0) write_out<FORM>(A, b2, it.qc, it.qd);
+  }
+}
 
 template <int PREC>
 __global__ void __launch_bounds__(kFixWarps * 32) fixup_kernel(SdtwArgs A) {
   __shared__ __align__(16) uint32_t rings[kFixWarps * ring_words(PREC)];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int count = A.ints[kIntItems];
-  const int item = blockIdx.x * kFixWarps + warp;
-  if (item >= count) return;
-  dispatch_fixup<PREC>(A.items[item].S, A, item, rings + warp * ring_words(PREC), lane);
+  __shared__ int last;
+  const int warp = threadIdx.x >> 5;
+  const bool split = A.nseg_cap > kFixSolo;
+  const int item = split ? blockIdx.x : blockIdx.x * kFixWarps + warp;
+  const int part = split ? blockIdx.y : -1;
+  uint32_t *ring = rings + warp * ring_words(PREC);
+  if (item >= A.ints[kIntItems]) return;
+  if constexpr (PREC == HARU_FP32) {
+    fixup_item<kFormF32>(A, item, part, ring, &last);
+  } else if constexpr (PREC == HARU_INT16_ACC32) {
+    fixup_item<kFormExactWide>(A, item, part, ring, &last);
+  } else if constexpr (PREC == kPrecF32Span) {
+    fixup_item<kFormF32Span>(A, item, part, ring, &last);
+  } else if constexpr (PREC == kPrecWideSpan) {
+    fixup_item<kFormWideSpan>(A, item, part, ring, &last);
+  } else if (A.items[item].qmax > A.half_max) {
+    fixup_item<kFormI16Large>(A, item, part, ring, &last);
+  } else {
+    fixup_item<kFormI16>(A, item, part, ring, &last);
+  }
 }
 
 template <int PREC>
@@ -1082,7 +1168,10 @@ cudaError_t launch_sweep_prec(const SdtwArgs &a, int grid, cudaStream_t s) {
 template <int PREC>
 cudaError_t launch_fixup_prec(const SdtwArgs &a, int fix_items, cudaStream_t s) {
   if (fix_items <= 0) return cudaSuccess;
-  fixup_kernel<PREC><<<(fix_items + kFixWarps - 1) / kFixWarps, kFixWarps * 32, 0, s>>>(a);
+  const bool split = a.nseg_cap > kFixSolo;
+  const dim3 grid(split ? fix_items : (fix_items + kFixWarps - 1) / kFixWarps,
+                  split ? (a.nseg_cap + kFixWarps - 1) / kFixWarps : 1);
+  fixup_kernel<PREC><<<grid, kFixWarps * 32, 0, s>>>(a);
   return cudaGetLastError();
 }
 
