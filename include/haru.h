@@ -84,6 +84,8 @@ typedef struct {
 } haru_event_params;
 
 typedef struct {
+  /* launch shape of batches with an explicit units_target or ctas_per_sm, and of start-column batches (the
+   * default, units_target = 0 and ctas_per_sm = 0, spreads a batch by the planner's cost model instead) */
   int warps_per_cta;        /* warps (queries or query pairs) sharing one reference tile stream: 2, 4, 8
                                or 12 (start-column batches run at most 8); other values = 8 */
   int tile_cols;            /* reference columns per shared-memory tile, 2048..16384; 0 = auto */
@@ -99,7 +101,8 @@ typedef struct {
                                serve_budget_bytes gives (a batch holds admitted reads only) */
   uint32_t serve_prefix;    /* events per decision prefix; 0 = 250 (Section 4.1) */
   int units_target;         /* work units (query x reference segment) a batch is cut into, at least;
-                               0 = 4 x SMs x warps_per_cta; 1 = never split the reference */
+                               0 = by the planner's cost model (4 x SMs x warps_per_cta where the launch
+                               shape above applies); 1 = never split the reference */
   int stack_short;          /* queries of at most 256 events stacked two to a warp strip (lanes 0-15
                                and 16-31), doubling the rows each lane sweeps: more throughput, but
                                each strip takes longer. 0 (default) = in batches of at least
@@ -422,14 +425,14 @@ int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float *events, c
                             uint32_t nq, float *out_cost, int64_t *out_col, uintptr_t stream, uint32_t flags);
 
 /* Autotuner: run the batch path on this batch (layout and flags as in
- * haru_sdtw_batch; HARU_ON_DEVICE and HARU_RAW are honoured) under every
- * combination of warps per CTA {4, 8, 12}, tile width {2048, 4096, 8192, 16384}
- * and work-unit target {1 (no reference segments), auto / 2, auto,
- * 2 x auto}, then, at the best of those, every stack_short rule (auto,
- * always, never: 32-lane strips or stacked 16-lane strips of twice the rows
- * per lane for queries of <= 256 events), keep the fastest (minimum of two
- * timed runs each) in the context's configuration
- * for later batches, and copy the resulting configuration to *chosen (may be
+ * haru_sdtw_batch; HARU_ON_DEVICE and HARU_RAW are honoured) under the
+ * planner's cost model (units_target 0) and under every combination of warps
+ * per CTA {4, 8, 12}, tile width {2048, 4096, 8192, 16384} and work-unit
+ * target {1 (no reference segments), 4 x SMs x 8, twice that}, then, at the
+ * best of those, every stack_short rule (auto, always, never: 32-lane strips
+ * or stacked 16-lane strips of twice the rows per lane for queries of <= 256
+ * events), keep the fastest (minimum of two timed runs each) in the context's
+ * configuration for later batches, and copy the resulting configuration to *chosen (may be
  * NULL). The strip height is fixed by each query's length. Results of the
  * trial runs are discarded. Errors: as haru_sdtw_batch. */
 int haru_autotune(haru_ctx *ctx, int precision, const float *events, const uint32_t *offsets, uint32_t nq,

@@ -66,9 +66,10 @@ haru::LaunchCfg haru_ctx::launch_cfg() const {
   lc.tile = pick_tile(cfg);
   lc.ctas_per_sm = cfg.ctas_per_sm;
   lc.sms = sms;
-  lc.units_target = cfg.units_target;
+  lc.units_target = std::max(cfg.units_target, 0);
   lc.stack_short = cfg.stack_short > 0 ? 1 : (cfg.stack_short < 0 ? -1 : 0);
   lc.wait_ns = wait_ns(cfg);
+  lc.N = static_cast<long>(N);
   return lc;
 }
 

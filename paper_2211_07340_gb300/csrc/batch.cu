@@ -18,7 +18,7 @@ cudaError_t record_event(cudaEvent_t e, cudaStream_t s) {
 }
 
 void ws_free(Workspace &ws) {
-  void *p[] = {ws.ints, ws.items, ws.arrived, ws.groups, ws.img, ws.states, ws.bests, ws.qstats};
+  void *p[] = {ws.ints, ws.items, ws.arrived, ws.groups, ws.sched, ws.done, ws.img, ws.states, ws.bests, ws.qstats};
   for (void *q : p)
     if (q) cudaFree(q);
   ws = Workspace();
@@ -26,82 +26,147 @@ void ws_free(Workspace &ws) {
 
 namespace {
 
+// Tile of a warp's own stream: two slots of (kSoloTile + kRefFront) words and
+// the tracking ring leave room for twelve warps in an SM's shared memory.
+constexpr int kSoloTile = 1536;
+
+// Clocks of one step of a strip of 1 .. 16 rows per lane, per warp of its
+// scheduler: with all twelve of the CTA at work (three a scheduler), and how many more on stacked items, with two warps and with
+// one. Measured on GB300, one strip height at a time, 152 CTAs (60,000 columns).
+struct StepClocks {
+  float full[kMaxS], stacked, two, one;
+};
+const StepClocks kStepI16 = {{21.3f, 21.5f, 25.7f, 28.7f, 34.4f, 39.7f, 44.6f, 47.5f, 53.4f, 59.5f, 64.1f, 67.1f,
+                              74.4f, 76.5f, 81.2f, 84.7f}, 2.0f, 6.0f, 23.0f};
+const StepClocks kStepF32 = {{19.0f, 18.0f, 21.2f, 23.8f, 28.9f, 32.4f, 37.5f, 41.9f, 47.2f, 51.5f, 56.1f, 59.0f,
+                              63.7f, 68.2f, 71.4f, 75.5f}, 1.4f, 4.0f, 13.0f};
+const StepClocks &step_clocks(int precision) {
+  return precision == HARU_INT16 ? kStepI16 : kStepF32;
+}
+
+// Work units that an explicit launch shape is cut into, and the count a batch
+// has to reach for its short queries to be stacked.
+long stack_units(int precision, const LaunchCfg &lc) {
+  return lc.units_target > 0 ? lc.units_target : 4L * lc.sms * kernel_warps(precision, lc);
+}
+
 // Buffer sizes one batch of nq queries needs.
 struct WsNeeds {
-  size_t max_items, units, qstats, states;
-  int nseg_cap, units_target;
+  size_t max_items, units, groups, ctas, qstats, states;
+  int nseg_cap;
 };
 
 WsNeeds ws_needs(int precision, uint32_t nq, const LaunchCfg &lc) {
   WsNeeds w;
+  const BatchShape sh = batch_shape(precision, nq, lc);
   const int mode = plan_mode(precision);
   w.max_items = items_bound(mode, nq);
-  // Work units: enough (query x reference segment) units to keep every SM
-  // busy to the end; nseg_cap bounds the segments per item for storage.
-  w.units_target = lc.units_target > 0 ? lc.units_target : 4 * lc.sms * kernel_warps(precision, lc);
   // Fewest items the batch can make (stacked: four int16 or two other
   // queries per item); the segment cap is sized for that case.
-  const size_t items_min = (mode == 0 || mode == 3) ? (static_cast<size_t>(nq) + 1) / 2
-                                                   : (static_cast<size_t>(nq) + 3) / 4;
-  // (twice that: the planner doubles the segments of the queue's tail)
-  w.nseg_cap = static_cast<int>(std::min<size_t>(
-      kMaxSeg, 2 * ((static_cast<size_t>(w.units_target) + items_min - 1) / std::max<size_t>(items_min, 1))));
-  if (w.nseg_cap < 1) w.nseg_cap = 1;
+  const size_t per_item = (mode == 1 ? 2 : 1) * (sh.stack ? 2 : 1);
+  const size_t items_min = (static_cast<size_t>(nq) + per_item - 1) / per_item;
+  if (!sh.solo) {
+    // (twice the wanted segments: the planner doubles those of the queue's tail)
+    const size_t units = static_cast<size_t>(stack_units(precision, lc));
+    w.nseg_cap = static_cast<int>(std::min<size_t>(64, 2 * ((units + items_min - 1) / items_min)));
+  } else {
+    // the cost model spreads a batch over at most about two units per resident warp
+    const size_t resident = static_cast<size_t>(lc.sms) * sh.per_sm * sh.warps;
+    w.nseg_cap = static_cast<int>(std::min<size_t>(kMaxSeg, 2 + (2 * resident + items_min - 1) / items_min));
+  }
   w.units = w.max_items * static_cast<size_t>(w.nseg_cap);
+  w.ctas = static_cast<size_t>(lc.sms) * sh.per_sm;
+  w.groups = sh.solo ? 1 : (w.max_items + kMaxS) * static_cast<size_t>(w.nseg_cap);
   w.qstats = 2 * static_cast<size_t>(nq);
-  w.states = w.nseg_cap > 1 ? w.units * 2 * state_words(precision) : 0;
+  w.states = w.units * 2 * state_words(precision);
   return w;
 }
 
-cudaError_t ws_alloc(Workspace &ws, size_t max_items, size_t units, size_t qstats, size_t states) {
+cudaError_t ws_alloc(Workspace &ws, const WsNeeds &w) {
   cudaError_t e = cudaSuccess;
   size_t c = ws.ints ? static_cast<size_t>(kIntWords) : 0;
   if ((e = grow(&ws.ints, &c, kIntWords)) != cudaSuccess) return e;
-  if (ws.cap_items < max_items) {
+  size_t cs = ws.sched ? 1 : 0;
+  if ((e = grow(&ws.sched, &cs, 1)) != cudaSuccess) return e;
+  if (ws.cap_items < w.max_items) {
     cudaFree(ws.items);
     cudaFree(ws.arrived);
-    cudaFree(ws.groups);
     cudaFree(ws.img);
     ws.items = nullptr;
     ws.arrived = nullptr;
-    ws.groups = nullptr;
     ws.img = nullptr;
     ws.cap_items = 0;
-    size_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;
-    if ((e = grow(&ws.items, &c0, max_items)) != cudaSuccess) return e;
-    if ((e = grow(&ws.arrived, &c3, max_items)) != cudaSuccess) return e;
-    if ((e = grow(&ws.groups, &c1, (max_items + kMaxS) * kMaxSeg)) != cudaSuccess) return e;
-    if ((e = grow(&ws.img, &c2, max_items * kImgStride)) != cudaSuccess) return e;
-    ws.cap_items = max_items;
+    size_t c0 = 0, c1 = 0, c2 = 0;
+    if ((e = grow(&ws.items, &c0, w.max_items)) != cudaSuccess) return e;
+    if ((e = grow(&ws.arrived, &c1, w.max_items)) != cudaSuccess) return e;
+    if ((e = grow(&ws.img, &c2, w.max_items * kImgStride)) != cudaSuccess) return e;
+    ws.cap_items = w.max_items;
   }
-  if ((e = grow(&ws.bests, &ws.cap_bests, 2 * units)) != cudaSuccess) return e;
-  if ((e = grow(&ws.qstats, &ws.cap_qstats, qstats)) != cudaSuccess) return e;
-  if (states > 0 && (e = grow(&ws.states, &ws.cap_states, states)) != cudaSuccess) return e;
-  return cudaSuccess;
+  if ((e = grow(&ws.groups, &ws.cap_groups, w.groups)) != cudaSuccess) return e;
+  if ((e = grow(&ws.done, &ws.cap_done, w.ctas)) != cudaSuccess) return e;
+  if ((e = grow(&ws.bests, &ws.cap_bests, 2 * w.units)) != cudaSuccess) return e;
+  if ((e = grow(&ws.qstats, &ws.cap_qstats, w.qstats)) != cudaSuccess) return e;
+  return grow(&ws.states, &ws.cap_states, w.states);
 }
 
 }  // namespace
 
+// One CTA per SM with as many warps as the kernel's registers allow, each
+// with its own tiles, on the planner's static schedule, which has a CTA's
+// warps run one strip height at a time: the instruction cache holds about
+// one (three four-warp CTAs of different heights took twice as long on 1,500
+// uneven reads), and units of any segments spread evenly over the schedulers
+// (CTAs of one warp left some with three and others with none). An explicit
+// unit target or CTA count, and the start-column forms (two strip heights of
+// whose code do not fit the cache together: 512 uneven queries took 5.4 ms,
+// 4.1 from the queue), run the configured shape: groups from a queue, each
+// sharing one stream of configured tiles.
+BatchShape batch_shape(int precision, uint32_t nq, const LaunchCfg &lc) {
+  BatchShape sh;
+  const long seg_room = std::min<long>(64, lc.N / 8192);
+  const long units = stack_units(precision, lc);
+  // Auto stacking: when the batch alone fills the unit count, or when its
+  // stacked items (up to four queries each) cut into reference segments
+  // (at most 64, each counted as 8,192 steps: about four warm-ups of a 16-row strip)
+  // still do; small batches on short references stay unstacked for latency.
+  const bool fills = static_cast<long>(nq) >= units || static_cast<long>(nq) * seg_room >= 4 * units;
+  sh.stack = lc.stack_short > 0 || (lc.stack_short == 0 && fills);
+  sh.warps = kernel_warps(precision, lc);
+  sh.tile = lc.tile;
+  sh.solo = false;
+  sh.per_sm = lc.ctas_per_sm > 0 ? lc.ctas_per_sm : 0;
+  if (sh.per_sm == 0) sh.per_sm = sdtw_max_ctas_per_sm(precision, sh.tile, sh.warps, 0);
+  if (lc.units_target == 0 && lc.ctas_per_sm == 0 && !prec_span(precision)) {
+    sh.solo = true;
+    sh.warps = kMaxWarps;
+    sh.tile = kSoloTile;
+    sh.per_sm = 1;
+  }
+  if (sh.per_sm < 1) sh.per_sm = 1;
+  return sh;
+}
+
 cudaError_t ws_reserve(Workspace &ws, int precision, uint32_t nq, const LaunchCfg &lc) {
   const WsNeeds w = ws_needs(precision, nq, lc);
-  cudaError_t e = ws_alloc(ws, w.max_items, w.units, w.qstats, w.states);
+  cudaError_t e = ws_alloc(ws, w);
   if (e != cudaSuccess) return e;
   ws.max_items = w.max_items;
   ws.nseg_cap = w.nseg_cap;
-  ws.units_target = w.units_target;
   return cudaSuccess;
 }
 
 cudaError_t ws_reserve_upto(Workspace &ws, int precision, uint32_t max_nq, const LaunchCfg &lc) {
-  size_t items = 0, units = 0, qstats = 0, states = 0;
+  WsNeeds most{};
   for (uint32_t n = 1; n <= max_nq; ++n) {  // sizing arithmetic only; one allocation per buffer
     const WsNeeds w = ws_needs(precision, n, lc);
-    items = std::max(items, w.max_items);
-    units = std::max(units, w.units);
-    qstats = std::max(qstats, w.qstats);
-    states = std::max(states, w.states);
+    most.max_items = std::max(most.max_items, w.max_items);
+    most.units = std::max(most.units, w.units);
+    most.groups = std::max(most.groups, w.groups);
+    most.ctas = std::max(most.ctas, w.ctas);
+    most.qstats = std::max(most.qstats, w.qstats);
+    most.states = std::max(most.states, w.states);
   }
-  return ws_alloc(ws, items, units, qstats, states);
+  return ws_alloc(ws, most);
 }
 
 cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const float *d_events,
@@ -117,17 +182,19 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
   pa.nq = nq;
   pa.N = ref.N;
   pa.pair = plan_mode(precision);
-  const int warps = kernel_warps(precision, lc);
-  pa.warps = warps;
-  pa.units_target = ws.units_target;
-  // Auto stacking: when the batch alone fills the unit target, or when its
-  // stacked items (up to four queries each) cut into reference segments
-  // (at most 64, each counted as 8,192 steps: about four warm-ups of a 16-row strip)
-  // still do; small batches on short references stay unstacked for latency.
-  const long seg_room = std::min<long>(kMaxSeg, ref.N / 8192);
-  const bool fills = nq >= static_cast<uint32_t>(ws.units_target) ||
-                     static_cast<long>(nq) * seg_room >= 4L * ws.units_target;
-  pa.stack = lc.stack_short > 0 || (lc.stack_short == 0 && fills) ? 1 : 0;
+  const BatchShape sh = batch_shape(precision, nq, lc);
+  pa.warps = sh.warps;
+  pa.units_target = sh.solo ? 0 : static_cast<int>(stack_units(precision, lc));
+  const int slots = lc.sms * sh.per_sm;
+  pa.slots = slots;
+  const StepClocks &sc = step_clocks(precision);
+  for (int S = 1; S <= kMaxS; ++S) pa.clocks[S - 1] = sc.full[S - 1];
+  pa.stacked = sc.stacked;
+  pa.two = sc.two;
+  pa.one = sc.one;
+  pa.sched = ws.sched;
+  pa.done = ws.done;
+  pa.stack = sh.stack ? 1 : 0;
   pa.nseg_cap = ws.nseg_cap;
   pa.items = ws.items;
   pa.arrived = ws.arrived;
@@ -165,23 +232,24 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
   sa.states = ws.states;
   sa.bests = ws.bests;
   sa.bests2 = ws.bests + ws.max_items * static_cast<size_t>(ws.nseg_cap);
+  sa.sched = ws.sched;
+  sa.done = ws.done;
   sa.arrived = ws.arrived;
   sa.out_start = d_start;
   sa.nseg_cap = ws.nseg_cap;
   sa.out_cost = d_cost;
   sa.out_col = d_col;
   sa.inv_scale = 1.0f / static_cast<float>(1 << ref.scale_log2);
-  sa.tile_cols = lc.tile;
-  sa.warps = warps;
+  sa.tile_cols = sh.tile;
+  sa.warps = sh.warps;
+  sa.solo = sh.solo;
   sa.wait_ns = lc.wait_ns;
-  const size_t groups_max = ((ws.max_items + warps - 1) / warps + kMaxS) * static_cast<size_t>(ws.nseg_cap);
   if (ev_sweep && (e = record_event(ev_sweep, s)) != cudaSuccess) return e;
   // One persistent sweep kernel over the whole group list (tallest strips
   // first), then the fix-up kernel, which verifies segments and writes every
   // query's result.
-  int per_sm = lc.ctas_per_sm > 0 ? lc.ctas_per_sm : sdtw_max_ctas_per_sm(precision, lc.tile, warps);
-  if (per_sm < 1) per_sm = 1;
-  const int grid = static_cast<int>(std::min<size_t>(static_cast<size_t>(lc.sms) * per_sm, groups_max));
+  const size_t groups_max = ((ws.max_items + sh.warps - 1) / sh.warps + kMaxS) * static_cast<size_t>(ws.nseg_cap);
+  const int grid = sh.solo ? slots : static_cast<int>(std::min<size_t>(slots, groups_max));
   return launch_sdtw(precision, sa, grid, static_cast<int>(ws.max_items), s, ev_fix);
 }
 

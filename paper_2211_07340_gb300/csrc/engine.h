@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <condition_variable>
 #include <cstdint>
@@ -36,7 +37,8 @@ struct LaunchCfg {
   int tile = 4096;
   int ctas_per_sm = 0;
   int sms = 1;
-  int units_target = 0;  // 0: 4 x sms x warps
+  int units_target = 0;  // work units to cut a batch into; 0: the planner's cost model
+  long N = 0;            // reference columns
   int stack_short = 0;   // stack short queries: 0 auto (batch >= units target), 1 always, -1 never
   unsigned long long wait_ns = 2000000000ull;
 };
@@ -58,9 +60,18 @@ inline int plan_mode(int precision) {
 // Most items a batch of nq queries can make in `mode` (per-bucket rounding
 // included: each strip height has a plain and a stacked bucket).
 inline size_t items_bound(int mode, size_t nq) {
-  if (mode == 0 || mode == 3) return nq + kMaxS;
-  return (nq + 1) / 2 + 2 * kMaxS;
+  if (mode == 0 || mode == 3) return nq;
+  return std::min(nq, (nq + 1) / 2 + 2 * kMaxS);
 }
+
+// How a batch of nq queries is launched: warps per CTA (items per group),
+// reference tile, CTAs resident per SM, a tile stream per warp or per CTA,
+// whether short queries are stacked.
+struct BatchShape {
+  int warps, tile, per_sm;
+  bool solo, stack;
+};
+BatchShape batch_shape(int precision, uint32_t nq, const LaunchCfg &lc);
 
 // The reference as the kernels read it.
 struct RefView {
@@ -90,6 +101,10 @@ struct Workspace {
   Item *items = nullptr;
   int *arrived = nullptr;  // per item
   Group *groups = nullptr;
+  size_t cap_groups = 0;
+  Schedule *sched = nullptr;
+  int *done = nullptr;     // per CTA
+  size_t cap_done = 0;
   uint32_t *img = nullptr;
   size_t cap_items = 0;
   uint32_t *states = nullptr;
@@ -101,7 +116,6 @@ struct Workspace {
   // plan of the last reservation
   size_t max_items = 0;
   int nseg_cap = 1;
-  int units_target = 0;
 };
 
 // Size `ws` for a batch of nq queries (allocates only when it must grow).

@@ -37,17 +37,6 @@ struct Item {
 // time one strip takes, so small (latency-bound) batches stay unstacked.
 constexpr int kStackMax = 16 * 16;
 
-// Consecutive items with the same S swept over the same segment by one CTA,
-// sharing one stream of reference tiles.
-struct Group {
-  int S;
-  int first;
-  int count;
-  int seg;
-  int nseg;
-  int pad[3];
-};
-
 // Last-row minimum of one unit (item, segment): int16 halves a and b, or fp32.
 struct Best {
   int ia, ib;
@@ -65,7 +54,9 @@ constexpr int kImgStride = 2 * 16 * 32;
 // start-column forms follow them with their start columns, as many words).
 constexpr int kStateStride = 2 * 16 * 32;
 constexpr int kMaxS = 16;
-constexpr int kMaxSeg = 64;
+constexpr int kMaxWarps = 12;       // per CTA
+constexpr int kSharedHeader = 2560;  // shared-memory bytes before the tracking rings
+constexpr int kMaxSeg = 320;  // segments per item, at most
 constexpr int kQmax = HARU_INT16_QMAX;
 // An int16 code as a sign-magnitude half is the fp16 number code * 2^-24 (a
 // subnormal up to 1023, then the first normal binade, whose spacing is the
@@ -110,6 +101,43 @@ __host__ __device__ constexpr int ring_words(int p) { return (prec_span(p) ? 4 :
 // Words of one saved strip state: costs, and start columns for the span forms.
 __host__ __device__ constexpr int state_words(int p) { return prec_span(p) ? 2 * kStateStride : kStateStride; }
 
+// Consecutive items with the same S swept over the same segment by one CTA,
+// sharing one stream of reference tiles (the dynamic queue of a batch with an
+// explicit unit target).
+struct Group {
+  int S;
+  int first;
+  int count;
+  int seg;
+  int nseg;
+  int pad[3];
+};
+
+// The static schedule of a batch planned by the cost model. Units (item x
+// segment, segment-major) of each strip height form bundles of `members`, run
+// by a CTA's warps side by side; the few items beyond the last full bundle
+// (`rest`) are cut into segments of their own so that theirs are full too. The bundles' estimated times, tallest strips
+// first, lie end to end on one line, and CTA p runs the line's stretch
+// [p * share, (p + 1) * share). No bundle is longer than a share, so at most
+// one crosses each border: the CTA before the border runs the bundle's first
+// steps before anything else, the one after it the remaining steps from the
+// exact state they left, after everything else. Every CTA is busy for one
+// share, and only ever waits for a CTA that started before it.
+struct ScheduleRow {
+  int items, base;       // count, first item
+  int nseg;
+  int bundles, bundle0;  // count, number of bundles before them
+  int last;              // warps at work in the last bundle
+  long long start;       // on the line
+  long long cost, last_cost;  // of a full bundle, and of the last one
+};
+struct Schedule {
+  int members, bundles;
+  long long share, total;
+  ScheduleRow row[2 * kMaxS];  // on the line from the last to the first; see schedule_row
+};
+__host__ __device__ constexpr int schedule_row(int S, int rest) { return 2 * (S - 1) + 1 - rest; }
+
 // Opt a kernel in to `bytes` of dynamic shared memory on the current
 // device, calling the driver only when the size grows past what was set
 // before on that device (a serving loop launches every few hundred
@@ -137,12 +165,12 @@ inline cudaError_t opt_in_smem(K kernel, SmemOptIn &rec, size_t bytes) {
 
 // Layout of the small integer block every batch uses: the status word, the
 // planner's group and item counts, the fix-up count, the sweep kernel's work
-// queue counter, the most segments any item was cut into and the queue
-// counter of the large-code int16 sweep.
+// queue counter, the most segments any item was cut into, the queue counter
+// of the large-code int16 sweep, and whether a sweep gave up on a wait.
 constexpr int kIntStatus = 0, kIntGroups = 1, kIntItems = 2, kIntFixups = 3, kIntQueue = 4, kIntMaxSeg = 5,
-              kIntQueueLarge = 6, kIntWords = 7;
+              kIntQueueLarge = 6, kIntAbort = 7, kIntWords = 8;
 
-__host__ __device__ inline int steps_per_chunk(int S) { return (S % 2 == 0) ? S : 2 * S; }
+__host__ __device__ inline int steps_per_chunk(int S) { return S < 8 ? 8 : S + S % 2; }
 
 // Tile width (columns) for strip height S: a multiple of lcm(U, 4) not above T.
 __host__ __device__ inline int tile_width(int S, int T) {
@@ -179,6 +207,15 @@ __host__ __device__ inline void seg_bounds(int S, int nseg, int seg, long N, lon
   *t_start = seg == 0 ? 0 : (w > 0 ? w : 0);
 }
 
+// Steps from t_start to where a bundle cut at `at` of `cost` on the schedule's
+// line stops (whole chunks; the same operands give the same cut on both sides).
+__host__ __device__ inline long cut_steps(int S, long t_start, long t_end, long long at, long long cost) {
+  const int U = steps_per_chunk(S);
+  if (at <= 0) return 0;
+  if (at >= cost) return t_end - t_start;
+  return static_cast<long>(static_cast<double>((t_end - t_start) / U) * (static_cast<double>(at) / cost)) * U;
+}
+
 struct SdtwArgs {
   const void *ref_img;     // INT16: uint32 (h | h << 16), h the half code; integer forms in FP32: (r | r << 16);
                            // FP32: float. Column 0 of N + kRefPad words, kRefFront zero words before it
@@ -193,6 +230,9 @@ struct SdtwArgs {
   uint32_t *states;        // [item][nseg_cap][2] saved states (start, final), kStateStride words each
   Best *bests;             // [item][nseg_cap]: the strip's (upper stack's) last-row minimum
   Best *bests2;            // [item][nseg_cap]: the lower stack's, for stacked items
+  const Schedule *sched;   // the static schedule (solo)
+  int *done;               // [CTA]: whether its part of the bundle across its right border is done (solo; zeroed by
+                           // the planner)
   int *arrived;            // [item]: CTAs of the fix-up kernel that verified their segments (zeroed by the planner)
   int64_t *out_start;      // span forms: the alignment start column per query
   int nseg_cap;
@@ -201,6 +241,7 @@ struct SdtwArgs {
   float inv_scale;         // INT16: 2^-k
   int tile_cols;           // requested tile width T (columns)
   int warps;               // warps per CTA = items per group
+  int solo;                // static schedule, each warp streams its own tiles; else the queue of groups
   unsigned long long wait_ns;
 };
 
@@ -211,8 +252,13 @@ struct PlanArgs {
   long N;
   int pair;                 // 0: FP32 singles; 1: INT16 pairs; 3: exact-integer singles, unsaturated
                             // (HARU_INT16_ACC32)
-  int warps;                // items per group
-  int units_target;         // wanted work units (item x segment) in the batch
+  int warps;                // warps per CTA (explicit unit target: items per group)
+  int units_target;         // wanted work units (item x segment) in the batch; 0: by the cost model below
+  int slots;                // cost model: CTAs
+  float clocks[kMaxS];      //   clocks of a step of S rows per lane and warp, with all of the CTA's warps at work;
+  float stacked, two, one;  //   more of them on stacked items, with two warps, and with one, on a scheduler
+  Schedule *sched;          //   result
+  int *done;                //   zeroed, one word per CTA
   int stack;                // 1: stack queries of <= kStackMax events two to a strip
   int nseg_cap;             // most segments per item (state storage is sized for it)
   Item *items;
@@ -249,8 +295,8 @@ cudaError_t record_event(cudaEvent_t e, cudaStream_t s);
 // and the sweep and fix-up kernels of a precision.
 cudaError_t load_prep_kernels();
 cudaError_t load_sdtw(int precision);
-size_t sdtw_smem_bytes(int precision, int tile_cols, int warps);
-int sdtw_max_ctas_per_sm(int precision, int tile_cols, int warps);
+size_t sdtw_smem_bytes(int precision, int tile_cols, int warps, int solo);
+int sdtw_max_ctas_per_sm(int precision, int tile_cols, int warps, int solo);
 
 // Reference preparation.
 cudaError_t launch_ref_levels(const uint8_t *bases, size_t n, const float *model, int k, float *out,

@@ -28,7 +28,7 @@ namespace {
 // per query, the int16 form one per pair) and each query's mean and sigma
 // (raw events). This path never splits the reference into segments, so it
 // needs no saved states.
-constexpr size_t kNaItems = HARU_NOALLOC_MAX_QUERIES + kMaxS;  // items_bound(0, max), >= items_bound(1, max)
+constexpr size_t kNaItems = HARU_NOALLOC_MAX_QUERIES + kMaxS;  // items_bound(0, max), and kMaxS short groups
 constexpr size_t kNaHead = 256;  // kIntWords status and counter words
 constexpr size_t kNaItemsOff = kNaHead;
 constexpr size_t kNaGroupsOff = kNaItemsOff + ((kNaItems * sizeof(Item) + 255) / 256) * 256;
@@ -109,6 +109,9 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   pa.pair = precision == HARU_INT16;
   pa.warps = warps;
   pa.units_target = 1;
+  pa.slots = 1;
+  pa.sched = nullptr;
+  pa.done = nullptr;
   pa.stack = 0;  // at most HARU_NOALLOC_MAX_QUERIES queries: latency over throughput
   pa.nseg_cap = 1;
   pa.items = items;
@@ -145,6 +148,8 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   sa.states = nullptr;
   sa.bests = bests;
   sa.bests2 = bests + kNaItems;
+  sa.sched = nullptr;
+  sa.done = nullptr;
   sa.arrived = nullptr;
   sa.nseg_cap = 1;
   sa.out_cost = out_cost;
@@ -152,9 +157,10 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   sa.inv_scale = 1.0f / static_cast<float>(1 << ref.scale_log2);
   sa.tile_cols = tile;
   sa.warps = warps;
+  sa.solo = 0;
   sa.wait_ns = wait;
   const size_t groups_max = (max_items + warps - 1) / warps + kMaxS;
-  const int cps = per_sm > 0 ? per_sm : sdtw_max_ctas_per_sm(precision, tile, warps);
+  const int cps = per_sm > 0 ? per_sm : sdtw_max_ctas_per_sm(precision, tile, warps, 0);
   size_t grid = static_cast<size_t>(sms) * (cps > 0 ? cps : 1);
   if (grid > groups_max) grid = groups_max;
   if ((e = launch_sdtw(precision, sa, static_cast<int>(grid), static_cast<int>(max_items), s)) != cudaSuccess)

@@ -134,15 +134,164 @@ __device__ __forceinline__ bool singles(int mode) { return mode == 0 || mode == 
 __device__ __forceinline__ int stacked_items(int mode, int n) { return singles(mode) ? (n + 1) / 2 : (n + 3) / 4; }
 __device__ __forceinline__ int bucket_items(int mode, int n) { return singles(mode) ? n : (n + 1) / 2; }
 
+// Segments of each strip height and the static schedule by a cost model (the
+// whole CTA).
+//
+// A step of a strip of S rows takes I = clocks[S - 1] for each warp on its
+// scheduler when all of the CTA's warps are at work, some more with fewer. A
+// segment after the first repeats warmup_steps(S). A candidate is a longest
+// segment time h, which gives n = ceil(T * I / h) segments of each height,
+// and m warps at work per CTA; its estimate is a CTA's share: the bundles'
+// whole time over the CTAs, or the longest bundle's. Each warp estimates
+// candidates with a lane per strip height and part: kTries values of h, 2^(1/4)
+// apart, by three of m, then kTries between the best one's neighbours.
+// Segments shorter than a quarter of their warm-up buy too little for their
+// work.
+constexpr int kTries = 32;
+
+struct PlanTables {
+  int cnt[2 * (kMaxS + 1)];                                   // queries per bucket key
+  int ibase[kMaxS + 1], sbase[kMaxS + 1], icount[kMaxS + 1];  // items
+  int nseg[2 * kMaxS], full[kMaxS + 1];  // of 2 * (16 - S) + rest; items of S before its rest
+  int gbase[kMaxS + 1], gcount[kMaxS + 1];
+  float est[3 * kTries];
+  float h;  // the cost model's choice
+  int c;
+};
+
+__device__ __forceinline__ float warp_max(float v) {
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ float warp_sum(float v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+__device__ void cost_model(const PlanArgs &a, PlanTables &t) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  // lane l: strip height 16 - l / 2, its full bundles or its rest (the schedule's order)
+  const int S = kMaxS - lane / 2;
+  const bool rest = lane & 1;
+  const int items = t.icount[S];
+  const float T = static_cast<float>(sweep_steps(S, a.N)), V = static_cast<float>(warmup_steps(S));
+  const float I = a.clocks[S - 1] +
+                  (items > 0 ? a.stacked * (items - (t.sbase[S] - t.ibase[S])) / static_cast<float>(items) : 0.0f);
+  const float most_n = floorf(fminf(fmaxf(4.0f * T / V, 1.0f), static_cast<float>(a.nseg_cap)));
+  const float longest = warp_max(items > 0 ? T * I : 0.0f);
+  // all of the CTA's warps at work, or four or eight fewer (a warp per scheduler at least)
+  auto width = [&](int c) { return max(min(a.warps, 4), a.warps - 4 * c); };
+  auto segments = [&](float h) { return static_cast<int>(fminf(ceilf(T * I / h), most_n)); };
+  auto bundle = [&](int n, int warps) {  // a bundle's time
+    const int x = (warps + 3) / 4;
+    return (T / n + (n > 1 ? V : 0.0f)) * x * (I + (x * 4 >= a.warps ? 0.0f : (x == 1 ? a.one : a.two)));
+  };
+  auto time_of = [&](int units, int n, int m, float *top) {  // all bundles' time, and the longest one's
+    const int full = units / m, last = units - full * m;
+    *top = units > 0 ? bundle(n, full > 0 ? m : last) : 0.0f;
+    return full * *top + (last > 0 ? bundle(n, last) : 0.0f);
+  };
+  auto try_h = [&](float h, int round, int q) {
+    return round == 0 ? longest * exp2f(-0.25f * q) * 1.0001f
+                      : h * exp2f(0.25f * (q - 0.5f * (kTries - 1)) / (0.5f * kTries));
+  };
+  float h = longest;
+  for (int round = 0; round < 2; ++round) {
+    for (int k = warp; k < 3 * kTries; k += nw) {
+      float all = 0.0f, top = 0.0f;
+      if (items > 0 && !rest) {
+        const int n = segments(try_h(h, round, k % kTries));
+        all = time_of(items * n, n, width(k / kTries), &top);
+      }
+      const float e = fmaxf(warp_max(top), warp_sum(all) / a.slots);
+      if (lane == 0) t.est[k] = e;
+    }
+    __syncthreads();
+    if (warp == 0) {  // the smallest estimate; the wider bundles and longer segments on a tie
+      float e = t.est[lane];
+      int at = lane;
+      for (int k = lane + 32; k < 3 * kTries; k += 32)
+        if (t.est[k] < e) { e = t.est[k]; at = k; }
+      for (int o = 16; o > 0; o >>= 1) {
+        const float oe = __shfl_xor_sync(0xffffffffu, e, o);
+        const int oat = __shfl_xor_sync(0xffffffffu, at, o);
+        if (oe < e || (oe == e && oat < at)) { e = oe; at = oat; }
+      }
+      if (lane == 0) {
+        t.h = try_h(h, round, at % kTries);
+        t.c = at / kTries;
+      }
+    }
+    __syncthreads();
+    h = t.h;
+  }
+  if (warp == 0) {
+    const int m = width(t.c);
+    int n = items > 0 ? segments(h) : 1;
+    // Items beyond those whose n segments fill whole bundles: they take the
+    // multiple of n (up to kMore) that runs them in the least time.
+    constexpr int kMore = 6;
+    int g = m;  // m / gcd(m, n): items that fill bundles together
+    for (int f = 2; f <= 3; ++f)
+      for (int k = n; g % f == 0 && k % f == 0; k /= f) g /= f;
+    const int own = rest ? items % g : items - items % g;
+    if (rest && own > 0) {
+      const int base = n;
+      float least = 0.0f, top_k;
+      for (int k = 1; k <= kMore && base * k <= static_cast<int>(fmaxf(most_n, base)); ++k) {
+        const float all_k = time_of(own * base * k, base * k, m, &top_k);
+        if (k == 1 || all_k < least) { least = all_k; n = base * k; }
+      }
+    }
+    const int units = own * n, bundles = (units + m - 1) / m, last = units - (bundles - 1) * m;
+    const long long cost = own > 0 ? static_cast<long long>(bundle(n, m)) + 1 : 0;
+    const long long last_cost = own > 0 ? static_cast<long long>(bundle(n, last)) + 1 : 0;
+    const long long all = bundles > 0 ? (bundles - 1) * cost + last_cost : 0;
+    long long end = all, top = bundles > 1 ? cost : last_cost;
+    int bend = bundles;
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long v = __shfl_up_sync(0xffffffffu, end, o);
+      const int b = __shfl_up_sync(0xffffffffu, bend, o);
+      if (lane >= o) { end += v; bend += b; }
+    }
+    for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    t.nseg[lane] = n;
+    if (!rest) t.full[S] = own;
+    ScheduleRow r;
+    r.items = own;
+    r.base = t.ibase[S] + (rest ? items - own : 0);
+    r.nseg = n;
+    r.bundles = bundles;
+    r.bundle0 = bend - bundles;
+    r.last = last;
+    r.start = end - all;
+    r.cost = cost;
+    r.last_cost = last_cost;
+    a.sched->row[schedule_row(S, rest)] = r;
+    if (lane == 31) {
+      a.sched->members = m;
+      a.sched->bundles = bend;
+      a.sched->total = end;
+      a.sched->share = max(top, (end + a.slots - 1) / a.slots);
+      a.ints[kIntGroups] = bend;
+    }
+    const int most = __reduce_max_sync(0xffffffffu, own > 0 ? n : 0);
+    if (lane == 0) a.ints[kIntMaxSeg] = most;
+  }
+  for (int p = threadIdx.x; p < a.slots; p += blockDim.x) a.done[p] = 0;
+  __syncthreads();
+}
+
 // One CTA of 1024 threads. Buckets queries by strip height S (descending,
 // the longest-processing-time-first order of the work queue), keeps the
-// input order inside a bucket, pairs neighbours for the int16 form, and cuts
-// each bucket into groups of `warps` items.
+// input order inside a bucket, pairs neighbours for the int16 form, and writes
+// the static schedule or (explicit unit target) the queue of groups.
 __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
   constexpr int kKeys = 2 * (kMaxS + 1);  // plain and stacked buckets of each S
-  __shared__ int cnt[kKeys], ibase[kMaxS + 1], sbase[kMaxS + 1], icount[kMaxS + 1], nseg_of[kMaxS + 1];
-  __shared__ int gbase[kMaxS + 1], gcount[kMaxS + 1];
+  __shared__ PlanTables t;
   __shared__ int wrun[32][kKeys];  // per warp and bucket: count, then next position
+  int *const ibase = t.ibase, *const sbase = t.sbase, *const icount = t.icount;
+  auto nseg_of = [&](int S, int item) { return t.nseg[2 * (kMaxS - S) + (item - t.ibase[S] >= t.full[S] ? 1 : 0)]; };
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   int *status = a.ints + kIntStatus;
   // Each warp owns a contiguous range of queries, so bucket positions
@@ -163,79 +312,87 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
   if (tid >= 1 && tid < kKeys) {
     int c = 0;
     for (int w = 0; w < nw; ++w) {
-      const int t = wrun[w][tid];
+      const int v = wrun[w][tid];
       wrun[w][tid] = c;
-      c += t;
+      c += v;
     }
-    cnt[tid] = c;
+    t.cnt[tid] = c;
   }
   __syncthreads();
   if (tid == 0) {
     int base = 0;
     for (int S = kMaxS; S >= 1; --S) {  // plain items of height S, then stacked ones
-      const int plain = bucket_items(a.pair, cnt[S]);
-      icount[S] = plain + stacked_items(a.pair, cnt[S + kMaxS + 1]);
+      const int plain = bucket_items(a.pair, t.cnt[S]);
+      icount[S] = plain + stacked_items(a.pair, t.cnt[S + kMaxS + 1]);
       ibase[S] = base;
       sbase[S] = base + plain;
       base += icount[S];
     }
     a.ints[kIntItems] = base;
-    // Segments per item: enough work units for the machine, each segment
-    // at least four warm-ups (and 2048 steps) long.
-    int want = base > 0 ? (a.units_target + base - 1) / base : 1;
-    if (want < 1) want = 1;
-    if (want > a.nseg_cap) want = a.nseg_cap;
-    // The buckets at the end of the longest-first queue (the cheapest strips,
-    // up to a fifth of the work) get twice the segments: shorter final work
-    // units leave less of the machine idle while the last ones finish.
-    long total = 0, acc = 0;
-    for (int S = 1; S <= kMaxS; ++S) total += static_cast<long>(icount[S]) * S;
-    int tail_to = 0;  // buckets S <= tail_to form the tail
-    if (a.units_target > 1) {
-      for (int S = 1; S <= kMaxS; ++S) {
-        const long w = static_cast<long>(icount[S]) * S;
-        if ((acc + w) * 5 > total) break;
-        acc += w;
-        tail_to = S;
+    a.ints[kIntQueue] = 0;
+    if (a.units_target > 0) {
+      // An explicit unit target: segments per item to reach it, each
+      // at least four warm-ups (and 2048 steps) long.
+      int want = base > 0 ? (a.units_target + base - 1) / base : 1;
+      if (want < 1) want = 1;
+      if (want > a.nseg_cap) want = a.nseg_cap;
+      // The buckets at the end of the longest-first queue (the cheapest strips,
+      // up to a fifth of the work) get twice the segments: shorter final work
+      // units leave less of the machine idle while the last ones finish.
+      long total = 0, acc = 0;
+      for (int S = 1; S <= kMaxS; ++S) total += static_cast<long>(icount[S]) * S;
+      int tail_to = 0;  // buckets S <= tail_to form the tail
+      if (a.units_target > 1) {
+        for (int S = 1; S <= kMaxS; ++S) {
+          const long w = static_cast<long>(icount[S]) * S;
+          if ((acc + w) * 5 > total) break;
+          acc += w;
+          tail_to = S;
+        }
+      }
+      // Groups, tallest strips first: one longest-first queue for the sweep kernel.
+      int g = 0;
+      for (int S = kMaxS; S >= 1; --S) {
+        const long minlen = 4 * warmup_steps(S) > 2048 ? 4 * warmup_steps(S) : 2048;
+        long lim = sweep_steps(S, a.N) / minlen;
+        if (lim < 1) lim = 1;
+        int ws = S <= tail_to ? 2 * want : want;
+        if (ws > a.nseg_cap) ws = a.nseg_cap;
+        const int n = ws < lim ? ws : static_cast<int>(lim);
+        t.nseg[2 * (kMaxS - S)] = n;
+        t.full[S] = icount[S];
+        t.gbase[S] = g;
+        t.gcount[S] = n * ((icount[S] + a.warps - 1) / a.warps);
+        g += t.gcount[S];
+      }
+      a.ints[kIntGroups] = g;
+      int most = 0;
+      for (int S = 1; S <= kMaxS; ++S)
+        if (icount[S] > 0 && t.nseg[2 * (kMaxS - S)] > most) most = t.nseg[2 * (kMaxS - S)];
+      a.ints[kIntMaxSeg] = most;
+    }
+  }
+  __syncthreads();
+  if (a.units_target == 0) {
+    cost_model(a, t);
+  } else {
+    // Groups of each bucket, segment-major: (seg, first item), in parallel.
+    for (int S = kMaxS; S >= 1; --S) {
+      const int per_seg = (icount[S] + a.warps - 1) / a.warps;
+      for (int j = tid; j < t.gcount[S]; j += blockDim.x) {
+        const int seg = j / per_seg, f = (j % per_seg) * a.warps;
+        Group gr;
+        gr.S = S;
+        gr.first = ibase[S] + f;
+        gr.count = icount[S] - f < a.warps ? icount[S] - f : a.warps;
+        gr.seg = seg;
+        gr.nseg = t.nseg[2 * (kMaxS - S)];
+        gr.pad[0] = gr.pad[1] = gr.pad[2] = 0;
+        a.groups[t.gbase[S] + j] = gr;
       }
     }
-    // Groups, tallest strips first: one longest-first queue for the sweep kernel.
-    int g = 0;
-    a.ints[kIntQueue] = 0;
-    for (int S = kMaxS; S >= 1; --S) {
-      const long minlen = 4 * warmup_steps(S) > 2048 ? 4 * warmup_steps(S) : 2048;
-      long lim = sweep_steps(S, a.N) / minlen;
-      if (lim < 1) lim = 1;
-      int ws = S <= tail_to ? 2 * want : want;
-      if (ws > a.nseg_cap) ws = a.nseg_cap;
-      nseg_of[S] = ws < lim ? ws : static_cast<int>(lim);
-      gbase[S] = g;
-      gcount[S] = nseg_of[S] * ((icount[S] + a.warps - 1) / a.warps);
-      g += gcount[S];
-    }
-    a.ints[kIntGroups] = g;
-    int most = 0;
-    for (int S = 1; S <= kMaxS; ++S)
-      if (icount[S] > 0 && nseg_of[S] > most) most = nseg_of[S];
-    a.ints[kIntMaxSeg] = most;
+    __syncthreads();
   }
-  __syncthreads();
-  // Groups of each bucket, segment-major: (seg, first item), in parallel.
-  for (int S = kMaxS; S >= 1; --S) {
-    const int per_seg = (icount[S] + a.warps - 1) / a.warps;
-    for (int j = tid; j < gcount[S]; j += blockDim.x) {
-      const int seg = j / per_seg, f = (j % per_seg) * a.warps;
-      Group gr;
-      gr.S = S;
-      gr.first = ibase[S] + f;
-      gr.count = icount[S] - f < a.warps ? icount[S] - f : a.warps;
-      gr.seg = seg;
-      gr.nseg = nseg_of[S];
-      gr.pad[0] = gr.pad[1] = gr.pad[2] = 0;
-      a.groups[gbase[S] + j] = gr;
-    }
-  }
-  __syncthreads();
   const int n_items = a.ints[kIntItems];
   for (int i = tid; i < n_items; i += blockDim.x) {
     Item it;
@@ -256,8 +413,9 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
       const int pos = wrun[warp][key] + __popc(peers & lt);
       const int per = singles(a.pair) ? 2 : 4;
       const int slot = singles(a.pair) ? 2 * (pos % 2) : pos % 4;
-      Item *it = &a.items[sbase[b] + pos / per];
-      if (slot == 0) { it->qa = static_cast<int>(q); it->S = b; it->nseg = nseg_of[b]; it->stacked = 1; }
+      const int item = sbase[b] + pos / per;
+      Item *it = &a.items[item];
+      if (slot == 0) { it->qa = static_cast<int>(q); it->S = b; it->nseg = nseg_of(b, item); it->stacked = 1; }
       else if (slot == 1) it->qb = static_cast<int>(q);
       else if (slot == 2) it->qc = static_cast<int>(q);
       else it->qd = static_cast<int>(q);
@@ -265,12 +423,13 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
       const int b = key;
       const int pos = wrun[warp][b] + __popc(peers & lt);  // position in bucket b
       if (a.pair == 1) {
-        Item *it = &a.items[ibase[b] + pos / 2];
-        if (pos % 2 == 0) { it->qa = static_cast<int>(q); it->S = b; it->nseg = nseg_of[b]; }
+        const int item = ibase[b] + pos / 2;
+        Item *it = &a.items[item];
+        if (pos % 2 == 0) { it->qa = static_cast<int>(q); it->S = b; it->nseg = nseg_of(b, item); }
         else it->qb = static_cast<int>(q);
       } else {
         Item it;
-        it.qa = static_cast<int>(q); it.qb = -1; it.S = b; it.nseg = nseg_of[b];
+        it.qa = static_cast<int>(q); it.qb = -1; it.S = b; it.nseg = nseg_of(b, ibase[b] + pos);
         it.qmax = 0;
         it.qc = -1; it.qd = -1; it.stacked = 0;
         a.items[ibase[b] + pos] = it;

@@ -15,7 +15,7 @@ namespace haru {
 #define HARU_SDTW_DECLARE(P)                                                        \
   cudaError_t sdtw_sweep_##P(const SdtwArgs &a, int grid, cudaStream_t s);          \
   cudaError_t sdtw_fixup_##P(const SdtwArgs &a, int fix_items, cudaStream_t s);     \
-  int sdtw_occupancy_##P(int tile_cols, int warps);                                 \
+  int sdtw_occupancy_##P(int tile_cols, int warps, int solo);                                 \
   cudaError_t sdtw_sweep_load_##P();                                                \
   cudaError_t sdtw_fixup_load_##P();
 HARU_SDTW_DECLARE(0)
@@ -25,40 +25,41 @@ HARU_SDTW_DECLARE(3)
 HARU_SDTW_DECLARE(4)
 HARU_SDTW_DECLARE(5)
 
-size_t sdtw_smem_bytes(int precision, int tile_cols, int warps) {
-  // Shared header, per-warp tracking rings, two tile slots (each with the
-  // kRefFront columns before its tile)
-  return 128 + static_cast<size_t>(warps) * ring_words(precision) * 4 +
-         2 * static_cast<size_t>(tile_cols + kRefFront) * 4;
+size_t sdtw_smem_bytes(int precision, int tile_cols, int warps, int solo) {
+  // Shared header, per-warp tracking rings, two tile slots per stream (each
+  // with the kRefFront columns before its tile)
+  return kSharedHeader + static_cast<size_t>(warps) * ring_words(precision) * 4 +
+         (solo ? warps : 1) * 2 * static_cast<size_t>(tile_cols + kRefFront) * 4;
 }
 
 namespace {
-int occupancy_query(int precision, int tile_cols, int warps) {
+int occupancy_query(int precision, int tile_cols, int warps, int solo) {
   switch (precision) {
-    case HARU_INT16: return sdtw_occupancy_1(tile_cols, warps);
-    case HARU_INT16_ACC32: return sdtw_occupancy_2(tile_cols, warps);
-    case kPrecF32Span: return sdtw_occupancy_3(tile_cols, warps);
-    case kPrecWideSpan: return sdtw_occupancy_4(tile_cols, warps);
-    default: return sdtw_occupancy_0(tile_cols, warps);
+    case HARU_INT16: return sdtw_occupancy_1(tile_cols, warps, solo);
+    case HARU_INT16_ACC32: return sdtw_occupancy_2(tile_cols, warps, solo);
+    case kPrecF32Span: return sdtw_occupancy_3(tile_cols, warps, solo);
+    case kPrecWideSpan: return sdtw_occupancy_4(tile_cols, warps, solo);
+    default: return sdtw_occupancy_0(tile_cols, warps, solo);
   }
 }
 }  // namespace
 
 // Resident CTAs per SM of a launch shape, asked of the runtime once per
-// (device, precision, tile, warps): every batch launch needs it.
-int sdtw_max_ctas_per_sm(int precision, int tile_cols, int warps) {
+// (device, precision, shape): every batch launch needs it.
+int sdtw_max_ctas_per_sm(int precision, int tile_cols, int warps, int solo) {
   struct Entry {
-    int dev, precision, tile_cols, warps, ctas;
+    int dev, precision, tile_cols, warps, solo, ctas;
   };
   static std::mutex mu;
   static std::vector<Entry> memo;
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return occupancy_query(precision, tile_cols, warps);
+  if (cudaGetDevice(&dev) != cudaSuccess) return occupancy_query(precision, tile_cols, warps, solo);
   std::lock_guard<std::mutex> lk(mu);
   for (const Entry &x : memo)
-    if (x.dev == dev && x.precision == precision && x.tile_cols == tile_cols && x.warps == warps) return x.ctas;
-  const int n = occupancy_query(precision, tile_cols, warps);
-  if (n > 0) memo.push_back(Entry{dev, precision, tile_cols, warps, n});
+    if (x.dev == dev && x.precision == precision && x.tile_cols == tile_cols && x.warps == warps && x.solo == solo)
+      return x.ctas;
+  const int n = occupancy_query(precision, tile_cols, warps, solo);
+  if (n > 0) memo.push_back(Entry{dev, precision, tile_cols, warps, solo, n});
   return n;
 }
 

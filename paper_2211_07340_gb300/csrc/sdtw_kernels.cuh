@@ -36,9 +36,13 @@
 // results stand; otherwise it recomputes the segment from the exact state.
 // The result is always the plain DP's.
 //
-// The reference streams through shared memory: every CTA sweeps a group of
-// warps (same S, same segment) over the same columns; tiles of T_S columns,
-// each with the kRefFront columns before it (the lanes lag the warp's step by
+// Schedule. Units are spread over the CTAs by estimated time (Schedule): a
+// unit cut at a border between two CTAs saves its exact state there and goes
+// on from it on the other one, so balance costs no further warm-up.
+//
+// The reference streams through shared memory, one stream per warp (a CTA's
+// warps run any units of one strip height), or, with an explicit unit
+// target, one per CTA (same S, same segment). Tiles of T_S columns, each with the kRefFront columns before it (the lanes lag the warp's step by
 // up to 31 * S columns), are fetched by cp.async.bulk (TMA) into a two-slot
 // ring guarded by mbarriers. The warp that releases a slot last issues the
 // copy of the tile two ahead.
@@ -173,7 +177,11 @@ struct RingStore {
 
 template <int S>
 struct Geo {
-  static constexpr int U = (S % 2 == 0) ? S : 2 * S;  // steps per unrolled chunk (register renaming period)
+  // Steps per unrolled chunk, the period of the register renaming: the
+  // reference samples rotate through U registers and the costs alternate
+  // between two, so U is S rounded up to even; at least 8, to spread the
+  // chunk's own work (flush and segment checks) over the steps of low strips.
+  static constexpr int U = S < 8 ? 8 : S + S % 2;
 };
 
 // ---------------------------------------------------------------- INT16 --
@@ -208,7 +216,7 @@ __device__ __forceinline__ uint32_t half_diff(uint32_t q, uint32_t r) {
 // of the row above the lane.
 template <int S>
 struct StateI16 {
-  uint32_t G[2][S], Rr[S];
+  uint32_t G[2][S], Rr[Geo<S>::U];
   uint32_t gprev;
 
   // As if the reference began at the current step: every row, pad rows
@@ -224,8 +232,9 @@ struct StateI16 {
     for (int k = 0; k < S; ++k) {
       G[0][k] = kCap2;
       G[1][k] = kCap2;
-      Rr[k] = 0u;
     }
+#pragma unroll
+    for (int k = 0; k < Geo<S>::U; ++k) Rr[k] = 0u;
     gprev = ng ? kCap2 : 0u;
   }
   // Exact state before step t: G[1] = step t-1, G[0] = step t-2, and the
@@ -233,9 +242,9 @@ struct StateI16 {
   __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, uint32_t ng) {
 #pragma unroll
     for (int k = 0; k < S; ++k) {
-      G[1][k] = st[k * 32 + lane];
-      G[0][k] = st[(S + k) * 32 + lane];
-      Rr[(1 + k) % S] = gref[t - 1 - static_cast<long>(lane) * S - k];
+      G[1][k] = __ldcg(st + k * 32 + lane);
+      G[0][k] = __ldcg(st + (S + k) * 32 + lane);
+      Rr[(1 + k) % Geo<S>::U] = gref[t - 1 - static_cast<long>(lane) * S - k];
     }
     const uint32_t g = __shfl_up_sync(kFull, G[0][S - 1], 1);
     gprev = ng ? g : 0u;
@@ -261,7 +270,7 @@ struct StateI16 {
     LaneWindow<S> win;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int p = (S - (u % S)) % S;
+      const int p = (U - u) % U;
       const int a = (u + 1) & 1;
       const int b = u & 1;
       uint32_t gup = __shfl_up_sync(kFull, G[a][S - 1], 1);
@@ -274,7 +283,7 @@ struct StateI16 {
       Rr[p] = win.get(ref, u);  // row 0's reference: column t - lane * S
       uint32_t d[S], m[S];
 #pragma unroll
-      for (int k = S - 1; k >= 0; --k) d[k] = dist(k, Rr[(p + k) % S]);
+      for (int k = S - 1; k >= 0; --k) d[k] = dist(k, Rr[(p + k) % U]);
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) {
         const uint32_t up = k ? G[a][k - 1] : gup;
@@ -353,6 +362,7 @@ struct TrackI16 {
       if (ob < bb || (ob == bb && static_cast<unsigned long>(pb) < static_cast<unsigned long>(cb))) { bb = ob; cb = pb; }
     }
   }
+  __device__ __forceinline__ void merge(const Best *b);
   __device__ __forceinline__ void store(Best *b) const {
     b->ia = ba; b->ib = bb; b->f = 0.0f; b->pad = 0; b->ca = ca; b->cb = cb;
   }
@@ -364,7 +374,7 @@ struct TrackI16 {
 // int16 arithmetic, run through the FP32 units (see FormOf below).
 template <int S, bool CODES>
 struct StripF32 {
-  float Q[S], W[S], G[2][S], Rr[S];
+  float Q[S], W[S], G[2][S], Rr[Geo<S>::U];
   float gprev;
 
   __device__ __forceinline__ static float ref_value(uint32_t w) {
@@ -393,16 +403,17 @@ struct StripF32 {
     for (int k = 0; k < S; ++k) {
       G[0][k] = kBig;
       G[1][k] = kBig;
-      Rr[k] = 0.0f;
     }
+#pragma unroll
+    for (int k = 0; k < Geo<S>::U; ++k) Rr[k] = 0.0f;
     gprev = ng ? kBig : 0.0f;
   }
   __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, uint32_t ng) {
 #pragma unroll
     for (int k = 0; k < S; ++k) {
-      G[1][k] = __uint_as_float(st[k * 32 + lane]);
-      G[0][k] = __uint_as_float(st[(S + k) * 32 + lane]);
-      Rr[(1 + k) % S] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
+      G[1][k] = __uint_as_float(__ldcg(st + k * 32 + lane));
+      G[0][k] = __uint_as_float(__ldcg(st + (S + k) * 32 + lane));
+      Rr[(1 + k) % Geo<S>::U] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
     }
     const float g = __shfl_up_sync(kFull, G[0][S - 1], 1);
     gprev = ng ? g : 0.0f;
@@ -422,7 +433,7 @@ struct StripF32 {
     RingStore<U> out;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int p = (S - (u % S)) % S;
+      const int p = (U - u) % U;
       const int a = (u + 1) & 1;
       const int b = u & 1;
       float gup = __shfl_up_sync(kFull, G[a][S - 1], 1);
@@ -433,7 +444,7 @@ struct StripF32 {
       Rr[p] = ref_value(win.get(ref, u));  // row 0's reference: column t - lane * S
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) {
-        const float r = Rr[(p + k) % S];
+        const float r = Rr[(p + k) % U];
         // q - r rounded once on real rows (weight -1), exactly 0 on pad rows
         // (weight 0, q = 0); off the critical path, so the cost update that
         // depends on the minimum is a plain add
@@ -468,6 +479,7 @@ struct TrackF32 {
       }
     }
   }
+  __device__ __forceinline__ void merge(const Best *b);
   __device__ __forceinline__ void store(Best *b) const {
     b->ia = 0; b->ib = 0; b->f = best; b->pad = 0; b->ca = col; b->cb = -1;
   }
@@ -484,7 +496,7 @@ struct TrackF32 {
 // column, like the free-start row of Eq. 1. CODES as for StripF32.
 template <int S, bool CODES>
 struct StripF32Span {
-  float Q[S], W[S], G[2][S], Rr[S];
+  float Q[S], W[S], G[2][S], Rr[Geo<S>::U];
   int P[2][S];
   float gprev;
   int pprev;
@@ -514,11 +526,12 @@ struct StripF32Span {
     for (int k = 0; k < S; ++k) {
       G[0][k] = kBig;
       G[1][k] = kBig;
-      Rr[k] = 0.0f;
       const int i = lane * S + k;
       P[1][k] = static_cast<int>(t_start) - 1 - i;
       P[0][k] = static_cast<int>(t_start) - 2 - i;
     }
+#pragma unroll
+    for (int k = 0; k < Geo<S>::U; ++k) Rr[k] = 0.0f;
     gprev = ng ? kBig : 0.0f;
     pprev = static_cast<int>(t_start) - 1 - lane * S;  // the row above row 0 at step t_start - 2
   }
@@ -526,11 +539,11 @@ struct StripF32Span {
   __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, uint32_t ng) {
 #pragma unroll
     for (int k = 0; k < S; ++k) {
-      G[1][k] = __uint_as_float(st[k * 32 + lane]);
-      G[0][k] = __uint_as_float(st[(S + k) * 32 + lane]);
-      P[1][k] = static_cast<int>(st[(2 * S + k) * 32 + lane]);
-      P[0][k] = static_cast<int>(st[(3 * S + k) * 32 + lane]);
-      Rr[(1 + k) % S] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
+      G[1][k] = __uint_as_float(__ldcg(st + k * 32 + lane));
+      G[0][k] = __uint_as_float(__ldcg(st + (S + k) * 32 + lane));
+      P[1][k] = static_cast<int>(__ldcg(st + (2 * S + k) * 32 + lane));
+      P[0][k] = static_cast<int>(__ldcg(st + (3 * S + k) * 32 + lane));
+      Rr[(1 + k) % Geo<S>::U] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
     }
     const float g = __shfl_up_sync(kFull, G[0][S - 1], 1);
     const int pg = __shfl_up_sync(kFull, P[0][S - 1], 1);
@@ -556,7 +569,7 @@ struct StripF32Span {
     LaneWindow<S> win;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int p = (S - (u % S)) % S;
+      const int p = (U - u) % U;
       const int a = (u + 1) & 1;
       const int b = u & 1;
       float gup = __shfl_up_sync(kFull, G[a][S - 1], 1);
@@ -566,7 +579,7 @@ struct StripF32Span {
       Rr[p] = ref_value(win.get(ref, u));  // row 0's reference: column t - lane * S
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) {
-        const float r = Rr[(p + k) % S];
+        const float r = Rr[(p + k) % U];
         const float d = __fmaf_rn(r, W[k], Q[k]);  // q - r on real rows, 0 on pad rows
         const float up = k ? G[a][k - 1] : gup;
         const int pu = k ? P[a][k - 1] : pup;
@@ -608,6 +621,7 @@ struct TrackF32Span {
       }
     }
   }
+  __device__ __forceinline__ void merge(const Best *b);
   __device__ __forceinline__ void store(Best *b) const {
     b->ia = 0; b->ib = 0; b->f = best; b->pad = 0; b->ca = col; b->cb = start;
   }
@@ -660,23 +674,32 @@ struct FormOf<kFormWideSpan, S> {
 };
 
 // ----------------------------------------------------------- tile sources --
-// Shared state of one CTA.
-struct Shared {
+// Shared state of one tile stream (a CTA's, or each warp's own).
+struct Stream {
   uint64_t full[2];
   int cnt[2];
   int uses[2];
-  int group;
   int tile_base;
-  int abort;
-  int pad;
+  int pad[3];
 };
+// Shared state of one CTA.
+struct Shared {
+  int group;
+  int abort;
+  int stop;
+  int pad;
+  Stream streams[kMaxWarps];
+  Schedule sched;
+};
+static_assert(sizeof(Shared) <= kSharedHeader, "shared-memory header");
 
 // Reference tiles streamed into shared memory by TMA (the sweep kernel).
 // Slot of tile k: the kRefFront columns before the tile, then its
 // tile_cols columns, so a lane that reads up to 31 * S columns behind the
 // warp's step finds its samples in the current slot.
 struct TileStream {
-  Shared *sh;
+  Stream *sh;
+  int *abort;                  // the CTA's
   char *slots;                 // two slots of tile_cols + kRefFront words
   const char *src;             // reference image (column 0; kRefFront zero words before it)
   int tile_cols;               // T_S
@@ -684,7 +707,7 @@ struct TileStream {
   int K;                       // tiles in this group's sweep
   int n_active;                // warps consuming this stream
   unsigned long long wait_ns;  // longest single wait
-  int *status;
+  int *ints;
 
   __device__ void issue(int k) {  // one thread
     const int gk = sh->tile_base + k;
@@ -704,8 +727,9 @@ struct TileStream {
     const int gk = sh->tile_base + k;
     const int slot = gk & 1;
     if (!mbar_wait_bounded(&sh->full[slot], (gk >> 1) & 1, now_ns() + wait_ns)) {
-      report(status, HARU_ETIMEDOUT);
-      sh->abort = 1;
+      report(ints + kIntStatus, HARU_ETIMEDOUT);
+      ints[kIntAbort] = 1;
+      *abort = 1;
       return nullptr;
     }
     return reinterpret_cast<const uint32_t *>(slots + static_cast<size_t>(slot) * (tile_cols + kRefFront) * 4);
@@ -811,59 +835,135 @@ __device__ bool run_steps(typename FormOf<FORM, S>::Strip &st, typename FormOf<F
   return true;
 }
 
-// Speculative sweep of one unit (item, segment) in the sweep kernel.
+// Merge a unit's later steps' minimum with its earlier ones': the smaller
+// cost, the earlier (smaller) column on a tie.
+__device__ __forceinline__ void TrackI16::merge(const Best *b) {
+  const int ia = __ldcg(&b->ia), ib = __ldcg(&b->ib);
+  if (ia <= ba) { ba = ia; ca = __ldcg(&b->ca); }
+  if (ib <= bb) { bb = ib; cb = __ldcg(&b->cb); }
+}
+__device__ __forceinline__ void TrackF32::merge(const Best *b) {
+  const float f = __ldcg(&b->f);
+  if (f <= best) { best = f; col = __ldcg(&b->ca); }
+}
+__device__ __forceinline__ void TrackF32Span::merge(const Best *b) {
+  const float f = __ldcg(&b->f);
+  if (f <= best) { best = f; col = __ldcg(&b->ca); start = static_cast<int>(__ldcg(&b->cb)); }
+}
+
+// Steps [p_lo, p_hi) of the sweep of one unit (item, segment). From the
+// segment's start they start from the fresh state, otherwise from the state
+// that the steps before them saved as the unit's last one, where its final
+// state goes too.
 template <int FORM, int S>
-__device__ void sweep_unit(const SdtwArgs &A, TileStream &ts, const Group &g, int item, uint32_t *ring,
-                           int lane) {
+__device__ void sweep_unit(const SdtwArgs &A, TileStream &ts, int nseg, int seg, long p_lo, long p_hi, int item,
+                           uint32_t *ring, int lane) {
   typename FormOf<FORM, S>::Strip st;
   typename FormOf<FORM, S>::Track tr;
   st.load(A.img + static_cast<size_t>(item) * kImgStride, lane);
   long t_start, t_own, t_end;
-  seg_bounds(S, g.nseg, g.seg, A.N, &t_start, &t_own, &t_end);
-  const bool stk0 = A.items[item].stacked != 0;
-  st.fresh(t_start, lane, (stk0 ? (lane & 15) : lane) != 0 ? 1u : 0u);
-  uint32_t *ss = nullptr, *sf = nullptr;
-  const size_t unit = static_cast<size_t>(item) * A.nseg_cap + g.seg;
+  seg_bounds(S, nseg, seg, A.N, &t_start, &t_own, &t_end);
+  const bool stk = A.items[item].stacked != 0, whole = p_lo == t_start;
+  const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
+  const size_t unit = static_cast<size_t>(item) * A.nseg_cap + seg;
   constexpr size_t kWords = state_rows_per_s<FORM>() * 16 * 32;
-  if (g.seg > 0) ss = A.states + (unit * 2 + 0) * kWords;
-  if (g.seg + 1 < g.nseg) sf = A.states + (unit * 2 + 1) * kWords;
-  const bool stk = A.items[item].stacked != 0;
-  const bool ok =
-      run_steps<FORM, S>(st, tr, ts, ts.tile_cols, t_start, t_own, t_end, true, A.N, ss, sf, ring, lane, stk);
+  uint32_t *ss = nullptr, *sf = nullptr;
+  if (seg > 0) ss = A.states + (unit * 2 + 0) * kWords;
+  if (seg + 1 < nseg || p_hi < t_end) sf = A.states + (unit * 2 + 1) * kWords;
+  if (whole)
+    st.fresh(t_start, lane, ng);
+  else
+    st.restore(A.states + (unit * 2 + 1) * kWords, reinterpret_cast<const uint32_t *>(ts.src), p_lo, lane, ng);
+  const bool ok = run_steps<FORM, S>(st, tr, ts, ts.tile_cols, p_lo, t_own, p_hi, true, A.N, ss, sf, ring, lane, stk);
   tr.reduce(stk ? 16 : 32);
-  if (ok && lane == 0) tr.store(A.bests + unit);
-  if (ok && stk && lane == 16) tr.store(A.bests2 + unit);
+  if (ok && lane == 0) {
+    if (!whole) tr.merge(A.bests + unit);
+    tr.store(A.bests + unit);
+  }
+  if (ok && stk && lane == 16) {
+    if (!whole) tr.merge(A.bests2 + unit);
+    tr.store(A.bests2 + unit);
+  }
 }
 
 template <int PREC, int S>
-__device__ __forceinline__ void sweep_any(const SdtwArgs &A, TileStream &ts, const Group &g, int item,
-                                          uint32_t *ring, int lane) {
+__device__ __forceinline__ void sweep_any(const SdtwArgs &A, TileStream &ts, int nseg, int seg, long p_lo,
+                                          long p_hi, int item, uint32_t *ring, int lane) {
   if constexpr (PREC == HARU_FP32) {
-    sweep_unit<kFormF32, S>(A, ts, g, item, ring, lane);
+    sweep_unit<kFormF32, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   } else if constexpr (PREC == HARU_INT16_ACC32) {
-    sweep_unit<kFormExactWide, S>(A, ts, g, item, ring, lane);
+    sweep_unit<kFormExactWide, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   } else if constexpr (PREC == kPrecF32Span) {
-    sweep_unit<kFormF32Span, S>(A, ts, g, item, ring, lane);
+    sweep_unit<kFormF32Span, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   } else if constexpr (PREC == kPrecWideSpan) {
-    sweep_unit<kFormWideSpan, S>(A, ts, g, item, ring, lane);
+    sweep_unit<kFormWideSpan, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   } else if constexpr (PREC == kPrecI16Large) {
-    sweep_unit<kFormI16Large, S>(A, ts, g, item, ring, lane);
+    sweep_unit<kFormI16Large, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   } else {
-    sweep_unit<kFormI16, S>(A, ts, g, item, ring, lane);
+    sweep_unit<kFormI16, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   }
+}
+
+// Hand-over of the bundle across a border of the schedule (one thread,
+// between CTA barriers): the states and minima written before finish_part are
+// seen after wait_part.
+__device__ __forceinline__ void finish_part(const SdtwArgs &A, int cta) {
+  __threadfence();
+  asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(A.done + cta), "r"(1) : "memory");
+}
+__device__ __forceinline__ bool wait_part(const SdtwArgs &A, int cta, unsigned long long limit_ns) {
+  const unsigned long long deadline = now_ns() + limit_ns;
+  for (;;) {
+    int n;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(n) : "l"(A.done + cta) : "memory");
+    if (n) break;
+    if (*static_cast<volatile int *>(A.ints + kIntAbort)) return false;  // a CTA gave up: its part never finishes
+    if (now_ns() > deadline) {
+      report(A.ints + kIntStatus, HARU_ETIMEDOUT);
+      A.ints[kIntAbort] = 1;
+      return false;
+    }
+    __nanosleep(200);
+  }
+  __threadfence();
+  return true;
 }
 
 // One kernel covers every strip height S = 1..16 (registers are allocated
 // for the tallest), fed by one longest-first queue of groups.
 template <int PREC, int S = 1>
-__device__ __forceinline__ void dispatch_sweep(int s, const SdtwArgs &A, TileStream &ts, const Group &g, int item,
-                                               uint32_t *ring, int lane) {
+__device__ __forceinline__ void dispatch_sweep(int s, const SdtwArgs &A, TileStream &ts, int nseg, int seg,
+                                               long p_lo, long p_hi, int item, uint32_t *ring, int lane) {
   if constexpr (S <= kMaxS) {
     if (s == S)
-      sweep_any<PREC, S>(A, ts, g, item, ring, lane);
+      sweep_any<PREC, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
     else
-      dispatch_sweep<PREC, S + 1>(s, A, ts, g, item, ring, lane);
+      dispatch_sweep<PREC, S + 1>(s, A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   }
+}
+
+// The bundle at place x of the schedule's line: the number of bundles that
+// end at or before x; *inside: x lies within that bundle, not at its start.
+__device__ __forceinline__ int bundle_at(const Schedule &c, long long x, bool *inside) {
+  *inside = false;
+  if (x >= c.total) return c.bundles;
+  for (int k = 2 * kMaxS - 1; k >= 0; --k) {
+    const ScheduleRow &r = c.row[k];
+    if (r.bundles == 0) continue;
+    const long long y = x - r.start;
+    if (y >= (r.bundles - 1) * r.cost + r.last_cost) continue;
+    const int i = min(static_cast<int>(y / r.cost), r.bundles - 1);
+    *inside = y > i * r.cost;
+    return r.bundle0 + i;
+  }
+  return c.bundles;
+}
+// The row of bundle b.
+__device__ __forceinline__ const ScheduleRow &find_row(const Schedule &c, int b, int *S) {
+  int k = 2 * kMaxS - 1;
+  while (k > 0 && b >= c.row[k].bundle0 + c.row[k].bundles) --k;
+  *S = k / 2 + 1;
+  return c.row[k];
 }
 
 // Up to 12 warps per CTA (3 per scheduler): the int16, FP32 and wide strips
@@ -872,71 +972,139 @@ template <int PREC>
 __global__ void __launch_bounds__(prec_span(PREC) ? 256 : 384, 1) sdtw_kernel(SdtwArgs A) {
   extern __shared__ __align__(128) unsigned char smem[];
   Shared *sh = reinterpret_cast<Shared *>(smem);
-  // layout: Shared (128 B) | per-warp tracking rings | two tile slots
-  uint32_t *rings = reinterpret_cast<uint32_t *>(smem + 128);
+  // layout: Shared | per-warp tracking rings | two tile slots per stream
+  uint32_t *rings = reinterpret_cast<uint32_t *>(smem + kSharedHeader);
   constexpr int kRing = ring_words(PREC);
-  char *slots = reinterpret_cast<char *>(smem + 128 + A.warps * kRing * 4);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) {
-    mbar_init(&sh->full[0], 1);
-    mbar_init(&sh->full[1], 1);
-    sh->cnt[0] = sh->cnt[1] = 0;
-    sh->uses[0] = sh->uses[1] = 0;
-    sh->tile_base = 0;
-    sh->abort = 0;
+  constexpr bool kPairs = PREC == HARU_INT16 || PREC == kPrecI16Large;
+  const bool solo = A.solo != 0;
+  const int stream = solo ? warp : 0;
+  char *slots = reinterpret_cast<char *>(rings + A.warps * kRing) +
+                static_cast<size_t>(stream) * 2 * (A.tile_cols + kRefFront) * 4;
+  if (threadIdx.x < kMaxWarps) {
+    Stream *t = &sh->streams[threadIdx.x];
+    mbar_init(&t->full[0], 1);
+    mbar_init(&t->full[1], 1);
+    t->cnt[0] = t->cnt[1] = 0;
+    t->uses[0] = t->uses[1] = 0;
+    t->tile_base = 0;
+    if (threadIdx.x == 0) sh->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  const int count = A.ints[kIntGroups];
   int *queue = A.ints + (PREC == kPrecI16Large ? kIntQueueLarge : kIntQueue);
-  for (;;) {
+  // Static schedule: this CTA's place on the line, in the order the CTAs
+  // started, and the bundles first .. first + n - 1 that its stretch touches.
+  int place = 0, first = 0, n = 0;
+  bool left = false, right = false;  // the first / last of them crosses a border
+  const Schedule &sched = sh->sched;
+  if (solo) {
     if (threadIdx.x == 0) sh->group = atomicAdd(queue, 1);
+    for (int i = threadIdx.x; i < static_cast<int>(sizeof(Schedule) / 4); i += blockDim.x)
+      reinterpret_cast<int *>(&sh->sched)[i] = reinterpret_cast<const int *>(A.sched)[i];
     __syncthreads();
-    const int gi = sh->group;
-    if (gi >= count || sh->abort) break;
-    const Group grp = A.groups[gi];
-    if constexpr (PREC == HARU_INT16 || PREC == kPrecI16Large) {
-      // A group with a code too large for the half-code cell belongs to the
-      // large-code sweep, every other one to this form's.
-      bool large = false;
-      if (A.large_possible) {
-        const int it = lane < grp.count ? lane : 0;
-        large = __any_sync(kFull, A.items[grp.first + it].qmax > A.half_max);
-      }
-      if (large != (PREC == kPrecI16Large)) {
-        __syncthreads();  // every thread has read sh->group
-        continue;
-      }
+    place = sh->group;
+    const long long lo = place * sched.share, hi = lo + sched.share;
+    const int begin = bundle_at(sched, lo, &left), end = bundle_at(sched, hi, &right);
+    first = begin;
+    n = end - begin + (right ? 1 : 0);
+  }
+  const int count = A.ints[kIntGroups];
+  for (int e = 0;; ++e) {
+    // The next work: S, nseg, `members` warps at work, this warp's item and
+    // segment, and the part [cut_lo, cut_hi) of `cost` of its steps.
+    int S, nseg, members, item, seg;
+    long long cut_lo = 0, cut_hi = 1, cost = 1;
+    bool large = false, waits = false, hands = false;
+    if (solo) {
+      if (e >= n) break;
+      // the bundle across the right border first, the one across the left border last
+      const int b = first + (right ? (e == 0 ? n - 1 : e - 1 + (left ? 1 : 0)) : e + (left ? 1 : 0));
+      const int at = b >= first + n - (right && e > 0 ? 1 : 0) ? first : b;
+      const ScheduleRow &row = find_row(sched, at, &S);
+      const int i = at - row.bundle0;
+      const long long start = row.start + i * row.cost;
+      cost = i + 1 < row.bundles ? row.cost : row.last_cost;
+      cut_lo = place * sched.share - start;
+      cut_hi = cut_lo + sched.share;
+      waits = left && at == first;
+      hands = right && at == first + n - 1;
+      nseg = row.nseg;
+      members = i + 1 < row.bundles ? sched.members : row.last;
+      const int u0 = i * sched.members, u = u0 + min(warp, members - 1);
+      item = row.base + u % row.items;
+      seg = u / row.items;
+      if (kPairs && A.large_possible)
+        large = __any_sync(kFull, A.items[row.base + (u0 + min(lane, members - 1)) % row.items].qmax > A.half_max);
+    } else {
+      if (threadIdx.x == 0) sh->group = atomicAdd(queue, 1);
+      __syncthreads();
+      const int gi = sh->group;
+      if (gi >= count || sh->abort) break;
+      const Group grp = A.groups[gi];
+      S = grp.S;
+      nseg = grp.nseg;
+      members = grp.count;
+      item = grp.first + warp;
+      seg = grp.seg;
+      if (kPairs && A.large_possible)
+        large = __any_sync(kFull, A.items[grp.first + min(lane, members - 1)].qmax > A.half_max);
     }
-    const int S = grp.S;
+    // A group with a code too large for the half-code cell belongs to the
+    // large-code sweep, every other one to this form's.
+    const bool mine = !kPairs || large == (PREC == kPrecI16Large);
     const int TS = tile_width(S, A.tile_cols);
     long t_start, t_own, t_end;
-    seg_bounds(S, grp.nseg, grp.seg, A.N, &t_start, &t_own, &t_end);
+    seg_bounds(S, nseg, seg, A.N, &t_start, &t_own, &t_end);
+    const long p_lo = t_start + cut_steps(S, t_start, t_end, cut_lo, cost);
+    const long p_hi = t_start + cut_steps(S, t_start, t_end, cut_hi, cost);
+    // (after a wait that gave up, this CTA's streams are not used again)
+    const bool runs = mine && warp < members && p_lo < p_hi && !__any_sync(kFull, *static_cast<volatile int *>(&sh->abort));
     TileStream ts;
-    ts.sh = sh;
+    ts.sh = &sh->streams[stream];
+    ts.abort = &sh->abort;
     ts.slots = slots;
     ts.src = reinterpret_cast<const char *>(PREC == kPrecI16Large ? A.ref_large : A.ref_img);
     ts.tile_cols = TS;
-    ts.k_first = static_cast<int>(t_start / TS);
-    ts.K = static_cast<int>((t_end + TS - 1) / TS - t_start / TS);
-    ts.n_active = grp.count;
+    ts.k_first = static_cast<int>(p_lo / TS);
+    ts.K = static_cast<int>((p_hi + TS - 1) / TS - p_lo / TS);
+    ts.n_active = solo ? 1 : members;
     ts.wait_ns = A.wait_ns;
-    ts.status = A.ints + kIntStatus;
-    if (threadIdx.x == 0) {
+    ts.ints = A.ints;
+    const bool streams = lane == 0 && runs && (solo || warp == 0);  // this thread runs a tile stream
+    if (waits && mine) {
+      // the CTA placed before this one ran its part of the bundle first (a step takes well under 1 us)
+      if (threadIdx.x == 0)
+        sh->stop = !wait_part(A, place - 1, A.wait_ns + 1000ull * static_cast<unsigned long long>(t_end - t_start));
+      __syncthreads();
+      if (sh->stop) break;
+    }
+    if (streams) {
       ts.issue(0);
       if (ts.K > 1) ts.issue(1);
     }
-    __syncthreads();
-    if (warp < grp.count) dispatch_sweep<PREC>(S, A, ts, grp, grp.first + warp, rings + warp * kRing, lane);
-    __syncthreads();
-    if (threadIdx.x == 0) sh->tile_base += ts.K;
+    if (solo)
+      __syncwarp();
+    else
+      __syncthreads();
+    if (runs) dispatch_sweep<PREC>(S, A, ts, nseg, seg, p_lo, p_hi, item, rings + warp * kRing, lane);
+    if (solo)
+      __syncwarp();
+    else
+      __syncthreads();
+    if (streams) ts.sh->tile_base += ts.K;
+    if (hands && mine) {
+      __syncthreads();
+      if (threadIdx.x == 0 && !sh->abort) finish_part(A, place);
+    }
   }
   // On abort, wait (bounded) for this CTA's copies still in flight before exit.
   __syncthreads();
-  if (threadIdx.x == 0 && sh->abort) {
+  if (threadIdx.x < kMaxWarps && sh->abort) {
+    Stream *t = &sh->streams[threadIdx.x];
     const unsigned long long dl = now_ns() + A.wait_ns;
     for (int s = 0; s < 2; ++s)
-      if (sh->uses[s] > 0) mbar_wait_bounded(&sh->full[s], (sh->uses[s] - 1) & 1, dl);
+      if (t->uses[s] > 0) mbar_wait_bounded(&t->full[s], (t->uses[s] - 1) & 1, dl);
   }
 }
 
@@ -1156,10 +1324,15 @@ __global__ void __launch_bounds__(kFixWarps * 32) fixup_kernel(SdtwArgs A) {
 }
 
 template <int PREC>
+SmemOptIn &smem_record() {
+  static SmemOptIn rec;
+  return rec;
+}
+
+template <int PREC>
 cudaError_t launch_sweep_prec(const SdtwArgs &a, int grid, cudaStream_t s) {
-  static SmemOptIn opt;
-  const size_t sm = sdtw_smem_bytes(PREC, a.tile_cols, a.warps);
-  cudaError_t e = opt_in_smem(sdtw_kernel<PREC>, opt, sm);
+  const size_t sm = sdtw_smem_bytes(PREC, a.tile_cols, a.warps, a.solo);
+  cudaError_t e = opt_in_smem(sdtw_kernel<PREC>, smem_record<PREC>(), sm);
   if (e != cudaSuccess) return e;
   sdtw_kernel<PREC><<<grid, a.warps * 32, sm, s>>>(a);
   return cudaGetLastError();
@@ -1176,10 +1349,11 @@ cudaError_t launch_fixup_prec(const SdtwArgs &a, int fix_items, cudaStream_t s) 
 }
 
 template <int PREC>
-int occupancy_prec(int tile_cols, int warps) {
+int occupancy_prec(int tile_cols, int warps, int solo) {
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sdtw_kernel<PREC>, warps * 32,
-                                                sdtw_smem_bytes(PREC, tile_cols, warps));
+  const size_t sm = sdtw_smem_bytes(PREC, tile_cols, warps, solo);
+  if (opt_in_smem(sdtw_kernel<PREC>, smem_record<PREC>(), sm) != cudaSuccess) return 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sdtw_kernel<PREC>, warps * 32, sm);
   return n;
 }
 
@@ -1195,7 +1369,7 @@ int occupancy_prec(int tile_cols, int warps) {
   cudaError_t sdtw_sweep_##P(const SdtwArgs &a, int grid, cudaStream_t s) {                   \
     return launch_sweep_prec<P>(a, grid, s);                                                   \
   }                                                                                            \
-  int sdtw_occupancy_##P(int tile_cols, int warps) { return occupancy_prec<P>(tile_cols, warps); } \
+  int sdtw_occupancy_##P(int tile_cols, int warps, int solo) { return occupancy_prec<P>(tile_cols, warps, solo); } \
   cudaError_t sdtw_sweep_load_##P() {                                                          \
     cudaFuncAttributes f;                                                                      \
     return cudaFuncGetAttributes(&f, sdtw_kernel<P>);                                          \

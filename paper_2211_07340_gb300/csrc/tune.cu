@@ -3,7 +3,8 @@
 //
 // Tuned: warps per CTA (queries or pairs sharing one reference tile stream),
 // reference tile width and the work-unit target (how finely sweeps are cut
-// into verified reference segments; 1 = never cut), then at the best of
+// into verified reference segments; 0 = the planner's cost model, 1 = never
+// cut), then at the best of
 // those the strip geometry of queries of <= 256 events (32-lane strips or
 // stacked 16-lane strips with twice the rows per lane). Beyond that the
 // strip height is not a free choice: S = floor(M / 32) + 1 rows per
@@ -68,7 +69,7 @@ extern "C" int haru_autotune(haru_ctx *ctx, int precision, const float *events, 
   const int auto_units = 4 * ctx->sms * 8;
   const int warps_c[] = {4, 8, 12};
   const int tiles_c[] = {2048, 4096, 8192, 16384};
-  const int units_c[] = {1, auto_units / 2, auto_units, 2 * auto_units};
+  const int units_c[] = {1, auto_units, 2 * auto_units};
   float best_ms = -1.0f;
   LaunchCfg best = base;
   // One trial: the minimum of two timed runs after one warm-up; kept if fastest.
@@ -94,7 +95,12 @@ extern "C" int haru_autotune(haru_ctx *ctx, int precision, const float *events, 
       best = lc;
     }
   };
-  // Launch shape first, at the context's stacking rule ...
+  // The planner's own schedule, and explicit launch shapes, at the context's
+  // stacking rule ...
+  LaunchCfg own = base;
+  own.units_target = 0;
+  own.ctas_per_sm = 0;
+  trial(own);
   for (int w : warps_c)
     for (int t : tiles_c)
       for (int u : units_c) {
