@@ -18,7 +18,7 @@ cudaError_t record_event(cudaEvent_t e, cudaStream_t s) {
 }
 
 void ws_free(Workspace &ws) {
-  void *p[] = {ws.ints, ws.items, ws.arrived, ws.groups, ws.sched, ws.done, ws.img, ws.states, ws.bests, ws.qstats};
+  void *p[] = {ws.ints, ws.items, ws.arrived, ws.groups, ws.sched, ws.done, ws.img, ws.states, ws.bests, ws.qstats, ws.checkpoints};
   for (void *q : p)
     if (q) cudaFree(q);
   ws = Workspace();
@@ -36,10 +36,10 @@ constexpr int kSoloTile = 1536;
 struct StepClocks {
   float full[kMaxS], stacked, two, one;
 };
-const StepClocks kStepI16 = {{21.3f, 21.5f, 25.7f, 28.7f, 34.4f, 39.7f, 44.6f, 47.5f, 53.4f, 59.5f, 64.1f, 67.1f,
-                              74.4f, 76.5f, 81.2f, 84.7f}, 2.0f, 6.0f, 23.0f};
-const StepClocks kStepF32 = {{19.0f, 18.0f, 21.2f, 23.8f, 28.9f, 32.4f, 37.5f, 41.9f, 47.2f, 51.5f, 56.1f, 59.0f,
-                              63.7f, 68.2f, 71.4f, 75.5f}, 1.4f, 4.0f, 13.0f};
+const StepClocks kStepI16 = {{22.3f, 22.1f, 25.6f, 28.5f, 34.7f, 39.6f, 45.4f, 47.7f, 58.1f, 58.6f, 65.1f, 69.4f,
+                              77.1f, 76.3f, 81.5f, 86.6f}, 2.0f, 5.0f, 23.0f};
+const StepClocks kStepF32 = {{19.9f, 18.4f, 21.0f, 24.4f, 29.4f, 34.3f, 38.5f, 42.7f, 47.7f, 53.0f, 57.8f, 59.8f,
+                              63.8f, 68.9f, 71.9f, 76.8f}, 1.4f, 4.0f, 13.5f};
 const StepClocks &step_clocks(int precision) {
   return precision == HARU_INT16 ? kStepI16 : kStepF32;
 }
@@ -52,12 +52,36 @@ long stack_units(int precision, const LaunchCfg &lc) {
 
 // Buffer sizes one batch of nq queries needs.
 struct WsNeeds {
-  size_t max_items, units, groups, ctas, qstats, states;
+  size_t max_items, units, groups, ctas, qstats, states, checkpoints;
   int nseg_cap;
 };
 
+// Start-column batches on references of at least kTraceColumns run the cost
+// form and trace the starts back from checkpoints; on shorter ones, of few
+// query lengths, the starts are carried along. At 2,000
+// columns tracing took 163 us for one query, 479 for 100 and 2,090 for 8,000
+// uneven ones, carrying 227, 615 and 1,920; at 1,000 columns 161, 494 and
+// 1,754 against 165, 409 and 1,229.
+constexpr long kTraceColumns = 2048;
+bool traced(int precision, const LaunchCfg &lc) { return prec_span(precision) && lc.N >= kTraceColumns; }
+int cost_form(int precision) {
+  return precision == kPrecF32Span ? HARU_FP32 : (precision == kPrecWideSpan ? HARU_INT16_ACC32 : precision);
+}
+
+// Checkpoints per item: up to 128 (a trace runs half the distance between two
+// of them on average beside two strip heights), fewer in batches whose
+// states would pass 512 MB, at least 8; at least 256 steps apart.
+int checkpoint_cap(size_t max_items, long N) {
+  const size_t fit = (static_cast<size_t>(512) << 20) / (max_items * kStateStride * sizeof(uint32_t));
+  const long most = std::min<long>(std::min<size_t>(std::max<size_t>(fit, 8), 128), (N + 32 * kMaxS) / 256);
+  return static_cast<int>(std::max<long>(most, 1));
+}
+int checkpoint_step(int cap, long N) { return static_cast<int>((N + 32 * kMaxS + cap) / cap); }
+
 WsNeeds ws_needs(int precision, uint32_t nq, const LaunchCfg &lc) {
   WsNeeds w;
+  const bool trace = traced(precision, lc);
+  if (trace) precision = cost_form(precision);
   const BatchShape sh = batch_shape(precision, nq, lc);
   const int mode = plan_mode(precision);
   w.max_items = items_bound(mode, nq);
@@ -79,6 +103,7 @@ WsNeeds ws_needs(int precision, uint32_t nq, const LaunchCfg &lc) {
   w.groups = sh.solo ? 1 : (w.max_items + kMaxS) * static_cast<size_t>(w.nseg_cap);
   w.qstats = 2 * static_cast<size_t>(nq);
   w.states = w.units * 2 * state_words(precision);
+  w.checkpoints = trace ? w.max_items * static_cast<size_t>(checkpoint_cap(w.max_items, lc.N)) * kStateStride : 0;
   return w;
 }
 
@@ -106,6 +131,7 @@ cudaError_t ws_alloc(Workspace &ws, const WsNeeds &w) {
   if ((e = grow(&ws.done, &ws.cap_done, w.ctas)) != cudaSuccess) return e;
   if ((e = grow(&ws.bests, &ws.cap_bests, 2 * w.units)) != cudaSuccess) return e;
   if ((e = grow(&ws.qstats, &ws.cap_qstats, w.qstats)) != cudaSuccess) return e;
+  if (w.checkpoints && (e = grow(&ws.checkpoints, &ws.cap_checkpoints, w.checkpoints)) != cudaSuccess) return e;
   return grow(&ws.states, &ws.cap_states, w.states);
 }
 
@@ -135,7 +161,7 @@ BatchShape batch_shape(int precision, uint32_t nq, const LaunchCfg &lc) {
   sh.tile = lc.tile;
   sh.solo = false;
   sh.per_sm = lc.ctas_per_sm > 0 ? lc.ctas_per_sm : 0;
-  if (sh.per_sm == 0) sh.per_sm = sdtw_max_ctas_per_sm(precision, sh.tile, sh.warps, 0);
+  if (sh.per_sm == 0) sh.per_sm = sdtw_max_ctas_per_sm(precision, sh.tile, sh.warps);
   if (lc.units_target == 0 && lc.ctas_per_sm == 0 && !prec_span(precision)) {
     sh.solo = true;
     sh.warps = kMaxWarps;
@@ -174,6 +200,9 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
                        const LaunchCfg &lc, cudaStream_t s, cudaEvent_t ev_prep, cudaEvent_t ev_sweep,
                        int64_t *d_start, bool zero_counters, cudaEvent_t ev_fix) {
   cudaError_t e;
+  const int asked = precision;
+  const bool trace = traced(precision, lc);
+  if (trace) precision = cost_form(precision);
   // (a caller that ran kernels reporting into the status word first has zeroed the counters itself)
   if (zero_counters && (e = cudaMemsetAsync(ws.ints, 0, kIntWords * sizeof(int), s)) != cudaSuccess) return e;
   if (ev_prep && (e = record_event(ev_prep, s)) != cudaSuccess) return e;
@@ -236,6 +265,9 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
   sa.done = ws.done;
   sa.arrived = ws.arrived;
   sa.out_start = d_start;
+  sa.checkpoints = trace ? ws.checkpoints : nullptr;
+  sa.checkpoint_cap = trace ? checkpoint_cap(ws.max_items, ref.N) : 0;
+  sa.checkpoint_step = trace ? checkpoint_step(sa.checkpoint_cap, ref.N) : 0;
   sa.nseg_cap = ws.nseg_cap;
   sa.out_cost = d_cost;
   sa.out_col = d_col;
@@ -250,7 +282,8 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
   // query's result.
   const size_t groups_max = ((ws.max_items + sh.warps - 1) / sh.warps + kMaxS) * static_cast<size_t>(ws.nseg_cap);
   const int grid = sh.solo ? slots : static_cast<int>(std::min<size_t>(slots, groups_max));
-  return launch_sdtw(precision, sa, grid, static_cast<int>(ws.max_items), s, ev_fix);
+  if ((e = launch_sdtw(precision, sa, grid, static_cast<int>(ws.max_items), s, ev_fix)) != cudaSuccess || !trace) return e;
+  return launch_trace(asked, sa, static_cast<int>(ws.max_items), sh.stack, s);
 }
 
 }  // namespace haru

@@ -111,6 +111,8 @@ struct Workspace {
   size_t cap_states = 0;
   Best *bests = nullptr;  // 2 x units: upper stacks, then lower stacks
   size_t cap_bests = 0;
+  uint32_t *checkpoints = nullptr;  // traced batches: states along each item's sweep
+  size_t cap_checkpoints = 0;
   double *qstats = nullptr;  // per query (mean, sigma) of raw batches
   size_t cap_qstats = 0;
   // plan of the last reservation

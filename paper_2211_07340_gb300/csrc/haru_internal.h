@@ -207,6 +207,12 @@ __host__ __device__ inline void seg_bounds(int S, int nseg, int seg, long N, lon
   *t_start = seg == 0 ? 0 : (w > 0 ? w : 0);
 }
 
+// Steps between two checkpoints of strip height S: `step` rounded up to whole chunks.
+__host__ __device__ inline int checkpoint_steps(int S, int step) {
+  const int U = steps_per_chunk(S);
+  return (step + U - 1) / U * U;
+}
+
 // Steps from t_start to where a bundle cut at `at` of `cost` on the schedule's
 // line stops (whole chunks; the same operands give the same cut on both sides).
 __host__ __device__ inline long cut_steps(int S, long t_start, long t_end, long long at, long long cost) {
@@ -235,6 +241,9 @@ struct SdtwArgs {
                            // the planner)
   int *arrived;            // [item]: CTAs of the fix-up kernel that verified their segments (zeroed by the planner)
   int64_t *out_start;      // span forms: the alignment start column per query
+  uint32_t *checkpoints;   // [item][checkpoint_cap] states, kStateStride words each, before steps checkpoint_steps(S) *
+                           // 1, 2, ...; nullptr: none (a traced batch's cost sweep saves them)
+  int checkpoint_cap, checkpoint_step;
   int nseg_cap;
   float *out_cost;
   int64_t *out_col;
@@ -288,6 +297,9 @@ cudaError_t launch_qstats(const float *events, const uint32_t *offsets, uint32_t
                           cudaStream_t s);
 cudaError_t launch_sdtw(int precision, const SdtwArgs &a, int grid, int fix_items, cudaStream_t s,
                         cudaEvent_t ev_fix = nullptr);
+// Start columns from the checkpoints of a cost sweep whose results are in
+// out_cost / out_col (span precisions).
+cudaError_t launch_trace(int precision, const SdtwArgs &a, int max_items, bool stacked, cudaStream_t s);
 // cudaEventRecord that also works inside a stream capture (batch.cu).
 cudaError_t record_event(cudaEvent_t e, cudaStream_t s);
 // Load kernels into the current context now instead of at their first
@@ -295,8 +307,8 @@ cudaError_t record_event(cudaEvent_t e, cudaStream_t s);
 // and the sweep and fix-up kernels of a precision.
 cudaError_t load_prep_kernels();
 cudaError_t load_sdtw(int precision);
-size_t sdtw_smem_bytes(int precision, int tile_cols, int warps, int solo);
-int sdtw_max_ctas_per_sm(int precision, int tile_cols, int warps, int solo);
+size_t sdtw_smem_bytes(int precision, int tile_cols, int warps, bool solo);
+int sdtw_max_ctas_per_sm(int precision, int tile_cols, int warps);
 
 // Reference preparation.
 cudaError_t launch_ref_levels(const uint8_t *bases, size_t n, const float *model, int k, float *out,

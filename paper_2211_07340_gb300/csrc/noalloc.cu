@@ -152,6 +152,8 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   sa.done = nullptr;
   sa.arrived = nullptr;
   sa.nseg_cap = 1;
+  sa.checkpoints = nullptr;
+  sa.checkpoint_cap = sa.checkpoint_step = 0;
   sa.out_cost = out_cost;
   sa.out_col = out_col;
   sa.inv_scale = 1.0f / static_cast<float>(1 << ref.scale_log2);
@@ -160,7 +162,7 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   sa.solo = 0;
   sa.wait_ns = wait;
   const size_t groups_max = (max_items + warps - 1) / warps + kMaxS;
-  const int cps = per_sm > 0 ? per_sm : sdtw_max_ctas_per_sm(precision, tile, warps, 0);
+  const int cps = per_sm > 0 ? per_sm : sdtw_max_ctas_per_sm(precision, tile, warps);
   size_t grid = static_cast<size_t>(sms) * (cps > 0 ? cps : 1);
   if (grid > groups_max) grid = groups_max;
   if ((e = launch_sdtw(precision, sa, static_cast<int>(grid), static_cast<int>(max_items), s)) != cudaSuccess)

@@ -1,0 +1,4 @@
+// FP32: the queue's sweep kernel, every strip height (1..16).
+#include "sdtw_kernels.cuh"
+
+HARU_SDTW_QUEUE_INSTANCE(0)

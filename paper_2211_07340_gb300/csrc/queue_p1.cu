@@ -1,0 +1,4 @@
+// int16 (packed DPX pairs): the queue's sweep kernel, every strip height (1..16).
+#include "sdtw_kernels.cuh"
+
+HARU_SDTW_QUEUE_INSTANCE(1)

@@ -1,7 +1,7 @@
-// FP32 with start columns: the sweep kernel, every strip height (1..16).
+// FP32 with start columns: the queue's sweep kernel, every strip height (1..16).
 #include "sdtw_kernels.cuh"
 
-HARU_SDTW_SWEEP_INSTANCE(3)
+HARU_SDTW_QUEUE_INSTANCE(3)
 
 // The saved-state size the batch engine allocates per work unit (state_words)
 // is the one the kernels index, for every form.

@@ -494,6 +494,7 @@ struct TrackF32 {
 // first lane of a stack (the row above row i processed column t - i at
 // step t - 1); the first real row therefore starts its paths at its own
 // column, like the free-start row of Eq. 1. CODES as for StripF32.
+constexpr int kUnknownStart = -2147483647 - 1;
 template <int S, bool CODES>
 struct StripF32Span {
   float Q[S], W[S], G[2][S], Rr[Geo<S>::U];
@@ -549,6 +550,22 @@ struct StripF32Span {
     const int pg = __shfl_up_sync(kFull, P[0][S - 1], 1);
     gprev = ng ? g : 0.0f;
     pprev = ng ? pg : static_cast<int>(t) - 1 - lane * S;
+  }
+  // A cost form's exact state before step t: every start column before it is
+  // kUnknownStart; the free-start rows pass known ones down from step t on.
+  __device__ __forceinline__ void restore_costs(const uint32_t *st, const uint32_t *gref, long t, int lane,
+                                                uint32_t ng) {
+#pragma unroll
+    for (int k = 0; k < S; ++k) {
+      G[1][k] = __uint_as_float(__ldcg(st + k * 32 + lane));
+      G[0][k] = __uint_as_float(__ldcg(st + (S + k) * 32 + lane));
+      P[1][k] = kUnknownStart;
+      P[0][k] = kUnknownStart;
+      Rr[(1 + k) % Geo<S>::U] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
+    }
+    const float g = __shfl_up_sync(kFull, G[0][S - 1], 1);
+    gprev = ng ? g : 0.0f;
+    pprev = kUnknownStart;
   }
   __device__ __forceinline__ void save(uint32_t *st, int lane) const {
 #pragma unroll
@@ -762,8 +779,7 @@ struct GlobalTiles {
 
 // ------------------------------------------------------------ one unit --
 // Runs steps [t_start, t_end) of one strip (a query or a pair) and tracks
-// the last row over own steps [t_own, t_end). fresh: the strip starts from
-// the fresh state at t_start.
+// the last row over own steps [t_own, t_end).
 // save_start / save_final: where to store the state before step t_own and
 // before step t_end (nullptr: not stored). stk: a stacked item (lanes 0..15
 // and 16..31 are two strips; each lane tracks its own stack's last row).
@@ -773,10 +789,14 @@ struct GlobalTiles {
 // carry start columns keep them 2W further on. Each flush scans W/32
 // entries per lane.
 // Returns false on abort.
-template <int FORM, int S, class Src>
-__device__ bool run_steps(typename FormOf<FORM, S>::Strip &st, typename FormOf<FORM, S>::Track &tr, Src &src,
-                          int TS, long t_start, long t_own, long t_end, bool fresh, long N, uint32_t *save_start,
-                          uint32_t *save_final, uint32_t *ring, int lane, bool stk) {
+// With checkpoints (A.checkpoints, cost forms) the state before every
+// checkpoint step of the own range is stored too.
+template <int FORM, int S, class Src, class Track>
+__device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>::Strip &st, Track &tr, Src &src,
+                          int TS, long t_start, long t_own, long t_end, uint32_t *save_start, uint32_t *save_final,
+                          uint32_t *ring, int lane, bool stk) {
+  constexpr bool kCheckpoints = FORM == kFormF32 || FORM == kFormExactWide;
+  const long N = A.N;
   constexpr int U = Geo<S>::U;
   constexpr int W = flush_words(form_i16(FORM) ? HARU_INT16 : HARU_FP32);
   // chunks between two flushes: a stack's entries fill its share of a buffer
@@ -808,8 +828,33 @@ __device__ bool run_steps(typename FormOf<FORM, S>::Strip &st, typename FormOf<F
     // lo + o - lane * S, found at (column - tk0 + kRefFront) in the slot;
     // lane * S <= 31 * kMaxS <= kRefFront keeps it inside the slot
     const uint32_t *tref = tile + (kRefFront + (lo - tk0) - static_cast<long>(lane) * S);
+    // the next step of this tile before which a state is stored
+    auto next_save = [&](int from) {
+      int at = own_at >= from ? own_at : n;
+      if constexpr (kCheckpoints) {
+        if (A.checkpoints) {
+          const long D = checkpoint_steps(S, A.checkpoint_step);
+          const long first = lo + from > t_own ? lo + from : t_own;
+          const long c = (first + D - 1) / D * D - lo;
+          if (c < at) at = static_cast<int>(c);
+        }
+      }
+      return at;
+    };
+    int save_at = next_save(0);
     for (int o = 0; o < n; o += U) {
-      if (o == own_at) st.save(save_start, lane);
+      if (o == save_at) {
+        if (o == own_at) st.save(save_start, lane);
+        if constexpr (kCheckpoints) {
+          if (A.checkpoints) {
+            const int D = checkpoint_steps(S, A.checkpoint_step);
+            const long c = (lo + o) / D;  // (checkpoint 0 is the fresh start)
+            if (c * D == lo + o && lo + o >= t_own && c > 0 && c <= A.checkpoint_cap)
+              st.save(A.checkpoints + (static_cast<size_t>(item) * A.checkpoint_cap + (c - 1)) * kStateStride, lane);
+          }
+        }
+        save_at = next_save(o + U);
+      }
       uint32_t *rg = ring + buf * W + soff;
       const int tabs = static_cast<int>(lo) + o;
       st.chunk(tref + o, lane, rg, fl * U, ng, tracked, tabs, top);
@@ -863,7 +908,9 @@ __device__ void sweep_unit(const SdtwArgs &A, TileStream &ts, int nseg, int seg,
   st.load(A.img + static_cast<size_t>(item) * kImgStride, lane);
   long t_start, t_own, t_end;
   seg_bounds(S, nseg, seg, A.N, &t_start, &t_own, &t_end);
-  const bool stk = A.items[item].stacked != 0, whole = p_lo == t_start;
+  const bool stk = A.items[item].stacked != 0;
+  // (start-column units are never cut)
+  const bool whole = FORM == kFormF32Span || FORM == kFormWideSpan || p_lo == t_start;
   const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
   const size_t unit = static_cast<size_t>(item) * A.nseg_cap + seg;
   constexpr size_t kWords = state_rows_per_s<FORM>() * 16 * 32;
@@ -874,7 +921,7 @@ __device__ void sweep_unit(const SdtwArgs &A, TileStream &ts, int nseg, int seg,
     st.fresh(t_start, lane, ng);
   else
     st.restore(A.states + (unit * 2 + 1) * kWords, reinterpret_cast<const uint32_t *>(ts.src), p_lo, lane, ng);
-  const bool ok = run_steps<FORM, S>(st, tr, ts, ts.tile_cols, p_lo, t_own, p_hi, true, A.N, ss, sf, ring, lane, stk);
+  const bool ok = run_steps<FORM, S>(A, item, st, tr, ts, ts.tile_cols, p_lo, t_own, p_hi, ss, sf, ring, lane, stk);
   tr.reduce(stk ? 16 : 32);
   if (ok && lane == 0) {
     if (!whole) tr.merge(A.bests + unit);
@@ -942,6 +989,103 @@ __device__ __forceinline__ void dispatch_sweep(int s, const SdtwArgs &A, TileStr
   }
 }
 
+// Up to 12 warps per CTA (3 per scheduler): the int16, FP32 and wide strips
+// fit in 168 registers a thread; the start-column strips (~240) up to 8.
+template <int PREC>
+__host__ __device__ constexpr int cta_threads() { return prec_span(PREC) ? 256 : 384; }
+template <int PREC>
+__host__ __device__ constexpr bool pairs() { return PREC == HARU_INT16 || PREC == kPrecI16Large; }
+
+// The CTA's shared state and this warp's tile slots; layout: Shared |
+// per-warp tracking rings | two tile slots per stream.
+__device__ __forceinline__ void init_shared(Shared *sh) {
+  if (threadIdx.x < kMaxWarps) {
+    Stream *t = &sh->streams[threadIdx.x];
+    mbar_init(&t->full[0], 1);
+    mbar_init(&t->full[1], 1);
+    t->cnt[0] = t->cnt[1] = 0;
+    t->uses[0] = t->uses[1] = 0;
+    t->tile_base = 0;
+    if (threadIdx.x == 0) sh->abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+}
+template <int PREC>
+__device__ __forceinline__ TileStream stream_of(const SdtwArgs &A, Shared *sh, int stream, int S, long p_lo, long p_hi,
+                                                int n_active) {
+  char *slots = reinterpret_cast<char *>(sh) + kSharedHeader + A.warps * ring_words(PREC) * 4;
+  const int TS = tile_width(S, A.tile_cols);
+  TileStream ts;
+  ts.sh = &sh->streams[stream];
+  ts.abort = &sh->abort;
+  ts.slots = slots + static_cast<size_t>(stream) * 2 * (A.tile_cols + kRefFront) * 4;
+  ts.src = reinterpret_cast<const char *>(PREC == kPrecI16Large ? A.ref_large : A.ref_img);
+  ts.tile_cols = TS;
+  ts.k_first = static_cast<int>(p_lo / TS);
+  ts.K = static_cast<int>((p_hi + TS - 1) / TS - p_lo / TS);
+  ts.n_active = n_active;
+  ts.wait_ns = A.wait_ns;
+  ts.ints = A.ints;
+  return ts;
+}
+// On abort, wait (bounded) for this CTA's copies still in flight before exit.
+__device__ __forceinline__ void drain_streams(const SdtwArgs &A, Shared *sh) {
+  __syncthreads();
+  if (threadIdx.x < kMaxWarps && sh->abort) {
+    Stream *t = &sh->streams[threadIdx.x];
+    const unsigned long long dl = now_ns() + A.wait_ns;
+    for (int s = 0; s < 2; ++s)
+      if (t->uses[s] > 0) mbar_wait_bounded(&t->full[s], (t->uses[s] - 1) & 1, dl);
+  }
+}
+
+// Groups from the queue: a CTA's warps sweep one segment, sharing one tile
+// stream. (A kernel apart from the scheduled sweep below: in one kernel the
+// start-column strips ran 10-20% longer a step.)
+template <int PREC>
+__global__ void __launch_bounds__(cta_threads<PREC>(), 1) queue_kernel(SdtwArgs A) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  Shared *sh = reinterpret_cast<Shared *>(smem);
+  uint32_t *rings = reinterpret_cast<uint32_t *>(smem + kSharedHeader);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  init_shared(sh);
+  const int count = A.ints[kIntGroups];
+  int *queue = A.ints + (PREC == kPrecI16Large ? kIntQueueLarge : kIntQueue);
+  for (;;) {
+    if (threadIdx.x == 0) sh->group = atomicAdd(queue, 1);
+    __syncthreads();
+    const int gi = sh->group;
+    if (gi >= count || sh->abort) break;
+    const Group grp = A.groups[gi];
+    if constexpr (pairs<PREC>()) {
+      // A group with a code too large for the half-code cell belongs to the
+      // large-code sweep, every other one to this form's.
+      bool large = false;
+      if (A.large_possible)
+        large = __any_sync(kFull, A.items[grp.first + min(lane, grp.count - 1)].qmax > A.half_max);
+      if (large != (PREC == kPrecI16Large)) {
+        __syncthreads();  // every thread has read sh->group
+        continue;
+      }
+    }
+    long t_start, t_own, t_end;
+    seg_bounds(grp.S, grp.nseg, grp.seg, A.N, &t_start, &t_own, &t_end);
+    TileStream ts = stream_of<PREC>(A, sh, 0, grp.S, t_start, t_end, grp.count);
+    if (threadIdx.x == 0) {
+      ts.issue(0);
+      if (ts.K > 1) ts.issue(1);
+    }
+    __syncthreads();
+    if (warp < grp.count)
+      dispatch_sweep<PREC>(grp.S, A, ts, grp.nseg, grp.seg, t_start, t_end, grp.first + warp,
+                           rings + warp * ring_words(PREC), lane);
+    __syncthreads();
+    if (threadIdx.x == 0) ts.sh->tile_base += ts.K;
+  }
+  drain_streams(A, sh);
+}
+
 // The bundle at place x of the schedule's line: the number of bundles that
 // end at or before x; *inside: x lies within that bundle, not at its start.
 __device__ __forceinline__ int bundle_at(const Schedule &c, long long x, bool *inside) {
@@ -966,146 +1110,76 @@ __device__ __forceinline__ const ScheduleRow &find_row(const Schedule &c, int b,
   return c.row[k];
 }
 
-// Up to 12 warps per CTA (3 per scheduler): the int16, FP32 and wide strips
-// fit in 168 registers a thread; the start-column strips (~240) up to 8.
+// The static schedule: this CTA's stretch of it, each warp with its own tile
+// stream.
 template <int PREC>
-__global__ void __launch_bounds__(prec_span(PREC) ? 256 : 384, 1) sdtw_kernel(SdtwArgs A) {
+__global__ void __launch_bounds__(cta_threads<PREC>(), 1) sdtw_kernel(SdtwArgs A) {
   extern __shared__ __align__(128) unsigned char smem[];
   Shared *sh = reinterpret_cast<Shared *>(smem);
-  // layout: Shared | per-warp tracking rings | two tile slots per stream
   uint32_t *rings = reinterpret_cast<uint32_t *>(smem + kSharedHeader);
-  constexpr int kRing = ring_words(PREC);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr bool kPairs = PREC == HARU_INT16 || PREC == kPrecI16Large;
-  const bool solo = A.solo != 0;
-  const int stream = solo ? warp : 0;
-  char *slots = reinterpret_cast<char *>(rings + A.warps * kRing) +
-                static_cast<size_t>(stream) * 2 * (A.tile_cols + kRefFront) * 4;
-  if (threadIdx.x < kMaxWarps) {
-    Stream *t = &sh->streams[threadIdx.x];
-    mbar_init(&t->full[0], 1);
-    mbar_init(&t->full[1], 1);
-    t->cnt[0] = t->cnt[1] = 0;
-    t->uses[0] = t->uses[1] = 0;
-    t->tile_base = 0;
-    if (threadIdx.x == 0) sh->abort = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  int *queue = A.ints + (PREC == kPrecI16Large ? kIntQueueLarge : kIntQueue);
-  // Static schedule: this CTA's place on the line, in the order the CTAs
-  // started, and the bundles first .. first + n - 1 that its stretch touches.
-  int place = 0, first = 0, n = 0;
-  bool left = false, right = false;  // the first / last of them crosses a border
+  // This CTA's place on the line, in the order the CTAs started, and the
+  // bundles first .. first + n - 1 that its stretch touches.
   const Schedule &sched = sh->sched;
-  if (solo) {
-    if (threadIdx.x == 0) sh->group = atomicAdd(queue, 1);
-    for (int i = threadIdx.x; i < static_cast<int>(sizeof(Schedule) / 4); i += blockDim.x)
-      reinterpret_cast<int *>(&sh->sched)[i] = reinterpret_cast<const int *>(A.sched)[i];
-    __syncthreads();
-    place = sh->group;
-    const long long lo = place * sched.share, hi = lo + sched.share;
-    const int begin = bundle_at(sched, lo, &left), end = bundle_at(sched, hi, &right);
-    first = begin;
-    n = end - begin + (right ? 1 : 0);
-  }
-  const int count = A.ints[kIntGroups];
-  for (int e = 0;; ++e) {
-    // The next work: S, nseg, `members` warps at work, this warp's item and
-    // segment, and the part [cut_lo, cut_hi) of `cost` of its steps.
-    int S, nseg, members, item, seg;
-    long long cut_lo = 0, cut_hi = 1, cost = 1;
-    bool large = false, waits = false, hands = false;
-    if (solo) {
-      if (e >= n) break;
-      // the bundle across the right border first, the one across the left border last
-      const int b = first + (right ? (e == 0 ? n - 1 : e - 1 + (left ? 1 : 0)) : e + (left ? 1 : 0));
-      const int at = b >= first + n - (right && e > 0 ? 1 : 0) ? first : b;
-      const ScheduleRow &row = find_row(sched, at, &S);
-      const int i = at - row.bundle0;
-      const long long start = row.start + i * row.cost;
-      cost = i + 1 < row.bundles ? row.cost : row.last_cost;
-      cut_lo = place * sched.share - start;
-      cut_hi = cut_lo + sched.share;
-      waits = left && at == first;
-      hands = right && at == first + n - 1;
-      nseg = row.nseg;
-      members = i + 1 < row.bundles ? sched.members : row.last;
-      const int u0 = i * sched.members, u = u0 + min(warp, members - 1);
-      item = row.base + u % row.items;
-      seg = u / row.items;
-      if (kPairs && A.large_possible)
+  if (threadIdx.x == 0) sh->group = atomicAdd(A.ints + (PREC == kPrecI16Large ? kIntQueueLarge : kIntQueue), 1);
+  for (int i = threadIdx.x; i < static_cast<int>(sizeof(Schedule) / 4); i += blockDim.x)
+    reinterpret_cast<int *>(&sh->sched)[i] = reinterpret_cast<const int *>(A.sched)[i];
+  init_shared(sh);
+  const int place = sh->group;
+  bool left, right;  // the first / last of them crosses a border
+  const int first = bundle_at(sched, place * sched.share, &left);
+  const int n = bundle_at(sched, (place + 1) * sched.share, &right) - first + (right ? 1 : 0);
+  for (int e = 0; e < n; ++e) {
+    // the bundle across the right border first, the one across the left border last
+    const int next = first + (right ? (e == 0 ? n - 1 : e - 1 + (left ? 1 : 0)) : e + (left ? 1 : 0));
+    const int b = next >= first + n - (right && e > 0 ? 1 : 0) ? first : next;
+    int S;
+    const ScheduleRow &row = find_row(sched, b, &S);
+    const int i = b - row.bundle0;
+    const long long cost = i + 1 < row.bundles ? row.cost : row.last_cost;
+    const long long cut_lo = place * sched.share - (row.start + i * row.cost), cut_hi = cut_lo + sched.share;
+    const bool waits = left && b == first, hands = right && b == first + n - 1;
+    const int members = i + 1 < row.bundles ? sched.members : row.last;
+    const int u0 = i * sched.members, u = u0 + min(warp, members - 1);  // this warp's unit
+    const int item = row.base + u % row.items, seg = u / row.items, nseg = row.nseg;
+    if constexpr (pairs<PREC>()) {
+      // A bundle with a code too large for the half-code cell belongs to the
+      // large-code sweep, every other one to this form's.
+      bool large = false;
+      if (A.large_possible)
         large = __any_sync(kFull, A.items[row.base + (u0 + min(lane, members - 1)) % row.items].qmax > A.half_max);
-    } else {
-      if (threadIdx.x == 0) sh->group = atomicAdd(queue, 1);
-      __syncthreads();
-      const int gi = sh->group;
-      if (gi >= count || sh->abort) break;
-      const Group grp = A.groups[gi];
-      S = grp.S;
-      nseg = grp.nseg;
-      members = grp.count;
-      item = grp.first + warp;
-      seg = grp.seg;
-      if (kPairs && A.large_possible)
-        large = __any_sync(kFull, A.items[grp.first + min(lane, members - 1)].qmax > A.half_max);
+      if (large != (PREC == kPrecI16Large)) continue;
     }
-    // A group with a code too large for the half-code cell belongs to the
-    // large-code sweep, every other one to this form's.
-    const bool mine = !kPairs || large == (PREC == kPrecI16Large);
-    const int TS = tile_width(S, A.tile_cols);
     long t_start, t_own, t_end;
     seg_bounds(S, nseg, seg, A.N, &t_start, &t_own, &t_end);
     const long p_lo = t_start + cut_steps(S, t_start, t_end, cut_lo, cost);
     const long p_hi = t_start + cut_steps(S, t_start, t_end, cut_hi, cost);
-    // (after a wait that gave up, this CTA's streams are not used again)
-    const bool runs = mine && warp < members && p_lo < p_hi && !__any_sync(kFull, *static_cast<volatile int *>(&sh->abort));
-    TileStream ts;
-    ts.sh = &sh->streams[stream];
-    ts.abort = &sh->abort;
-    ts.slots = slots;
-    ts.src = reinterpret_cast<const char *>(PREC == kPrecI16Large ? A.ref_large : A.ref_img);
-    ts.tile_cols = TS;
-    ts.k_first = static_cast<int>(p_lo / TS);
-    ts.K = static_cast<int>((p_hi + TS - 1) / TS - p_lo / TS);
-    ts.n_active = solo ? 1 : members;
-    ts.wait_ns = A.wait_ns;
-    ts.ints = A.ints;
-    const bool streams = lane == 0 && runs && (solo || warp == 0);  // this thread runs a tile stream
-    if (waits && mine) {
+    if (waits) {
       // the CTA placed before this one ran its part of the bundle first (a step takes well under 1 us)
       if (threadIdx.x == 0)
         sh->stop = !wait_part(A, place - 1, A.wait_ns + 1000ull * static_cast<unsigned long long>(t_end - t_start));
       __syncthreads();
       if (sh->stop) break;
     }
-    if (streams) {
-      ts.issue(0);
-      if (ts.K > 1) ts.issue(1);
+    // (after a wait that gave up, this CTA's streams are not used again)
+    const bool runs = warp < members && p_lo < p_hi && !__any_sync(kFull, *static_cast<volatile int *>(&sh->abort));
+    if (runs) {
+      TileStream ts = stream_of<PREC>(A, sh, warp, S, p_lo, p_hi, 1);
+      if (lane == 0) {
+        ts.issue(0);
+        if (ts.K > 1) ts.issue(1);
+      }
+      __syncwarp();
+      dispatch_sweep<PREC>(S, A, ts, nseg, seg, p_lo, p_hi, item, rings + warp * ring_words(PREC), lane);
+      __syncwarp();
+      if (lane == 0) ts.sh->tile_base += ts.K;
     }
-    if (solo)
-      __syncwarp();
-    else
-      __syncthreads();
-    if (runs) dispatch_sweep<PREC>(S, A, ts, nseg, seg, p_lo, p_hi, item, rings + warp * kRing, lane);
-    if (solo)
-      __syncwarp();
-    else
-      __syncthreads();
-    if (streams) ts.sh->tile_base += ts.K;
-    if (hands && mine) {
+    if (hands) {
       __syncthreads();
       if (threadIdx.x == 0 && !sh->abort) finish_part(A, place);
     }
   }
-  // On abort, wait (bounded) for this CTA's copies still in flight before exit.
-  __syncthreads();
-  if (threadIdx.x < kMaxWarps && sh->abort) {
-    Stream *t = &sh->streams[threadIdx.x];
-    const unsigned long long dl = now_ns() + A.wait_ns;
-    for (int s = 0; s < 2; ++s)
-      if (t->uses[s] > 0) mbar_wait_bounded(&t->full[s], (t->uses[s] - 1) & 1, dl);
-  }
+  drain_streams(A, sh);
 }
 
 // --------------------------------------------------------------- fix-up --
@@ -1182,7 +1256,7 @@ __device__ void recompute_segments(const SdtwArgs &A, int item, uint32_t *ring, 
     typename FormOf<FORM, S>::Track tr;
     GlobalTiles src{ref, TS, t_own / TS};
     uint32_t *sf = s + 1 < nseg ? A.states + ((base + s) * 2 + 1) * kWords : nullptr;
-    run_steps<FORM, S>(st, tr, src, TS, t_own, t_own, t_end, false, A.N, nullptr, sf, ring, lane, stk);
+    run_steps<FORM, S>(A, item, st, tr, src, TS, t_own, t_own, t_end, nullptr, sf, ring, lane, stk);
     tr.reduce(stk ? 16 : 32);
     if (lane == 0) {
       tr.store(A.bests + base + s);
@@ -1323,18 +1397,116 @@ __global__ void __launch_bounds__(kFixWarps * 32) fixup_kernel(SdtwArgs A) {
   }
 }
 
+// ---------------------------------------------------------------- trace --
+// Start columns without carrying them through the whole reference: the cost
+// sweep gives each query's cost and end column and leaves exact states
+// behind (checkpoints); from the nearest one at least two strip heights
+// before the end, the start-column strip runs on to the end column alone.
+// Every cost there is exact, so every cell picks the predecessor the full
+// sweep would; starts before the checkpoint are kUnknownStart, and the end
+// cell's is unknown only if its alignment began before the checkpoint: then
+// the strip runs again from an earlier one, at last from the fresh start.
+// (512 uneven FP32 queries on 59,796 columns: the whole call 4.1 ms with the
+// starts carried through the sweep, 1.9 ms this way.)
+struct TrackAt {
+  long want;  // the end column on the lanes of the query's stack, -1 on the others
+  int start = kUnknownStart;
+  __device__ __forceinline__ void add(const uint32_t *rg, int j, long c) {
+    if (c == want) start = static_cast<int>(rg[2 * flush_words(kPrecF32Span) + j]);
+  }
+};
+
+template <int FORM, int S>
+__device__ void trace_query(const SdtwArgs &A, int item, int q, bool lower, uint32_t *ring, int lane) {
+  const bool stk = A.items[item].stacked != 0;
+  const uint32_t *ref = static_cast<const uint32_t *>(A.ref_img);
+  const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
+  const long end = A.out_col[q];
+  int start = -1;
+  if (end >= 0) {
+    constexpr int U = Geo<S>::U;
+    const int TS = tile_width(S, 4096), D = checkpoint_steps(S, A.checkpoint_step);
+    const int rows = stk ? 16 * S : 32 * S;
+    const long t_last = end + (stk && !lower ? 16L : 32L) * S - 1, t_end = (t_last + U) / U * U;
+    const long back = t_last - 2 * rows - 32;
+    typename FormOf<FORM, S>::Strip st;
+    st.load(A.img + static_cast<size_t>(item) * kImgStride, lane);
+    long c = back > 0 ? back / D : 0, less = 1;
+    if (c > A.checkpoint_cap) c = A.checkpoint_cap;
+    for (;;) {
+      const long t0 = c * D;
+      if (c == 0)
+        st.fresh(0, lane, ng);
+      else
+        st.restore_costs(A.checkpoints + (static_cast<size_t>(item) * A.checkpoint_cap + (c - 1)) * kStateStride, ref,
+                         t0, lane, ng);
+      TrackAt tr;
+      tr.want = !stk || (lane >= 16) == lower ? end : -1;
+      GlobalTiles src{ref, TS, t0 / TS};
+      run_steps<FORM, S>(A, item, st, tr, src, TS, t0, t0, t_end, nullptr, nullptr, ring, lane, stk);
+      start = __reduce_max_sync(kFull, tr.start);
+      if (start != kUnknownStart || c == 0) break;
+      c = c > less ? c - less : 0;
+      less *= 2;
+    }
+  }
+  if (lane == 0) A.out_start[q] = start;
+}
+
+template <int FORM, int S = 1>
+__device__ __forceinline__ void dispatch_trace(int s, const SdtwArgs &A, int item, int q, bool lower, uint32_t *ring,
+                                               int lane) {
+  if constexpr (S <= kMaxS) {
+    if (s == S)
+      trace_query<FORM, S>(A, item, q, lower, ring, lane);
+    else
+      dispatch_trace<FORM, S + 1>(s, A, item, q, lower, ring, lane);
+  }
+}
+
+constexpr int kTraceWarps = 4;
+
+// One warp per query (`parts` = 2 in batches with stacked items).
 template <int PREC>
+__global__ void __launch_bounds__(kTraceWarps * 32) trace_kernel(SdtwArgs A, int parts) {
+  __shared__ __align__(16) uint32_t rings[kTraceWarps * ring_words(PREC)];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w = blockIdx.x * kTraceWarps + warp, item = w / parts;
+  const bool lower = w % parts != 0;
+  if (item >= A.ints[kIntItems]) return;
+  const int q = lower ? A.items[item].qc : A.items[item].qa;
+  if (q < 0) return;
+  constexpr int kForm = PREC == kPrecF32Span ? kFormF32Span : kFormWideSpan;
+  dispatch_trace<kForm>(A.items[item].S, A, item, q, lower, rings + warp * ring_words(PREC), lane);
+}
+
+template <int PREC>
+cudaError_t launch_trace_prec(const SdtwArgs &a, int max_items, bool stacked, cudaStream_t s) {
+  const int parts = stacked ? 2 : 1;
+  trace_kernel<PREC><<<(max_items * parts + kTraceWarps - 1) / kTraceWarps, kTraceWarps * 32, 0, s>>>(a, parts);
+  return cudaGetLastError();
+}
+
+template <int PREC, bool SOLO>
 SmemOptIn &smem_record() {
   static SmemOptIn rec;
   return rec;
 }
+template <int PREC, bool SOLO>
+constexpr auto sweep_kernel() {
+  if constexpr (SOLO)
+    return sdtw_kernel<PREC>;
+  else
+    return queue_kernel<PREC>;
+}
 
-template <int PREC>
+template <int PREC, bool SOLO>
 cudaError_t launch_sweep_prec(const SdtwArgs &a, int grid, cudaStream_t s) {
-  const size_t sm = sdtw_smem_bytes(PREC, a.tile_cols, a.warps, a.solo);
-  cudaError_t e = opt_in_smem(sdtw_kernel<PREC>, smem_record<PREC>(), sm);
+  const size_t sm = sdtw_smem_bytes(PREC, a.tile_cols, a.warps, SOLO);
+  const auto kernel = sweep_kernel<PREC, SOLO>();
+  cudaError_t e = opt_in_smem(kernel, smem_record<PREC, SOLO>(), sm);
   if (e != cudaSuccess) return e;
-  sdtw_kernel<PREC><<<grid, a.warps * 32, sm, s>>>(a);
+  kernel<<<grid, a.warps * 32, sm, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -1349,31 +1521,42 @@ cudaError_t launch_fixup_prec(const SdtwArgs &a, int fix_items, cudaStream_t s) 
 }
 
 template <int PREC>
-int occupancy_prec(int tile_cols, int warps, int solo) {
+int occupancy_prec(int tile_cols, int warps) {
   int n = 0;
-  const size_t sm = sdtw_smem_bytes(PREC, tile_cols, warps, solo);
-  if (opt_in_smem(sdtw_kernel<PREC>, smem_record<PREC>(), sm) != cudaSuccess) return 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sdtw_kernel<PREC>, warps * 32, sm);
+  const size_t sm = sdtw_smem_bytes(PREC, tile_cols, warps, false);
+  if (opt_in_smem(queue_kernel<PREC>, smem_record<PREC, false>(), sm) != cudaSuccess) return 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, queue_kernel<PREC>, warps * 32, sm);
   return n;
 }
 
 }  // namespace
 }  // namespace haru
 
-// Define the entry points of the sweep kernel (launch, occupancy) or of the
-// segment fix-up kernel for kernel precision P (0 FP32, 1 INT16, 2 int16
-// inputs with wide accumulation, 3 FP32 with start columns, 4 wide with start
-// columns); one per translation unit, so the kernels compile in parallel.
-#define HARU_SDTW_SWEEP_INSTANCE(P)                                                            \
-  namespace haru {                                                                             \
-  cudaError_t sdtw_sweep_##P(const SdtwArgs &a, int grid, cudaStream_t s) {                   \
-    return launch_sweep_prec<P>(a, grid, s);                                                   \
-  }                                                                                            \
-  int sdtw_occupancy_##P(int tile_cols, int warps, int solo) { return occupancy_prec<P>(tile_cols, warps, solo); } \
-  cudaError_t sdtw_sweep_load_##P() {                                                          \
-    cudaFuncAttributes f;                                                                      \
-    return cudaFuncGetAttributes(&f, sdtw_kernel<P>);                                          \
-  }                                                                                            \
+// Define the entry points of a kernel for kernel precision P (0 FP32, 1
+// INT16, 2 int16 inputs with wide accumulation, 3 FP32 with start columns, 4
+// wide with start columns, 5 INT16 groups with large codes): the scheduled
+// sweep, the queue's sweep, the segment fix-up, the trace. One per
+// translation unit, so the kernels compile in parallel.
+#define HARU_SDTW_SWEEP_INSTANCE(P)                                                                        \
+  namespace haru {                                                                                         \
+  cudaError_t sdtw_sweep_##P(const SdtwArgs &a, int grid, cudaStream_t s) {                               \
+    return launch_sweep_prec<P, true>(a, grid, s);                                                         \
+  }                                                                                                        \
+  cudaError_t sdtw_sweep_load_##P() {                                                                      \
+    cudaFuncAttributes f;                                                                                  \
+    return cudaFuncGetAttributes(&f, sdtw_kernel<P>);                                                      \
+  }                                                                                                        \
+  }
+#define HARU_SDTW_QUEUE_INSTANCE(P)                                                                        \
+  namespace haru {                                                                                         \
+  cudaError_t sdtw_queue_##P(const SdtwArgs &a, int grid, cudaStream_t s) {                               \
+    return launch_sweep_prec<P, false>(a, grid, s);                                                        \
+  }                                                                                                        \
+  int sdtw_occupancy_##P(int tile_cols, int warps) { return occupancy_prec<P>(tile_cols, warps); }         \
+  cudaError_t sdtw_queue_load_##P() {                                                                      \
+    cudaFuncAttributes f;                                                                                  \
+    return cudaFuncGetAttributes(&f, queue_kernel<P>);                                                     \
+  }                                                                                                        \
   }
 #define HARU_SDTW_FIXUP_INSTANCE(P)                                                            \
   namespace haru {                                                                             \
@@ -1383,5 +1566,11 @@ int occupancy_prec(int tile_cols, int warps, int solo) {
   cudaError_t sdtw_fixup_load_##P() {                                                          \
     cudaFuncAttributes f;                                                                      \
     return cudaFuncGetAttributes(&f, fixup_kernel<P>);                                         \
+  }                                                                                            \
+  }
+#define HARU_SDTW_TRACE_INSTANCE(P)                                                            \
+  namespace haru {                                                                             \
+  cudaError_t sdtw_trace_##P(const SdtwArgs &a, int max_items, bool stacked, cudaStream_t s) { \
+    return launch_trace_prec<P>(a, max_items, stacked, s);                                     \
   }                                                                                            \
   }

@@ -1,4 +1,4 @@
-// int16 inputs with wide accumulation: the sweep kernel, every strip height (1..16).
+// int16 inputs, wide accumulation: the scheduled sweep kernel, every strip height (1..16).
 #include "sdtw_kernels.cuh"
 
 HARU_SDTW_SWEEP_INSTANCE(2)

@@ -1,0 +1,4 @@
+// int16 inputs, wide accumulation, with start columns: the trace kernel, every strip height (1..16).
+#include "sdtw_kernels.cuh"
+
+HARU_SDTW_TRACE_INSTANCE(4)

@@ -42,3 +42,24 @@ def test_schedule_matches_unsplit(haru, nq, lo, hi, n, stack):
             np.testing.assert_array_equal(a[1], b[1])
             if prec == haru.HARU_INT16 and nq <= 26 and stack < 0:
                 compare_int16(a[0], a[1], ref, ev, off)
+
+
+# Tracing starts from checkpoints (references of 2,048 columns and more) against carrying them through the sweep: just
+# below and above the line; queries end anywhere, whole checkpoints back included.
+@pytest.mark.parametrize("n", [2047, 2048, 2049, 30011])
+@pytest.mark.parametrize("units,stack", [(0, -1), (0, 1), (1, 1), (2000, -1)])
+def test_start_columns_match_oracle(haru, n, units, stack):
+    import oracle
+    nq = 24
+    ref, ev, off = batch(nq, 1, 512, n, n)
+    ref, ev = (ref - 90) / 4 + 15, (ev - 90) / 4 + 15  # codes around 960, none at the clamp
+    ev[off[3]:off[4]] = ref[:off[4] - off[3]]          # from the first column on
+    ev[off[5]:off[6]] = ref[n - (off[6] - off[5]):]    # to the last
+    with haru.Context(stack_short=stack, units_target=units) as ctx:
+        ctx.ref_load(ref, normalize=False)
+        for prec, oprec in ((haru.HARU_FP32, oracle.PREC_F32), (haru.HARU_INT16_ACC32, oracle.PREC_I32)):
+            cost, col, start = ctx.sdtw_batch_span(prec, ev, off, raw=False)
+            o = oracle.batch(oprec, ref, ev, off, normalize_ref=False, normalize_q=False, start=True)
+            np.testing.assert_array_equal(cost, o.cost)
+            np.testing.assert_array_equal(col, o.col)
+            np.testing.assert_array_equal(start, o.start)
