@@ -203,8 +203,6 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
   const int asked = precision;
   const bool trace = traced(precision, lc);
   if (trace) precision = cost_form(precision);
-  // (a caller that ran kernels reporting into the status word first has zeroed the counters itself)
-  if (zero_counters && (e = cudaMemsetAsync(ws.ints, 0, kIntWords * sizeof(int), s)) != cudaSuccess) return e;
   if (ev_prep && (e = record_event(ev_prep, s)) != cudaSuccess) return e;
   PlanArgs pa;
   pa.offsets = d_offsets;
@@ -229,9 +227,9 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
   pa.arrived = ws.arrived;
   pa.groups = ws.groups;
   pa.ints = ws.ints;
-  if ((e = launch_plan(pa, s)) != cudaSuccess) return e;
-  if (raw && (e = launch_qstats(d_events, d_offsets, nq, ws.qstats, ws.ints + kIntStatus, s)) != cudaSuccess)
-    return e;
+  // (a caller that ran kernels reporting into the status word first has zeroed the counters itself)
+  pa.zero = zero_counters;
+  if ((e = launch_prep(pa, d_events, raw ? ws.qstats : nullptr, s)) != cudaSuccess) return e;
 
   PackArgs ka;
   ka.events = d_events;

@@ -261,6 +261,7 @@ struct PlanArgs {
   long N;
   int pair;                 // 0: FP32 singles; 1: INT16 pairs; 3: exact-integer singles, unsaturated
                             // (HARU_INT16_ACC32)
+  int zero;                 // 1: the planner zeroes ints first
   int warps;                // warps per CTA (explicit unit target: items per group)
   int units_target;         // wanted work units (item x segment) in the batch; 0: by the cost model below
   int slots;                // cost model: CTAs
@@ -283,18 +284,17 @@ struct PackArgs {
   const int *n_items;
   uint32_t *img;
   int raw;                  // z-score each query first
-  const double *qstats;     // raw: (mean, sigma) of query q at 2q, 2q+1 (launch_qstats)
+  const double *qstats;     // raw: (mean, sigma) of query q at 2q, 2q+1 (launch_prep)
   int pair;
   int scale_log2;
   int *status;
 };
 
 // Kernel launchers (stream-ordered, no synchronisation).
-cudaError_t launch_plan(const PlanArgs &a, cudaStream_t s);
+// The plan and, on raw events (qstats != nullptr), the mean and population
+// sigma (FP64, sequential order) of each query of 1..512 events.
+cudaError_t launch_prep(const PlanArgs &a, const float *events, double *qstats, cudaStream_t s);
 cudaError_t launch_pack(const PackArgs &a, uint32_t max_items, cudaStream_t s);
-// Mean and population sigma (FP64, sequential order) of each query of 1..512 events.
-cudaError_t launch_qstats(const float *events, const uint32_t *offsets, uint32_t nq, double *qstats, int *status,
-                          cudaStream_t s);
 cudaError_t launch_sdtw(int precision, const SdtwArgs &a, int grid, int fix_items, cudaStream_t s,
                         cudaEvent_t ev_fix = nullptr);
 // Start columns from the checkpoints of a cost sweep whose results are in

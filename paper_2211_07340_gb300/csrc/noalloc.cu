@@ -99,9 +99,8 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   double *qstats = reinterpret_cast<double *>(base + kNaStatsOff);
   const size_t max_items = items_bound(precision == HARU_INT16 ? 1 : 0, nq);
 
-  // The array keeps the previous call's contents: the status word and the
-  // counters must start at zero; items, groups and images are rewritten.
-  if ((e = cudaMemsetAsync(status, 0, kIntWords * sizeof(int), s)) != cudaSuccess) return ctx_cuda_fail(ctx, e);
+  // The array keeps the previous call's contents: the planner zeroes the
+  // status word and the counters; items, groups and images are rewritten.
   PlanArgs pa;
   pa.offsets = offsets;
   pa.nq = nq;
@@ -118,9 +117,8 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   pa.arrived = nullptr;  // one segment per item
   pa.groups = groups;
   pa.ints = status;
-  if ((e = launch_plan(pa, s)) != cudaSuccess) return ctx_cuda_fail(ctx, e);
-  if ((flags & HARU_RAW) &&
-      (e = launch_qstats(events, offsets, nq, qstats, status + kIntStatus, s)) != cudaSuccess)
+  pa.zero = 1;
+  if ((e = launch_prep(pa, events, (flags & HARU_RAW) ? qstats : nullptr, s)) != cudaSuccess)
     return ctx_cuda_fail(ctx, e);
   PackArgs ka;
   ka.events = events;

@@ -286,14 +286,22 @@ __device__ void cost_model(const PlanArgs &a, PlanTables &t) {
 // the longest-processing-time-first order of the work queue), keeps the
 // input order inside a bucket, pairs neighbours for the int16 form, and writes
 // the static schedule or (explicit unit target) the queue of groups.
-__global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
-  constexpr int kKeys = 2 * (kMaxS + 1);  // plain and stacked buckets of each S
-  __shared__ PlanTables t;
-  __shared__ int wrun[32][kKeys];  // per warp and bucket: count, then next position
+constexpr int kKeys = 2 * (kMaxS + 1);  // plain and stacked buckets of each S
+struct PlanShared {
+  PlanTables t;
+  int wrun[32][kKeys];  // per warp and bucket: count, then next position
+};
+__device__ void plan_block(const PlanArgs &a, PlanShared &sm) {
+  PlanTables &t = sm.t;
+  auto &wrun = sm.wrun;
   int *const ibase = t.ibase, *const sbase = t.sbase, *const icount = t.icount;
   auto nseg_of = [&](int S, int item) { return t.nseg[2 * (kMaxS - S) + (item - t.ibase[S] >= t.full[S] ? 1 : 0)]; };
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   int *status = a.ints + kIntStatus;
+  if (a.zero) {
+    if (tid < kIntWords) a.ints[tid] = 0;
+    __syncthreads();
+  }
   // Each warp owns a contiguous range of queries, so bucket positions
   // (earlier warps first, then the order inside the warp) keep input order.
   const uint32_t per_warp = (a.nq + nw - 1) / nw;
@@ -301,12 +309,15 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
   const uint32_t q_hi = min(a.nq, q_lo + per_warp);
   for (int b = lane; b < kKeys; b += 32) wrun[warp][b] = 0;
   __syncwarp();
-  for (uint32_t q0 = q_lo; q0 < q_hi; q0 += 32) {
-    const uint32_t q = q0 + lane;
-    const int key = q < q_hi ? bucket_key(a.offsets, q, a.N, a.pair, a.stack, status) : 0;
+  auto key_of = [&](uint32_t q, int *st) {
+    return q < q_hi ? bucket_key(a.offsets, q, a.N, a.pair, a.stack, st) : 0;
+  };
+  for (uint32_t q0 = q_lo, key = key_of(q_lo + lane, status); q0 < q_hi; q0 += 32) {
+    const uint32_t after = key_of(q0 + 32 + lane, status);  // loaded a round ahead
     const unsigned peers = __match_any_sync(0xffffffffu, key);
     if (key && lane == __ffs(peers) - 1) wrun[warp][key] += __popc(peers);
     __syncwarp();
+    key = after;
   }
   __syncthreads();
   if (tid >= 1 && tid < kKeys) {
@@ -319,17 +330,28 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
     t.cnt[tid] = c;
   }
   __syncthreads();
-  if (tid == 0) {
-    int base = 0;
-    for (int S = kMaxS; S >= 1; --S) {  // plain items of height S, then stacked ones
-      const int plain = bucket_items(a.pair, t.cnt[S]);
-      icount[S] = plain + stacked_items(a.pair, t.cnt[S + kMaxS + 1]);
-      ibase[S] = base;
-      sbase[S] = base + plain;
-      base += icount[S];
+  if (warp == 0) {  // lane l: height 16 - l, its plain items, then its stacked ones
+    const int S = lane < kMaxS ? kMaxS - lane : 0;
+    const int plain = S ? bucket_items(a.pair, t.cnt[S]) : 0;
+    const int items = S ? plain + stacked_items(a.pair, t.cnt[S + kMaxS + 1]) : 0;
+    int end = items;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += v;
     }
-    a.ints[kIntItems] = base;
-    a.ints[kIntQueue] = 0;
+    if (S) {
+      icount[S] = items;
+      ibase[S] = end - items;
+      sbase[S] = end - items + plain;
+    }
+    if (lane == 31) {
+      a.ints[kIntItems] = t.cnt[0] = end;
+      a.ints[kIntQueue] = 0;
+    }
+    __syncwarp();
+  }
+  if (tid == 0) {
+    const int base = t.cnt[0];
     if (a.units_target > 0) {
       // An explicit unit target: segments per item to reach it, each
       // at least four warm-ups (and 2048 steps) long.
@@ -393,7 +415,7 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
     }
     __syncthreads();
   }
-  const int n_items = a.ints[kIntItems];
+  const int n_items = t.cnt[0];
   for (int i = tid; i < n_items; i += blockDim.x) {
     Item it;
     it.qa = -1; it.qb = -1; it.S = 0; it.nseg = 1;
@@ -404,9 +426,10 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
   }
   __syncthreads();
   const unsigned lt = (1u << lane) - 1u;
-  for (uint32_t q0 = q_lo; q0 < q_hi; q0 += 32) {
+  for (uint32_t q0 = q_lo, next = key_of(q_lo + lane, nullptr); q0 < q_hi; q0 += 32) {
     const uint32_t q = q0 + lane;
-    const int key = q < q_hi ? bucket_key(a.offsets, q, a.N, a.pair, a.stack, nullptr) : 0;
+    const int key = static_cast<int>(next);
+    next = key_of(q0 + 32 + lane, nullptr);
     const unsigned peers = __match_any_sync(0xffffffffu, key);
     if (key > kMaxS) {  // stacked: slots qa, qb | qc, qd (INT16) or qa | qc (FP32)
       const int b = key - kMaxS - 1;
@@ -442,55 +465,189 @@ __global__ void __launch_bounds__(1024) plan_kernel(PlanArgs a) {
 }
 
 // ----------------------------------------------------------------- pack --
-// Mean and sigma of one query, sequentially (a query is shorter than one
-// z-score block, so this is the blocked rule's order).
-// Loads are issued eight at a time ahead of the (sequential) additions.
-__device__ void query_stats(const float *x, int m, double &mean, double &sigma) {
-  constexpr int B = 8;
-  float v[B];
-  double acc = 0.0;
-  int i = 0;
-  for (; i + B <= m; i += B) {
-#pragma unroll
-    for (int j = 0; j < B; ++j) v[j] = __ldg(x + i + j);
-#pragma unroll
-    for (int j = 0; j < B; ++j) acc = __dadd_rn(acc, static_cast<double>(v[j]));
-  }
-  for (; i < m; ++i) acc = __dadd_rn(acc, static_cast<double>(__ldg(x + i)));
-  mean = __ddiv_rn(acc, static_cast<double>(m));
-  double ss = 0.0;
-  i = 0;
-  for (; i + B <= m; i += B) {
-#pragma unroll
-    for (int j = 0; j < B; ++j) v[j] = __ldg(x + i + j);
-#pragma unroll
-    for (int j = 0; j < B; ++j) {
-      const double d = __dsub_rn(static_cast<double>(v[j]), mean);
-      ss = __dadd_rn(ss, __dmul_rn(d, d));
-    }
-  }
-  for (; i < m; ++i) {
-    const double d = __dsub_rn(static_cast<double>(__ldg(x + i)), mean);
-    ss = __dadd_rn(ss, __dmul_rn(d, d));
-  }
-  sigma = __dsqrt_rn(__ddiv_rn(ss, static_cast<double>(m)));
+// z = (float)((x - mean) / sigma), both roundings of the quotient kept, from
+// the reciprocal r = 1 / sigma: d * r is within two units in the last place
+// of the quotient in double, so the quotient's float is the product's unless
+// the product lies within a few units of the midpoint between two floats (29
+// bits below a float's last), is as small as a subnormal float, or is not
+// finite: then the division is done. (The double-precision unit takes 16
+// clocks a warp instruction on GB300; a division is about ten of them.)
+__device__ __forceinline__ float z_of(float x, double mean, double sigma, double r) {
+  const double d = __dsub_rn(static_cast<double>(x), mean);
+  const double q = __dmul_rn(d, r);
+  const unsigned hi = static_cast<unsigned>(__double2hiint(q)), lo = static_cast<unsigned>(__double2loint(q));
+  const unsigned exponent = (hi >> 20) & 0x7ffu;
+  const unsigned below = lo & 0x1fffffffu;  // the bits under a float's last
+  const bool near_half = below - (0x10000000u - 8u) <= 16u;
+  if (near_half || exponent < 1023u - 120u || exponent > 1023u + 120u) return __double2float_rn(__ddiv_rn(d, sigma));
+  return __double2float_rn(q);
 }
 
-// One thread per query: its mean and sigma (the sums are sequential chains,
-// so a query gets a thread of its own rather than a lane of a packing warp).
-__global__ void qstats_kernel(const float *events, const uint32_t *offsets, uint32_t nq, double *qstats,
-                              int *status) {
-  const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  const uint32_t b = offsets[q];
-  const uint32_t m = offsets[q + 1] - b;
-  double mu = 0.0, sg = 1.0;
-  if (m >= 1 && m <= HARU_MAX_QUERY) {  // other lengths are rejected by the planner
-    query_stats(events + b, static_cast<int>(m), mu, sg);
-    if (!(sg > 0.0) || !isfinite(sg) || !isfinite(mu)) report(status, HARU_EINVAL);
+// Mean and sigma (FP64) of each query of 1..512 events: the sums are those of
+// sequential additions in index order.
+// Mean: if every event is a multiple of 2^low and below 2^top in magnitude
+// with top + 9 - low <= 53, no partial sum of up to 512 of them rounds, in
+// any order, and the sum is taken on integers across a warp; other queries
+// are added up one by one.
+// Sigma: the additions of the squared deviations round, so they stay one
+// chain per query, 64 clocks each; a lane of the block's first warps (chain
+// warps) holds the chain of one query, and the other warps compute the
+// squares of the next chunk of events meanwhile (one thread per query, with
+// its loads and conversions in the chain, took 52 us at 250 events and 104
+// us on 8,192 queries of up to 500; this kernel, planner included, 16 and 48).
+constexpr int kStatQueries = 64;  // per block at most: two chain warps
+constexpr int kStatSquares = kStatQueries * 33;
+struct StatShared {
+  double sq[2][kStatSquares];  // [query][chunk + 1]
+  long long sum[kStatQueries];
+  double mean[kStatQueries];
+  int low[kStatQueries];  // exponent of the integer sum's unit; kInexact: add one by one
+  int length[kStatQueries];
+  uint32_t base[kStatQueries];
+  int longest;
+};
+constexpr int kInexact = 0x7fffffff;
+struct StatArgs {
+  const float *events;
+  const uint32_t *offsets;
+  uint32_t nq;
+  int per_block;  // queries, 32 or 64
+  double *qstats;
+};
+
+__device__ __forceinline__ double as_double(float x) {  // exact; normal numbers without the conversion unit
+  const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  if (e == 0u || e == 255u) return static_cast<double>(x);
+  return __hiloint2double(static_cast<int>((b & 0x80000000u) | ((e + 896u) << 20) | ((b >> 3) & 0xfffffu)),
+                          static_cast<int>(b << 29));
+}
+
+__device__ void stat_block(const StatArgs &a, int block, StatShared &sm) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const uint32_t q0 = static_cast<uint32_t>(block) * a.per_block;
+  // a block of up to 32 queries takes chunks of 64 events, one of 64 queries 32
+  const int chunk = a.per_block > 32 ? 32 : 64, row = chunk + 1, chain_warps = (a.per_block + 31) / 32;
+  if (tid == 0) sm.longest = 0;
+  __syncthreads();
+  if (tid < a.per_block) {
+    const uint32_t q = q0 + tid, b = q < a.nq ? a.offsets[q] : 0u, m = q < a.nq ? a.offsets[q + 1] - b : 0u;
+    const int len = m <= HARU_MAX_QUERY ? static_cast<int>(m) : 0;  // other lengths are rejected by the planner
+    sm.length[tid] = len;
+    sm.base[tid] = b;
+    atomicMax(&sm.longest, len);
   }
-  qstats[2 * static_cast<size_t>(q)] = mu;
-  qstats[2 * static_cast<size_t>(q) + 1] = sg;
+  __syncthreads();
+  for (int k = warp; k < a.per_block; k += nw) {
+    const float *x = a.events + sm.base[k];
+    const int m = sm.length[k];
+    constexpr int kPer = HARU_MAX_QUERY / 32;
+    unsigned v[kPer];
+    int low = 1 << 20, top = -(1 << 20);
+    bool finite = true;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const int i = j * 32 + lane;
+      v[j] = i < m ? __float_as_uint(__ldg(x + i)) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const unsigned mag = v[j] & 0x7fffffffu, e = mag >> 23;
+      if (mag == 0u) continue;
+      finite = finite && e != 255u;
+      const unsigned mant = (mag & 0x7fffffu) | (e ? 0x800000u : 0u);
+      const int at = max(static_cast<int>(e), 1) - 150;  // of the mantissa's last bit
+      low = min(low, at + __ffs(mant) - 1);
+      top = max(top, at + 32 - __clz(mant));
+    }
+    low = __reduce_min_sync(0xffffffffu, low);
+    top = __reduce_max_sync(0xffffffffu, top);
+    finite = __all_sync(0xffffffffu, finite);
+    const bool exact = finite && top + 9 - low <= 53;
+    long long sum = 0;
+    if (exact) {
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) {
+        const unsigned mag = v[j] & 0x7fffffffu, e = mag >> 23;
+        const unsigned mant = (mag & 0x7fffffu) | (e ? 0x800000u : 0u);
+        const int up = max(static_cast<int>(e), 1) - 150 - low;
+        const long long u = mag == 0u ? 0 : (up >= 0 ? static_cast<long long>(mant) << up : mant >> -up);
+        sum += (v[j] >> 31) ? -u : u;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) {
+      sm.sum[k] = sum;
+      sm.low[k] = exact ? low : kInexact;
+    }
+  }
+  __syncthreads();
+  const bool chain = tid < a.per_block;  // this thread's query: tid
+  double ss = 0.0, count = 1.0;
+  int own = 0;
+  if (chain) {
+    const float *x = a.events + sm.base[tid];
+    own = sm.length[tid];
+    double acc = 0.0;
+    if (sm.low[tid] != kInexact) {
+      // (low = 1 << 20: every event is 0)
+      const int low = sm.low[tid];
+      if (sm.sum[tid] != 0)
+        acc = __dmul_rn(__ll2double_rn(sm.sum[tid]), __hiloint2double((1023 + low) << 20, 0));
+    } else {
+      for (int i = 0; i < own; ++i) acc = __dadd_rn(acc, static_cast<double>(__ldg(x + i)));
+    }
+    count = static_cast<double>(max(own, 1));
+    sm.mean[tid] = __ddiv_rn(acc, count);
+  }
+  __syncthreads();
+  const int chunks = (sm.longest + chunk - 1) / chunk;
+  auto squares = [&](int c, int from, int warps) {  // by `warps` warps, this one's number `from`
+    for (int k = from; k < a.per_block; k += warps) {
+      const float *x = a.events + sm.base[k];
+      const int m = sm.length[k];
+      const double mean = sm.mean[k];
+      for (int o = lane; o < chunk; o += 32) {
+        const int i = c * chunk + o;
+        double p = 0.0;  // beyond the query: adding 0 changes nothing
+        if (i < m) {
+          const double d = __dsub_rn(as_double(__ldg(x + i)), mean);
+          p = __dmul_rn(d, d);
+        }
+        sm.sq[c & 1][k * row + o] = p;
+      }
+    }
+  };
+  if (chunks > 0) squares(0, warp, nw);
+  __syncthreads();
+  for (int c = 0; c < chunks; ++c) {
+    if (chain) {
+      const double *sq = &sm.sq[c & 1][tid * row];
+#pragma unroll 16
+      for (int i = 0; i < chunk; ++i) ss = __dadd_rn(ss, sq[i]);
+    } else if (warp >= chain_warps && c + 1 < chunks) {
+      squares(c + 1, warp - chain_warps, nw - chain_warps);
+    }
+    __syncthreads();
+  }
+  if (chain && q0 + tid < a.nq) {
+    const size_t q = q0 + tid;
+    a.qstats[2 * q] = own > 0 ? sm.mean[tid] : 0.0;
+    a.qstats[2 * q + 1] = own > 0 ? __dsqrt_rn(__ddiv_rn(ss, count)) : 1.0;
+  }
+}
+
+// Block 0 plans the batch; the others, on raw events, form the queries'
+// means and sigmas at the same time.
+__global__ void __launch_bounds__(1024) prep_kernel(PlanArgs p, StatArgs st) {
+  __shared__ union Shared {
+    PlanShared plan;
+    StatShared stat;
+    __device__ Shared() {}
+  } sm;
+  if (blockIdx.x == 0)
+    plan_block(p, sm.plan);
+  else
+    stat_block(st, static_cast<int>(blockIdx.x) - 1, sm.stat);
 }
 
 // One warp per item: lane l writes rows l*S .. l*S+S-1 of both halves (of
@@ -508,7 +665,7 @@ __global__ void pack_kernel(PackArgs a) {
   const int lane_in = it.stacked ? (lane & 15) : lane;   // lane within the stack
   int m[2] = {0, 0};
   uint32_t base[2] = {0, 0};
-  double mean[2] = {0.0, 0.0}, sigma[2] = {1.0, 1.0};
+  double mean[2] = {0.0, 0.0}, sigma[2] = {1.0, 1.0}, inv[2] = {1.0, 1.0};
   const bool packed = a.pair == 1;  // two int16 queries per word
   const bool codes = a.pair != 0;   // int16 codes (packed, or as floats)
   int most = 0;
@@ -524,6 +681,7 @@ __global__ void pack_kernel(PackArgs a) {
       if (qs[h] >= 0) {
         mean[h] = a.qstats[2 * static_cast<size_t>(qs[h])];
         sigma[h] = a.qstats[2 * static_cast<size_t>(qs[h]) + 1];
+        inv[h] = __drcp_rn(sigma[h]);
       }
     }
   }
@@ -538,10 +696,8 @@ __global__ void pack_kernel(PackArgs a) {
       float z = 0.0f;
       if (real) {
         const float x = a.events[base[h] + (row - P)];
-        if (a.raw)
-          z = __double2float_rn(__ddiv_rn(__dsub_rn(static_cast<double>(x), mean[h]), sigma[h]));
-        else
-          z = x;
+        z = a.raw ? z_of(x, mean[h], sigma[h], inv[h]) : x;
+        // (a query without spread has sigma 0: its quotients are not finite)
         if (!isfinite(z) || fabsf(z) > 1.0e20f) report(a.status, HARU_EINVAL);
       }
       if (packed) {
@@ -569,15 +725,20 @@ __global__ void pack_kernel(PackArgs a) {
 
 }  // namespace
 
-cudaError_t launch_plan(const PlanArgs &a, cudaStream_t s) {
-  plan_kernel<<<1, 1024, 0, s>>>(a);
+cudaError_t launch_prep(const PlanArgs &a, const float *events, double *qstats, cudaStream_t s) {
+  StatArgs st{events, a.offsets, a.nq, kStatQueries, qstats};
+  // As few queries to a block as run at once: the chains share the
+  // double-precision unit with the squares of their block's queries.
+  for (int k : {32, 8})
+    if (a.nq <= static_cast<uint32_t>(k) * 144u) st.per_block = k;
+  const unsigned blocks = qstats ? (a.nq + st.per_block - 1) / st.per_block : 0;
+  prep_kernel<<<1 + blocks, 1024, 0, s>>>(a, st);
   return cudaGetLastError();
 }
 
 cudaError_t load_prep_kernels() {
   cudaFuncAttributes f;
-  cudaError_t e = cudaFuncGetAttributes(&f, plan_kernel);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&f, qstats_kernel);
+  cudaError_t e = cudaFuncGetAttributes(&f, prep_kernel);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&f, pack_kernel);
   return e;
 }
@@ -586,14 +747,6 @@ cudaError_t launch_pack(const PackArgs &a, uint32_t max_items, cudaStream_t s) {
   if (max_items == 0) return cudaSuccess;
   const int warps = 8;
   pack_kernel<<<(max_items + warps - 1) / warps, warps * 32, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_qstats(const float *events, const uint32_t *offsets, uint32_t nq, double *qstats, int *status,
-                          cudaStream_t s) {
-  if (nq == 0) return cudaSuccess;
-  const int th = 32;  // one warp per block: the sequential chains spread over every SM
-  qstats_kernel<<<(nq + th - 1) / th, th, 0, s>>>(events, offsets, nq, qstats, status);
   return cudaGetLastError();
 }
 
