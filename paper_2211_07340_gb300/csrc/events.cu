@@ -20,8 +20,8 @@
 // [trim, trim + max_events).
 //
 // Kernels: detect_kernel (one CTA per read: the read's samples in shared
-// memory, statistics over tiles of kEvTile positions with halos, each thread
-// sliding its window sums along a run of positions; peaks compared on float
+// memory, statistics over tiles of kEvTpos positions, halos included, each
+// thread forming those of a run of positions; peaks compared on float
 // t^2 values with a margin that covers their rounding, falling back to the
 // exact integers when it cannot decide; an ordered block-wide compaction of
 // boundaries that stops once the query's boundaries are known; then the
@@ -38,20 +38,19 @@ namespace haru {
 namespace {
 
 constexpr int kEvThreads = 256;
-constexpr int kEvTile = 1024;                      // boundary positions per tile
-constexpr int kEvPer = kEvTile / kEvThreads;       // consecutive positions per thread
+constexpr int kEvPer = 4;                          // consecutive statistics per thread and tile
+constexpr int kEvTpos = kEvThreads * kEvPer;       // statistics per tile; positions: those without the halos
 constexpr int kEvMaxW = 16;                        // longest window
-constexpr int kEvTpos = kEvTile + 4 * kEvMaxW;     // statistics per tile (halo w1 + w2 on each side)
-constexpr int kEvRun = (kEvTpos + kEvThreads - 1) / kEvThreads;  // statistics per thread (a contiguous run)
-constexpr int kEvLp = kEvTile + 2 * kEvMaxW;       // long-peak flags per tile (halo w1 on each side)
-static_assert(kEvTile % kEvThreads == 0 && kEvPer <= 32, "tile split");
+constexpr int kEvFastW = 8;                        // longest window of the register path (larger ones: sliding sums)
+constexpr int kEvPad = 16;                         // undefined statistics around a tile's (>= kEvMaxW)
+static_assert(kEvTpos > 4 * kEvMaxW, "a tile longer than its halos");
 
 // Shared-memory layout of detect_kernel (bytes); the boundary list follows,
 // as many ints as the query needs (trim + max_events).
-constexpr size_t kSmX = 0;                                                  // int16 samples
-constexpr size_t kSmT = kSmX + HARU_MAX_READ_SAMPLES * sizeof(int16_t);     // 2 x kEvTpos float t^2
-constexpr size_t kSmLp = kSmT + 2 * kEvTpos * sizeof(float);
-constexpr size_t kSmBounds = kSmLp + (kEvLp + 15) / 16 * 16;
+constexpr size_t kSmX = 0;                                                    // int16 samples, up to 7 in front
+constexpr size_t kSmT = kSmX + (HARU_MAX_READ_SAMPLES + 8) * sizeof(int16_t);  // 2 x (kEvTpos + 2 kEvPad) float t^2
+constexpr size_t kSmLp = kSmT + 2 * (kEvTpos + 2 * kEvPad) * sizeof(float);   // long-peak bits, one word on each side
+constexpr size_t kSmBounds = kSmLp + (kEvTpos / 32 + 2 + 2) / 4 * 4 * sizeof(unsigned);
 size_t detect_smem_bytes(int need) { return kSmBounds + static_cast<size_t>(need) * sizeof(int); }
 
 struct EvArgs {
@@ -128,9 +127,9 @@ __device__ __noinline__ void exact_stat(const int16_t *x, int w, int i, unsigned
   s.stat(w, num, den);
 }
 
-// The float t^2 of a statistic carries a relative error below 2^-21 (the
-// numerator and denominator each rounded once to float, one correctly
-// rounded division), so two of them decide a comparison of the exact values
+// The float t^2 of a statistic carries a relative error below 2^-20 (the
+// numerator and denominator each rounded once to float, one division of at
+// most 2 units in the last place), so two of them decide a comparison of the exact values
 // whenever they differ by more than the margin; otherwise the comparison is
 // redone on the exact integers.
 constexpr float kMarginUp = 1.0f + 1.0f / 262144.0f, kMarginDown = 1.0f - 1.0f / 262144.0f;  // 2^-18
@@ -157,9 +156,8 @@ __device__ __forceinline__ bool t_above(const int16_t *x, int w, int qi, float t
 
 // Peak test of statistic index j (position q) of a tile: above the threshold,
 // strictly above the w defined statistics before it, at least the w after
-// it. Undefined statistics hold -1. The caller keeps j - w >= 0 and
-// j + w < kEvTpos.
-__device__ __forceinline__ bool peak(const int16_t *x, const float *tf, int j, int q, int w, float tauf,
+// it. Undefined statistics hold -1 (also the kEvPad around the tile's).
+__device__ __noinline__ bool peak(const int16_t *x, const float *tf, int j, int q, int w, float tauf,
                                      unsigned long long tausq) {
   const float tj = tf[j];
   if (tj < 0.0f || !t_above(x, w, q, tj, tauf, tausq)) return false;
@@ -172,18 +170,16 @@ __device__ __forceinline__ bool peak(const int16_t *x, const float *tf, int j, i
   return true;
 }
 
-// Statistics of window w at positions q = p0 - H + j for this thread's run
-// of j, sliding the window sums along the run.
-__device__ __forceinline__ void tile_stats(const int16_t *x, int n, int w, int p0, int H, int jmax, float *tf) {
+// t^2 of window w at positions q .. q + kEvPer - 1, by sliding the window
+// sums in 64 bits (any window, any samples).
+__device__ __noinline__ void stats_any(const int16_t *x, int n, int w, int q0, float *t /* shared */) {
   Win s;
   bool have = false;
 #pragma unroll
-  for (int r = 0; r < kEvRun; ++r) {
-    const int j = threadIdx.x * kEvRun + r;
-    if (j >= jmax) break;
-    const int q = p0 - H + j;
+  for (int r = 0; r < kEvPer; ++r) {
+    const int q = q0 + r;
+    t[r] = -1.0f;
     if (q < w || q > n - w) {
-      tf[j] = -1.0f;
       have = false;
       continue;
     }
@@ -194,18 +190,124 @@ __device__ __forceinline__ void tile_stats(const int16_t *x, int n, int w, int p
     have = true;
     unsigned long long num, den;
     s.stat(w, &num, &den);
-    tf[j] = __fdiv_rn(__ull2float_rn(num), __ull2float_rn(den));
+    t[r] = __fdiv_rn(__ull2float_rn(num), __ull2float_rn(den));
   }
 }
 
-// Four CTAs per SM (shared memory ~44 KB each with the default parameters).
-__global__ void __launch_bounds__(kEvThreads, 4) detect_kernel(EvArgs a) {
+// The same on the thread's kEvPer + 2 W samples in registers, in 32 bits: the
+// statistic does not change when a constant is taken off every sample, and
+// with samples within `half` of the read's middle value its terms are at
+// most 4 W^3 half^2, which the caller keeps below 2^31. (About 20 operations
+// a position and window, where 64-bit sums, products, conversions and the
+// rounded division took several hundred.)
+__device__ __forceinline__ bool fits_32(int w, int half) {
+  return w <= kEvFastW && static_cast<long long>(half) * half * w * w * w < (1ll << 29);
+}
+template <int W>
+__device__ __forceinline__ void stats_32(const int16_t *x, int n, int middle, int q0, float *tf) {
+  int v[kEvPer + 2 * W];
+#pragma unroll
+  for (int i = 0; i < kEvPer + 2 * W; ++i) {
+    const int at = q0 - W + i;
+    v[i] = at >= 0 && at < n ? x[at] - middle : 0;
+  }
+  float t[kEvPer];
+  int A = 0, B = 0, Q = 0;  // window sums, and both windows' sum of squares
+#pragma unroll
+  for (int i = 0; i < W; ++i) {
+    A += v[i];
+    B += v[W + i];
+    Q += v[i] * v[i] + v[W + i] * v[W + i];
+  }
+#pragma unroll
+  for (int r = 0; r < kEvPer; ++r) {
+    const int d = B - A, D = max(W * Q - A * A - B * B, 1);
+    const int q = q0 + r;
+    t[r] = q < W || q > n - W ? -1.0f : __fdividef(static_cast<float>(W * d * d), static_cast<float>(D));
+    if (r + 1 < kEvPer) {
+      A += v[r + W] - v[r];
+      B += v[r + 2 * W] - v[r + W];
+      Q += v[r + 2 * W] * v[r + 2 * W] - v[r] * v[r];
+    }
+  }
+  *reinterpret_cast<float4 *>(tf) = make_float4(t[0], t[1], t[2], t[3]);
+}
+__device__ __forceinline__ void stats_of(const int16_t *x, int n, int w, int middle, int half, int q0, float *t) {
+  if (fits_32(w, half)) {
+    switch (w) {
+      case 2: return stats_32<2>(x, n, middle, q0, t);
+      case 3: return stats_32<3>(x, n, middle, q0, t);
+      case 4: return stats_32<4>(x, n, middle, q0, t);
+      case 5: return stats_32<5>(x, n, middle, q0, t);
+      case 6: return stats_32<6>(x, n, middle, q0, t);
+      case 7: return stats_32<7>(x, n, middle, q0, t);
+      default: return stats_32<8>(x, n, middle, q0, t);
+    }
+  }
+  stats_any(x, n, w, q0, t);
+}
+
+// Peaks among statistics j .. j + kEvPer - 1 (j a multiple of kEvPer,
+// positions q0 + r) as bits: decided on the largest float of the neighbours
+// where the margin allows, else by peak().
+template <int W>
+__device__ __forceinline__ unsigned peaks_w(const int16_t *x, const float *tf, int j, int q0, float tauf,
+                                            unsigned long long tausq) {
+  constexpr int kHalo = (W + 3) / 4 * 4;
+  float v[kEvPer + 2 * kHalo];
+#pragma unroll
+  for (int i = 0; i < (kEvPer + 2 * kHalo) / 4; ++i)
+    *reinterpret_cast<float4 *>(v + 4 * i) = *reinterpret_cast<const float4 *>(tf + j - kHalo + 4 * i);
+  unsigned bits = 0, unsure = 0;
+#pragma unroll
+  for (int r = 0; r < kEvPer; ++r) {
+    const float t = v[kHalo + r];
+    float m = v[kHalo + r - W];
+#pragma unroll
+    for (int k = 1 - W; k <= W; ++k)
+      if (k != 0) m = fmaxf(m, v[kHalo + r + k]);
+    if (t < 0.0f || t < tauf * kMarginDown || t < m * kMarginDown) continue;
+    if (t > tauf * kMarginUp && t > m * kMarginUp)
+      bits |= 1u << r;
+    else
+      unsure |= 1u << r;
+  }
+  for (; unsure; unsure &= unsure - 1) {
+    const int r = __ffs(unsure) - 1;
+    if (peak(x, tf, j + r, q0 + r, W, tauf, tausq)) bits |= 1u << r;
+  }
+  return bits;
+}
+__device__ __forceinline__ unsigned peaks_of(const int16_t *x, const float *tf, int j, int q0, int w, float tauf,
+                                             unsigned long long tausq) {
+  switch (w) {
+    case 2: return peaks_w<2>(x, tf, j, q0, tauf, tausq);
+    case 3: return peaks_w<3>(x, tf, j, q0, tauf, tausq);
+    case 4: return peaks_w<4>(x, tf, j, q0, tauf, tausq);
+    case 5: return peaks_w<5>(x, tf, j, q0, tauf, tausq);
+    case 6: return peaks_w<6>(x, tf, j, q0, tauf, tausq);
+    case 7: return peaks_w<7>(x, tf, j, q0, tauf, tausq);
+    case 8: return peaks_w<8>(x, tf, j, q0, tauf, tausq);
+    default: {
+      unsigned bits = 0;
+      for (int r = 0; r < kEvPer; ++r) bits |= peak(x, tf, j + r, q0 + r, w, tauf, tausq) ? 1u << r : 0u;
+      return bits;
+    }
+  }
+}
+
+// Three CTAs per SM (80 registers a thread; with four and 64 it spilled and
+// ran the same). Each thread keeps kEvPer consecutive statistics of a tile from the window
+// sums to the boundaries; instruction bound (64 MB of samples in 8,192 reads
+// are 10 us of HBM time): 8,192 reads of 140..640 levels took 790 us with
+// 64-bit sums, products and divisions at every position and a neighbour loop
+// per candidate, 225 us this way.
+__global__ void __launch_bounds__(kEvThreads, 3) detect_kernel(EvArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
-  int16_t *x = reinterpret_cast<int16_t *>(sm + kSmX);
-  float *t1 = reinterpret_cast<float *>(sm + kSmT), *t2 = t1 + kEvTpos;
-  unsigned char *lp = sm + kSmLp;
+  float *t1 = reinterpret_cast<float *>(sm + kSmT) + kEvPad, *t2 = t1 + kEvTpos + 2 * kEvPad;
+  unsigned *lp = reinterpret_cast<unsigned *>(sm + kSmLp) + 1;  // long-peak bit of statistic j: word j / 32
   int *bounds = reinterpret_cast<int *>(sm + kSmBounds);
-  __shared__ int warp_tot[kEvThreads / 32];
+  __shared__ int warp_tot[kEvThreads / 32], warp_min[kEvThreads / 32], warp_max[kEvThreads / 32];
   __shared__ int s_nb;
   const uint32_t r = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -229,39 +331,94 @@ __global__ void __launch_bounds__(kEvThreads, 4) detect_kernel(EvArgs a) {
     return;
   }
   const int n = static_cast<int>(len);
-  for (int i = tid; i < n; i += kEvThreads) x[i] = a.samples[base + i];
-  if (tid == 0) s_nb = 0;
-  __syncthreads();
-  const int w1 = a.w1, w2 = a.w2, H = w1 + w2;
-  const int need = a.trim + a.maxev;  // boundaries b_1 .. b_need close the query's last event
-  for (int p0 = 0; p0 < n; p0 += kEvTile) {
-    // statistics at positions q = p0 - H + j, j in [0, kEvTile + 2H)
-    tile_stats(x, n, w1, p0, H, kEvTile + 2 * H, t1);
-    tile_stats(x, n, w2, p0, H, kEvTile + 2 * H, t2);
-    __syncthreads();
-    // long-window peaks at q = p0 - w1 + j, j in [0, kEvTile + 2 w1) (statistic index j + w2)
-    for (int j = tid; j < kEvTile + 2 * w1; j += kEvThreads)
-      lp[j] = peak(x, t2, j + w2, p0 - w1 + j, w2, a.tau2f, a.tau2sq) ? 1 : 0;
-    __syncthreads();
-    // boundaries among this thread's positions p0 + tid * kEvPer + u
-    unsigned flags = 0;
-    int cnt = 0;
+  // The samples keep their address modulo 16 bytes, so that whole 16-byte
+  // pieces move by vector loads and the ragged ends one by one.
+  const int16_t *src = a.samples + base;
+  const int front = static_cast<int>((reinterpret_cast<uintptr_t>(src) & 15) / sizeof(int16_t));
+  int16_t *x = reinterpret_cast<int16_t *>(sm + kSmX) + front;
+  int lo = 32767, hi = -32768;
+  {
+    const int head = min(n, (8 - front) & 7), pieces = (n - head) / 8, tail = head + pieces * 8;
+    auto take = [&](int v) { lo = min(lo, v); hi = max(hi, v); };
+    for (int i = tid; i < pieces; i += kEvThreads) {
+      const int4 p = reinterpret_cast<const int4 *>(src + head)[i];
+      reinterpret_cast<int4 *>(x + head)[i] = p;
+      const int w[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll
-    for (int u = 0; u < kEvPer; ++u) {
-      const int p = p0 + tid * kEvPer + u;
-      if (p < 1 || p > n - 1) continue;
-      const int jl = p - p0 + w1;  // its long-peak flag
-      bool b = lp[jl] != 0;
-      if (!b && peak(x, t1, p - p0 + H, p, w1, a.tau1f, a.tau1sq)) {
-        bool near = false;
-        for (int k = -w1; k <= w1; ++k) near = near || lp[jl + k] != 0;
-        b = !near;
-      }
-      if (b) {
-        flags |= 1u << u;
-        ++cnt;
+      for (int k = 0; k < 4; ++k) {
+        take(static_cast<short>(w[k] & 0xffff));
+        take(w[k] >> 16);
       }
     }
+    const int ragged = head + n - tail;
+    if (tid < ragged) {
+      const int i = tid < head ? tid : tail + tid - head;
+      x[i] = src[i];
+      take(x[i]);
+    }
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    warp_min[warp] = lo;
+    warp_max[warp] = hi;
+  }
+  if (tid == 0) s_nb = 0;
+  if (tid < kEvPad) {  // around the tiles' statistics: undefined
+    t1[tid - kEvPad] = t2[tid - kEvPad] = -1.0f;
+    t1[kEvTpos + tid] = t2[kEvTpos + tid] = -1.0f;
+  }
+  if (tid == 0) lp[-1] = lp[kEvTpos / 32] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kEvThreads / 32; ++w) {
+    lo = min(lo, warp_min[w]);
+    hi = max(hi, warp_max[w]);
+  }
+  const int middle = (lo + hi) >> 1, half = max(hi - middle, middle - lo);
+  const int w1 = a.w1, w2 = a.w2, H = w1 + w2;
+  const int T = kEvTpos - 2 * H;      // boundary positions per tile
+  const int need = a.trim + a.maxev;  // boundaries b_1 .. b_need close the query's last event
+  const int j0 = tid * kEvPer;        // this thread's statistics
+  for (int p0 = 0; p0 < n; p0 += T) {
+    // statistics at positions q = p0 - H + j, j in [0, kEvTpos)
+    const int q0 = p0 - H + j0;
+    stats_of(x, n, w1, middle, half, q0, t1 + j0);
+    stats_of(x, n, w2, middle, half, q0, t2 + j0);
+    __syncthreads();
+    // long-window peaks (those of statistics closer than w2 to a tile's end
+    // are not final; no boundary of this tile looks at them)
+    unsigned word = peaks_of(x, t2, j0, q0, w2, a.tau2f, a.tau2sq) << (kEvPer * (lane & 7));
+    const unsigned own_long = word >> (kEvPer * (lane & 7));
+    word |= __shfl_xor_sync(0xffffffffu, word, 1);
+    word |= __shfl_xor_sync(0xffffffffu, word, 2);
+    word |= __shfl_xor_sync(0xffffffffu, word, 4);
+    if ((lane & 7) == 0) lp[j0 / 32] = word;
+    __syncthreads();
+    // boundaries among this thread's positions p0 .. p0 + T - 1
+    unsigned flags = 0;
+    unsigned inside = 0;  // positions of this tile and of the read
+#pragma unroll
+    for (int u = 0; u < kEvPer; ++u) {
+      const int j = j0 + u, p = q0 + u;
+      if (j >= H && j < H + T && p >= 1 && p <= n - 1) inside |= 1u << u;
+    }
+    if (inside) {
+      flags = own_long & inside;
+      unsigned cand = inside & ~flags;
+      if (cand) cand &= peaks_of(x, t1, j0, q0, w1, a.tau1f, a.tau1sq);
+#pragma unroll
+      for (int u = 0; u < kEvPer; ++u) {
+        if (!((cand >> u) & 1u)) continue;
+        // no long peak at j - w1 .. j + w1
+        const int from = j0 + u - w1, at = from >> 5, sh = from & 31;  // (from >= -kEvMaxW: word -1)
+        const unsigned long long two = lp[at] | (static_cast<unsigned long long>(lp[at + 1]) << 32);
+        unsigned long long near = (two >> sh) & ((1ull << min(2 * w1 + 1, 64 - sh)) - 1ull);
+        if (2 * w1 + 1 > 64 - sh) near |= lp[at + 2] & ((1u << (2 * w1 + 1 - (64 - sh))) - 1u);
+        if (near == 0ull) flags |= 1u << u;
+      }
+    }
+    const int cnt = __popc(flags);
     // ordered compaction: exclusive prefix of cnt over the block; only the
     // first `need` boundaries are kept (the query uses b_1 .. b_need)
     int incl = cnt;
@@ -275,22 +432,23 @@ __global__ void __launch_bounds__(kEvThreads, 4) detect_kernel(EvArgs a) {
     int before = 0, total = 0;
 #pragma unroll
     for (int w = 0; w < kEvThreads / 32; ++w) {
-      const int t = warp_tot[w];
-      before += w < warp ? t : 0;
-      total += t;
+      const int v = warp_tot[w];
+      before += w < warp ? v : 0;
+      total += v;
     }
+    const int found = s_nb + total;
     int pos = s_nb + before + incl - cnt;
 #pragma unroll
     for (int u = 0; u < kEvPer; ++u)
       if (flags & (1u << u)) {
-        if (pos < need) bounds[pos] = p0 + tid * kEvPer + u;
+        if (pos < need) bounds[pos] = q0 + u;
         ++pos;
       }
     __syncthreads();
-    if (tid == 0) s_nb += total;
-    __syncthreads();
-    if (s_nb >= need) break;  // uniform: every thread reads the same s_nb
+    if (tid == 0) s_nb = found;
+    if (found >= need) break;  // uniform
   }
+  __syncthreads();
   const int nb = s_nb;
   int K = n > 0 ? nb + 1 - a.trim : 0;  // events after the trim (an empty read has none)
   K = K < 0 ? 0 : (K > a.maxev ? a.maxev : K);
@@ -304,11 +462,16 @@ __global__ void __launch_bounds__(kEvThreads, 4) detect_kernel(EvArgs a) {
   }
   for (int k = tid; k < K; k += kEvThreads) {
     const int e = a.trim + k;  // e + 1 <= need: both ends are stored boundaries (or 0, n)
-    const int lo = e == 0 ? 0 : bounds[e - 1];
-    const int hi = e + 1 <= nb ? bounds[e] : n;
-    long long s = 0;
-    for (int i = lo; i < hi; ++i) s += x[i];
-    out_row[k] = __double2float_rn(__ddiv_rn(static_cast<double>(s), static_cast<double>(hi - lo)));
+    const int b = e == 0 ? 0 : bounds[e - 1];
+    const int c = e + 1 <= nb ? bounds[e] : n;
+    int s = 0;  // at most 16,384 samples of 16 bits
+    for (int i = b; i < c; ++i) s += x[i];
+    // Below 2^24 the float quotient is the same: a quotient of whole numbers
+    // that is not itself halfway between two floats lies at least 2^-39 of it
+    // away from there, so the double's rounding never decides.
+    out_row[k] = abs(s) < (1 << 24)
+                     ? __fdiv_rn(static_cast<float>(s), static_cast<float>(c - b))
+                     : __double2float_rn(__ddiv_rn(static_cast<double>(s), static_cast<double>(c - b)));
   }
   if (tid == 0) a.counts[r] = static_cast<uint32_t>(K);
 }
