@@ -167,6 +167,7 @@ int haru_create(haru_ctx **out, int device, const haru_config *cfg) {
     size_t ci = 0;
     if (grow(&ctx->ws.ints, &ci, (size_t)haru::kIntWords) != cudaSuccess) { rc = HARU_ENOMEM; break; }
     if (cudaMalloc(&ctx->stats, 2 * sizeof(double)) != cudaSuccess) { rc = HARU_ENOMEM; break; }
+    if (cudaMallocHost(&ctx->stage, haru::kStageBytes) != cudaSuccess) { rc = HARU_ENOMEM; break; }
     bool ev_ok = true;
     for (auto &e : ctx->ev) ev_ok = ev_ok && cudaEventCreate(&e) == cudaSuccess;
     if (!ev_ok) { rc = HARU_ECUDA; break; }
@@ -206,6 +207,7 @@ void haru_destroy(haru_ctx *ctx) {
                   ctx->sig_strided, ctx->sig_events, ctx->sig_counts, ctx->sig_off};
   for (void *p : ptrs)
     if (p) cudaFree(p);
+  if (ctx->stage) cudaFreeHost(ctx->stage);
   free_ref_image(ctx->img16);
   free_ref_image(ctx->imgh);
   free_ref_image(ctx->img32);
@@ -400,9 +402,16 @@ int batch_call(haru_ctx *ctx, int precision, const float *events, const uint32_t
       HARU_CUDA(grow(&ctx->d_start, &c3, (size_t)nq + 1));
       ctx->cap_q = (size_t)nq + 1;
     }
-    HARU_CUDA(cudaMemcpyAsync(ctx->d_events, events, ne * sizeof(float), cudaMemcpyHostToDevice, s));
-    HARU_CUDA(cudaMemcpyAsync(ctx->d_offsets, offsets, ((size_t)nq + 1) * sizeof(uint32_t),
-                              cudaMemcpyHostToDevice, s));
+    const size_t eb = ne * sizeof(float), ob = ((size_t)nq + 1) * sizeof(uint32_t);
+    if (eb + ob <= haru::kStageBytes) {
+      std::memcpy(ctx->stage, events, eb);
+      std::memcpy(ctx->stage + eb, offsets, ob);
+      HARU_CUDA(cudaMemcpyAsync(ctx->d_events, ctx->stage, eb, cudaMemcpyHostToDevice, s));
+      HARU_CUDA(cudaMemcpyAsync(ctx->d_offsets, ctx->stage + eb, ob, cudaMemcpyHostToDevice, s));
+    } else {
+      HARU_CUDA(cudaMemcpyAsync(ctx->d_events, events, eb, cudaMemcpyHostToDevice, s));
+      HARU_CUDA(cudaMemcpyAsync(ctx->d_offsets, offsets, ob, cudaMemcpyHostToDevice, s));
+    }
     d_off = ctx->d_offsets;
     d_ev = ctx->d_events;
     d_cost = ctx->d_cost;
@@ -424,15 +433,27 @@ int batch_call(haru_ctx *ctx, int precision, const float *events, const uint32_t
     ctx->last_status = HARU_OK;
     return HARU_OK;
   }
+  // (the inputs have left the stage before the results, behind them on the stream, enter it)
+  const size_t cb = on_dev ? 0 : (size_t)nq * sizeof(float), jb = on_dev ? 0 : (size_t)nq * sizeof(int64_t);
+  const size_t sb = span ? jb : 0;
+  const bool staged = sizeof(int64_t) + cb + jb + sb <= haru::kStageBytes;
+  int64_t *st64 = reinterpret_cast<int64_t *>(ctx->stage);  // status | columns | starts | costs
+  unsigned char *cols = ctx->stage + sizeof(int64_t);
   if (!on_dev) {
-    HARU_CUDA(cudaMemcpyAsync(out_cost, d_cost, (size_t)nq * sizeof(float), cudaMemcpyDeviceToHost, s));
-    HARU_CUDA(cudaMemcpyAsync(out_col, d_col, (size_t)nq * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    HARU_CUDA(cudaMemcpyAsync(staged ? cols + jb + sb : (void *)out_cost, d_cost, cb, cudaMemcpyDeviceToHost, s));
+    HARU_CUDA(cudaMemcpyAsync(staged ? cols : (void *)out_col, d_col, jb, cudaMemcpyDeviceToHost, s));
     if (span)
-      HARU_CUDA(cudaMemcpyAsync(out_start, d_start, (size_t)nq * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+      HARU_CUDA(cudaMemcpyAsync(staged ? cols + jb : (void *)out_start, d_start, sb, cudaMemcpyDeviceToHost, s));
   }
-  int st = 0;
-  HARU_CUDA(cudaMemcpyAsync(&st, ctx->ws.ints, sizeof(int), cudaMemcpyDeviceToHost, s));
+  HARU_CUDA(cudaMemcpyAsync(st64, ctx->ws.ints, sizeof(int), cudaMemcpyDeviceToHost, s));
   HARU_CUDA(cudaStreamSynchronize(s));
+  int st = 0;
+  std::memcpy(&st, st64, sizeof(st));
+  if (!on_dev && staged) {
+    std::memcpy(out_cost, cols + jb + sb, cb);
+    std::memcpy(out_col, cols, jb);
+    if (span) std::memcpy(out_start, cols + jb, sb);
+  }
   ctx->last_status = st;
   return st;
 }

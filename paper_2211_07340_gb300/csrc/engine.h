@@ -158,6 +158,16 @@ cudaError_t load_event_kernels();
 // its time can be read after every replay.
 cudaError_t record_event(cudaEvent_t e, cudaStream_t s);
 
+// Pinned staging of a host call. A copy from or to pageable memory waits for
+// the stream on the way (about 3 us each beside a batch of 110 us); the inputs
+// of a batch up to kStageBytes, its results up to kStageBytes (87,380 queries,
+// 52,428 with start columns) and its status go through pinned memory instead
+// and are copied by the host: one 250-event query 124.2 -> 111.6 us. Larger
+// transfers stay direct, where the driver's own staging overlaps its copies
+// (4,096 x 250 events, 4 MB in: 7,832 and 7,823 us). The allocation adds about
+// 0.1 ms to haru_create.
+constexpr size_t kStageBytes = 1u << 20;
+
 class Server;  // serve.cu
 void server_destroy(Server *s);
 
@@ -193,6 +203,7 @@ struct haru_ctx {
   int64_t *d_col = nullptr;
   int64_t *d_start = nullptr;
   size_t cap_q = 0;
+  unsigned char *stage = nullptr;  // pinned, kStageBytes: host calls' small inputs, results and status
 
   // raw-signal path (signal.cu): staged samples and offsets, detected events
   int16_t *d_samples = nullptr;
