@@ -31,15 +31,21 @@ namespace {
 constexpr int kSoloTile = 1536;
 
 // Clocks of one step of a strip of 1 .. 16 rows per lane, per warp of its
-// scheduler: with all twelve of the CTA at work (three a scheduler), and how many more on stacked items, with two warps and with
-// one. Measured on GB300, one strip height at a time, 152 CTAs (60,000 columns).
+// scheduler: with all twelve of the CTA at work (three a scheduler), and how
+// many more on stacked items, with two warps and with one. Measured on GB300,
+// one strip height at a time, 152 CTAs (60,000 columns); alone on a scheduler
+// a warp takes 16 (int16) and 9 clocks more there, but CTAs of few warps also
+// tend to be those that change strip heights and fetch instructions anew, and
+// with those figures small uneven batches were cut too finely (ten batches of
+// 141 x 41..424 FP32 events on 29,166 columns: 329 us on average, 272 us with
+// these; 32 x 250 FP32 133 and 141 us).
 struct StepClocks {
   float full[kMaxS], stacked, two, one;
 };
-const StepClocks kStepI16 = {{22.3f, 22.1f, 25.6f, 28.5f, 34.7f, 39.6f, 45.4f, 47.7f, 58.1f, 58.6f, 65.1f, 69.4f,
-                              77.1f, 76.3f, 81.5f, 86.6f}, 2.0f, 5.0f, 23.0f};
-const StepClocks kStepF32 = {{19.9f, 18.4f, 21.0f, 24.4f, 29.4f, 34.3f, 38.5f, 42.7f, 47.7f, 53.0f, 57.8f, 59.8f,
-                              63.8f, 68.9f, 71.9f, 76.8f}, 1.4f, 4.0f, 13.5f};
+const StepClocks kStepI16 = {{18.5f, 18.5f, 22.3f, 26.1f, 32.6f, 36.8f, 41.8f, 46.4f, 51.6f, 56.5f, 61.1f, 66.9f,
+                              71.7f, 74.0f, 79.5f, 84.7f}, 2.0f, 5.0f, 23.0f};
+const StepClocks kStepF32 = {{16.8f, 15.4f, 18.5f, 21.0f, 25.7f, 31.6f, 36.0f, 39.3f, 44.7f, 48.7f, 53.6f, 56.7f,
+                              62.5f, 66.2f, 70.7f, 75.8f}, 1.4f, 4.0f, 13.5f};
 const StepClocks &step_clocks(int precision) {
   return precision == HARU_INT16 ? kStepI16 : kStepF32;
 }

@@ -170,15 +170,20 @@ inline cudaError_t opt_in_smem(K kernel, SmemOptIn &rec, size_t bytes) {
 constexpr int kIntStatus = 0, kIntGroups = 1, kIntItems = 2, kIntFixups = 3, kIntQueue = 4, kIntMaxSeg = 5,
               kIntQueueLarge = 6, kIntAbort = 7, kIntWords = 8;
 
-__host__ __device__ inline int steps_per_chunk(int S) { return S < 8 ? 8 : S + S % 2; }
+// Steps per unrolled chunk of every strip height. The costs alternate between
+// two registers and a lane reads its reference samples up to four at a time,
+// so it is a multiple of four; it spreads the chunk's own work (flush, state
+// and loop tests) and the tracked lane's stores. Clocks of an int16 step with
+// chunks of S steps (8 at least) and of 16, twelve warps an SM: 2 rows 20.2
+// and 17.7, 5 rows 33.4 and 33.2, 9 rows 54.4 and 51.9, 13 rows 71.7 and
+// 70.0, 8 rows 46.9 and 47.1; with four warps 45.1 and 38.7, 70.5 and 61.0
+// (8 rows), 90.2 and 89.1 (13).
+constexpr int kChunk = 16;
 
-// Tile width (columns) for strip height S: a multiple of lcm(U, 4) not above T.
-__host__ __device__ inline int tile_width(int S, int T) {
-  const int U = steps_per_chunk(S);
-  const int g = U % 4 == 0 ? 4 : (U % 2 == 0 ? 2 : 1);
-  const int L = U / g * 4;
-  const int w = (T / L) * L;
-  return w > 0 ? w : L;
+// Tile width (columns): whole chunks, not above T.
+__host__ __device__ inline int tile_width(int T) {
+  const int w = T / kChunk * kChunk;
+  return w > 0 ? w : kChunk;
 }
 
 // Steps a speculative segment runs before its own first step: three strip
@@ -186,40 +191,35 @@ __host__ __device__ inline int tile_width(int S, int T) {
 // it (alignments span fewer columns than rows here; a segment whose start
 // state still differs is recomputed by the fix-up kernel).
 __host__ __device__ inline long warmup_steps(int S) {
-  const int U = steps_per_chunk(S);
-  return (3L * 32 * S + U - 1) / U * U;
+  return (3L * 32 * S + kChunk - 1) / kChunk * kChunk;
 }
 
 // Whole-chunk step count of one sweep of strip height S over N columns.
 __host__ __device__ inline long sweep_steps(int S, long N) {
-  const int U = steps_per_chunk(S);
-  return (N + 32L * S - 1 + U - 1) / U * U;
+  return (N + 32L * S - 1 + kChunk - 1) / kChunk * kChunk;
 }
 
 // Steps of segment `seg` of `nseg`: own steps [t_own, t_end), warm-up from t_start.
 __host__ __device__ inline void seg_bounds(int S, int nseg, int seg, long N, long *t_start, long *t_own,
                                            long *t_end) {
-  const int U = steps_per_chunk(S);
-  const long chunks = sweep_steps(S, N) / U;
-  *t_own = chunks * seg / nseg * U;
-  *t_end = chunks * (seg + 1) / nseg * U;
+  const long chunks = sweep_steps(S, N) / kChunk;
+  *t_own = chunks * seg / nseg * kChunk;
+  *t_end = chunks * (seg + 1) / nseg * kChunk;
   const long w = *t_own - warmup_steps(S);
   *t_start = seg == 0 ? 0 : (w > 0 ? w : 0);
 }
 
-// Steps between two checkpoints of strip height S: `step` rounded up to whole chunks.
-__host__ __device__ inline int checkpoint_steps(int S, int step) {
-  const int U = steps_per_chunk(S);
-  return (step + U - 1) / U * U;
+// Steps between two checkpoints: `step` rounded up to whole chunks.
+__host__ __device__ inline int checkpoint_steps(int step) {
+  return (step + kChunk - 1) / kChunk * kChunk;
 }
 
 // Steps from t_start to where a bundle cut at `at` of `cost` on the schedule's
 // line stops (whole chunks; the same operands give the same cut on both sides).
-__host__ __device__ inline long cut_steps(int S, long t_start, long t_end, long long at, long long cost) {
-  const int U = steps_per_chunk(S);
+__host__ __device__ inline long cut_steps(long t_start, long t_end, long long at, long long cost) {
   if (at <= 0) return 0;
   if (at >= cost) return t_end - t_start;
-  return static_cast<long>(static_cast<double>((t_end - t_start) / U) * (static_cast<double>(at) / cost)) * U;
+  return static_cast<long>(static_cast<double>((t_end - t_start) / kChunk) * (static_cast<double>(at) / cost)) * kChunk;
 }
 
 struct SdtwArgs {

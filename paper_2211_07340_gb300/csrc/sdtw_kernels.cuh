@@ -133,8 +133,8 @@ __device__ __forceinline__ uint32_t imad(uint32_t a, uint32_t b, uint32_t c) {
 // This lane's reference sample of step u of a chunk, read A at a time. The
 // lane's window starts at column t0 - lane * S, a multiple of A (4 when the
 // strip height S is a multiple of 4, 2 when it is even, else 1; the chunk's
-// first step t0 is a multiple of U, which A divides), so every vector load is
-// aligned.
+// first step t0 is a multiple of kChunk, which A divides), so every vector load
+// is aligned.
 template <int S>
 struct LaneWindow {
   static constexpr int A = S % 4 == 0 ? 4 : (S % 2 == 0 ? 2 : 1);
@@ -155,33 +155,16 @@ struct LaneWindow {
 };
 
 // The tracked lane's last-row value of step u goes to ring[e0 + u]. Values
-// are held for four steps (two when U is not a multiple of four; U is always
-// even) and written by one vector store: e0 is a multiple of U and the ring
-// is 16-byte aligned, so every store is aligned. The FP32 strips use it; the
-// int16 strip stores every step, which measured faster there (the held
-// values must be moved into consecutive registers).
-template <int U>
+// are held for four steps and written by one vector store: e0 is a multiple
+// of kChunk and the ring is 16-byte aligned, so every store is aligned. The
+// FP32 strips use it; the int16 strip stores every two steps, which measured
+// faster there (the held values must be moved into consecutive registers).
 struct RingStore {
-  static constexpr int W = U % 4 == 0 ? 4 : 2;
-  uint32_t v[W];
+  uint32_t v[4];
   __device__ __forceinline__ void put(uint32_t *ring, int e0, int u, bool tracked, uint32_t x) {
-    v[u % W] = x;
-    if (u % W == W - 1 && tracked) {
-      if constexpr (W == 4)
-        *reinterpret_cast<uint4 *>(ring + e0 + u - 3) = make_uint4(v[0], v[1], v[2], v[3]);
-      else
-        *reinterpret_cast<uint2 *>(ring + e0 + u - 1) = make_uint2(v[0], v[1]);
-    }
+    v[u % 4] = x;
+    if (u % 4 == 3 && tracked) *reinterpret_cast<uint4 *>(ring + e0 + u - 3) = make_uint4(v[0], v[1], v[2], v[3]);
   }
-};
-
-template <int S>
-struct Geo {
-  // Steps per unrolled chunk, the period of the register renaming: the
-  // reference samples rotate through U registers and the costs alternate
-  // between two, so U is S rounded up to even; at least 8, to spread the
-  // chunk's own work (flush and segment checks) over the steps of low strips.
-  static constexpr int U = S < 8 ? 8 : S + S % 2;
 };
 
 // ---------------------------------------------------------------- INT16 --
@@ -216,7 +199,7 @@ __device__ __forceinline__ uint32_t half_diff(uint32_t q, uint32_t r) {
 // of the row above the lane.
 template <int S>
 struct StateI16 {
-  uint32_t G[2][S], Rr[Geo<S>::U];
+  uint32_t G[2][S], Rr[kChunk];
   uint32_t gprev;
 
   // As if the reference began at the current step: every row, pad rows
@@ -234,7 +217,7 @@ struct StateI16 {
       G[1][k] = kCap2;
     }
 #pragma unroll
-    for (int k = 0; k < Geo<S>::U; ++k) Rr[k] = 0u;
+    for (int k = 0; k < kChunk; ++k) Rr[k] = 0u;
     gprev = ng ? kCap2 : 0u;
   }
   // Exact state before step t: G[1] = step t-1, G[0] = step t-2, and the
@@ -244,7 +227,7 @@ struct StateI16 {
     for (int k = 0; k < S; ++k) {
       G[1][k] = __ldcg(st + k * 32 + lane);
       G[0][k] = __ldcg(st + (S + k) * 32 + lane);
-      Rr[(1 + k) % Geo<S>::U] = gref[t - 1 - static_cast<long>(lane) * S - k];
+      Rr[(1 + k) % kChunk] = gref[t - 1 - static_cast<long>(lane) * S - k];
     }
     const uint32_t g = __shfl_up_sync(kFull, G[0][S - 1], 1);
     gprev = ng ? g : 0u;
@@ -257,7 +240,7 @@ struct StateI16 {
     }
   }
 
-  // One chunk of U steps; dist(k, r) is row k's distance to the sample r.
+  // One chunk of kChunk steps; dist(k, r) is row k's distance to the sample r.
   // A step's distances, minima and sums are three passes over the rows, and
   // neighbouring rows name the value they share (G[a][k - 1]: `up` of row k,
   // `left` of row k - 1) in the same operand place: the cell is bound by
@@ -266,11 +249,10 @@ struct StateI16 {
   template <int RUN, class Dist>
   __device__ __forceinline__ void steps(const uint32_t *ref, uint32_t *ring, int e0, uint32_t ng, bool tracked,
                                         const Dist &dist) {
-    constexpr int U = Geo<S>::U;
     LaneWindow<S> win;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int p = (U - u) % U;
+    for (int u = 0; u < kChunk; ++u) {
+      const int p = (kChunk - u) % kChunk;
       const int a = (u + 1) & 1;
       const int b = u & 1;
       uint32_t gup = __shfl_up_sync(kFull, G[a][S - 1], 1);
@@ -283,7 +265,7 @@ struct StateI16 {
       Rr[p] = win.get(ref, u);  // row 0's reference: column t - lane * S
       uint32_t d[S], m[S];
 #pragma unroll
-      for (int k = S - 1; k >= 0; --k) d[k] = dist(k, Rr[(p + k) % U]);
+      for (int k = S - 1; k >= 0; --k) d[k] = dist(k, Rr[(p + k) % kChunk]);
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) {
         const uint32_t up = k ? G[a][k - 1] : gup;
@@ -295,7 +277,7 @@ struct StateI16 {
         G[b][k] = (S - 1 - k) % RUN == 0 ? __viaddmin_u16x2(d[k], m[k], kCap2) : m[k] + d[k];
       gprev = gup;
       // The last row's values of steps u - 1 and u sit in G[0] and G[1]: one
-      // 8-byte store every two steps (U is even, the ring 16-byte aligned).
+      // 8-byte store every two steps (the ring is 16-byte aligned).
       if ((u & 1) && tracked)
         *reinterpret_cast<uint2 *>(ring + e0 + u - 1) = make_uint2(G[0][S - 1], G[1][S - 1]);
     }
@@ -344,15 +326,33 @@ struct StripI16Large : StateI16<S> {
   }
 };
 
+// A tracker holds its best value's column as a 32-bit offset from a base that
+// moves with the tiles, and in full when the base moves: references may have
+// more than 2^31 columns, and a 64-bit column costs the scan two selects and
+// three compares an entry.
+constexpr int kNoOffset = -0x7fffffff - 1;
+template <int E>  // E ring entries, read at once
+struct Entries;
+template <>
+struct Entries<2> { using T = uint2; };
+template <>
+struct Entries<4> { using T = uint4; };
+
 struct TrackI16 {
   int ba = 0x7fffffff, bb = 0x7fffffff;
-  long ca = -1, cb = -1;
-  __device__ __forceinline__ void add(const uint32_t *rg, int j, long c) {
-    const uint32_t v = rg[j];
+  int ra = kNoOffset, rb = kNoOffset;
+  long ca = -1, cb = -1, base = 0;
+  __device__ __forceinline__ void rebase(long to) {
+    if (ra != kNoOffset) ca = base + ra;
+    if (rb != kNoOffset) cb = base + rb;
+    ra = rb = kNoOffset;
+    base = to;
+  }
+  __device__ __forceinline__ void add(uint32_t v, const uint32_t *, int rel, bool in) {
     const int va = static_cast<int>(v & 0xffffu);
     const int vb = static_cast<int>(v >> 16);
-    if (va < ba) { ba = va; ca = c; }
-    if (vb < bb) { bb = vb; cb = c; }
+    if (in && va < ba) { ba = va; ra = rel; }
+    if (in && vb < bb) { bb = vb; rb = rel; }
   }
   __device__ __forceinline__ void reduce(int width) {  // over aligned groups of `width` lanes
     for (int o = width >> 1; o > 0; o >>= 1) {
@@ -374,7 +374,7 @@ struct TrackI16 {
 // int16 arithmetic, run through the FP32 units (see FormOf below).
 template <int S, bool CODES>
 struct StripF32 {
-  float Q[S], W[S], G[2][S], Rr[Geo<S>::U];
+  float Q[S], W[S], G[2][S], Rr[kChunk];
   float gprev;
 
   __device__ __forceinline__ static float ref_value(uint32_t w) {
@@ -405,7 +405,7 @@ struct StripF32 {
       G[1][k] = kBig;
     }
 #pragma unroll
-    for (int k = 0; k < Geo<S>::U; ++k) Rr[k] = 0.0f;
+    for (int k = 0; k < kChunk; ++k) Rr[k] = 0.0f;
     gprev = ng ? kBig : 0.0f;
   }
   __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, uint32_t ng) {
@@ -413,7 +413,7 @@ struct StripF32 {
     for (int k = 0; k < S; ++k) {
       G[1][k] = __uint_as_float(__ldcg(st + k * 32 + lane));
       G[0][k] = __uint_as_float(__ldcg(st + (S + k) * 32 + lane));
-      Rr[(1 + k) % Geo<S>::U] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
+      Rr[(1 + k) % kChunk] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
     }
     const float g = __shfl_up_sync(kFull, G[0][S - 1], 1);
     gprev = ng ? g : 0.0f;
@@ -428,12 +428,11 @@ struct StripF32 {
 
   __device__ __forceinline__ void chunk(const uint32_t *ref, int lane, uint32_t *ring, int e0, uint32_t ng,
                                         bool tracked, int, int) {
-    constexpr int U = Geo<S>::U;
     LaneWindow<S> win;
-    RingStore<U> out;
+    RingStore out;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int p = (U - u) % U;
+    for (int u = 0; u < kChunk; ++u) {
+      const int p = (kChunk - u) % kChunk;
       const int a = (u + 1) & 1;
       const int b = u & 1;
       float gup = __shfl_up_sync(kFull, G[a][S - 1], 1);
@@ -444,7 +443,7 @@ struct StripF32 {
       Rr[p] = ref_value(win.get(ref, u));  // row 0's reference: column t - lane * S
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) {
-        const float r = Rr[(p + k) % U];
+        const float r = Rr[(p + k) % kChunk];
         // q - r rounded once on real rows (weight -1), exactly 0 on pad rows
         // (weight 0, q = 0); off the critical path, so the cost update that
         // depends on the minimum is a plain add
@@ -463,11 +462,17 @@ struct StripF32 {
 
 struct TrackF32 {
   float best;
-  long col;
-  __device__ TrackF32() : best(__builtin_huge_valf()), col(-1) {}
-  __device__ __forceinline__ void add(const uint32_t *rg, int j, long c) {
-    const float f = __uint_as_float(rg[j]);
-    if (f < best) { best = f; col = c; }
+  int rel_best = kNoOffset;
+  long col = -1, base = 0;
+  __device__ TrackF32() : best(__builtin_huge_valf()) {}
+  __device__ __forceinline__ void rebase(long to) {
+    if (rel_best != kNoOffset) col = base + rel_best;
+    rel_best = kNoOffset;
+    base = to;
+  }
+  __device__ __forceinline__ void add(uint32_t v, const uint32_t *, int rel, bool in) {
+    const float f = __uint_as_float(v);
+    if (in && f < best) { best = f; rel_best = rel; }
   }
   __device__ __forceinline__ void reduce(int width) {  // over aligned groups of `width` lanes
     for (int o = width >> 1; o > 0; o >>= 1) {
@@ -497,7 +502,7 @@ struct TrackF32 {
 constexpr int kUnknownStart = -2147483647 - 1;
 template <int S, bool CODES>
 struct StripF32Span {
-  float Q[S], W[S], G[2][S], Rr[Geo<S>::U];
+  float Q[S], W[S], G[2][S], Rr[kChunk];
   int P[2][S];
   float gprev;
   int pprev;
@@ -532,7 +537,7 @@ struct StripF32Span {
       P[0][k] = static_cast<int>(t_start) - 2 - i;
     }
 #pragma unroll
-    for (int k = 0; k < Geo<S>::U; ++k) Rr[k] = 0.0f;
+    for (int k = 0; k < kChunk; ++k) Rr[k] = 0.0f;
     gprev = ng ? kBig : 0.0f;
     pprev = static_cast<int>(t_start) - 1 - lane * S;  // the row above row 0 at step t_start - 2
   }
@@ -544,7 +549,7 @@ struct StripF32Span {
       G[0][k] = __uint_as_float(__ldcg(st + (S + k) * 32 + lane));
       P[1][k] = static_cast<int>(__ldcg(st + (2 * S + k) * 32 + lane));
       P[0][k] = static_cast<int>(__ldcg(st + (3 * S + k) * 32 + lane));
-      Rr[(1 + k) % Geo<S>::U] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
+      Rr[(1 + k) % kChunk] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
     }
     const float g = __shfl_up_sync(kFull, G[0][S - 1], 1);
     const int pg = __shfl_up_sync(kFull, P[0][S - 1], 1);
@@ -561,7 +566,7 @@ struct StripF32Span {
       G[0][k] = __uint_as_float(__ldcg(st + (S + k) * 32 + lane));
       P[1][k] = kUnknownStart;
       P[0][k] = kUnknownStart;
-      Rr[(1 + k) % Geo<S>::U] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
+      Rr[(1 + k) % kChunk] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
     }
     const float g = __shfl_up_sync(kFull, G[0][S - 1], 1);
     gprev = ng ? g : 0.0f;
@@ -582,11 +587,10 @@ struct StripF32Span {
   // columns sit 128 words after the costs.
   __device__ __forceinline__ void chunk(const uint32_t *ref, int lane, uint32_t *ring, int e0, uint32_t ng,
                                         bool tracked, int t0, int top) {
-    constexpr int U = Geo<S>::U;
     LaneWindow<S> win;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int p = (U - u) % U;
+    for (int u = 0; u < kChunk; ++u) {
+      const int p = (kChunk - u) % kChunk;
       const int a = (u + 1) & 1;
       const int b = u & 1;
       float gup = __shfl_up_sync(kFull, G[a][S - 1], 1);
@@ -596,7 +600,7 @@ struct StripF32Span {
       Rr[p] = ref_value(win.get(ref, u));  // row 0's reference: column t - lane * S
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) {
-        const float r = Rr[(p + k) % U];
+        const float r = Rr[(p + k) % kChunk];
         const float d = __fmaf_rn(r, W[k], Q[k]);  // q - r on real rows, 0 on pad rows
         const float up = k ? G[a][k - 1] : gup;
         const int pu = k ? P[a][k - 1] : pup;
@@ -619,12 +623,18 @@ struct StripF32Span {
 
 struct TrackF32Span {
   float best;
-  long col;
-  int start;
-  __device__ TrackF32Span() : best(__builtin_huge_valf()), col(-1), start(-1) {}
-  __device__ __forceinline__ void add(const uint32_t *rg, int j, long c) {
-    const float f = __uint_as_float(rg[j]);
-    if (f < best) { best = f; col = c; start = static_cast<int>(rg[2 * flush_words(kPrecF32Span) + j]); }
+  int rel_best = kNoOffset;
+  long col = -1, base = 0;
+  int start = -1;
+  __device__ TrackF32Span() : best(__builtin_huge_valf()) {}
+  __device__ __forceinline__ void rebase(long to) {
+    if (rel_best != kNoOffset) col = base + rel_best;
+    rel_best = kNoOffset;
+    base = to;
+  }
+  __device__ __forceinline__ void add(uint32_t v, const uint32_t *entry, int rel, bool in) {
+    const float f = __uint_as_float(v);
+    if (in && f < best) { best = f; rel_best = rel; start = static_cast<int>(entry[2 * flush_words(kPrecF32Span)]); }
   }
   __device__ __forceinline__ void reduce(int width) {  // over aligned groups of `width` lanes
     for (int o = width >> 1; o > 0; o >>= 1) {
@@ -787,7 +797,10 @@ struct GlobalTiles {
 // flush_words() words, each filled by the strip's tracked lane between two
 // scans (or half by each stack's, the lower stack's at +W/2); forms that
 // carry start columns keep them 2W further on. Each flush scans W/32
-// entries per lane.
+// neighbouring entries per lane, one vector load, against the range of
+// columns that count: with 64-bit columns and a load, a bounds test and
+// a branch per entry 8,192 uneven queries took 11.84 (int16) and 20.06 ms
+// (FP32), so 11.44 and 19.64 (at the same schedule).
 // Returns false on abort.
 // With checkpoints (A.checkpoints, cost forms) the state before every
 // checkpoint step of the own range is stored too.
@@ -797,12 +810,11 @@ __device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>:
                           uint32_t *ring, int lane, bool stk) {
   constexpr bool kCheckpoints = FORM == kFormF32 || FORM == kFormExactWide;
   const long N = A.N;
-  constexpr int U = Geo<S>::U;
   constexpr int W = flush_words(form_i16(FORM) ? HARU_INT16 : HARU_FP32);
   // chunks between two flushes: a stack's entries fill its share of a buffer
-  constexpr int kWhole = W / U > 0 ? W / U : 1;
-  constexpr int kHalf = W / 2 / U > 0 ? W / 2 / U : 1;
-  constexpr int nscan = W / 32;
+  constexpr int kWhole = W / kChunk, kHalf = W / 2 / kChunk;
+  static_assert(kHalf > 0 && kChunk % 4 == 0, "whole chunks, vector stores");
+  constexpr int E = W / 32;  // entries of a lane's scan
   const int F = stk ? kHalf : kWhole;
   // ng: 0 on a lane that starts a stack from the free-start row
   const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
@@ -813,7 +825,7 @@ __device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>:
   const long k_first = t_start / TS;
   const int K = static_cast<int>((t_end + TS - 1) / TS - k_first);
   int fl = 0, buf = 0;
-  long tflush = t_start;
+  const long first_col = t_own > last_row ? t_own - last_row : 0;
   for (int k = 0; k < K; ++k) {
     const uint32_t *tile = src.acquire(k);
     if (!tile) return false;
@@ -824,6 +836,13 @@ __device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>:
     const int n = static_cast<int>(hi - lo);
     const int own_at = (save_start && t_own >= lo && t_own < hi) ? static_cast<int>(t_own - lo) : -1;
     const bool last_tile = t_end <= tk0 + TS;
+    // columns as offsets from that of step lo: the buffer's first, the first and the end of those that count
+    const long base = lo - last_row;
+    tr.rebase(base);
+    int fcol = -fl * kChunk;
+    const long far = 1L << 30;
+    const int col_lo = static_cast<int>(min(max(first_col - base, -far), far));
+    const int col_hi = static_cast<int>(min(max(N - base, -far), far));
     // this lane's reference window of the chunk at o: columns from
     // lo + o - lane * S, found at (column - tk0 + kRefFront) in the slot;
     // lane * S <= 31 * kMaxS <= kRefFront keeps it inside the slot
@@ -833,7 +852,7 @@ __device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>:
       int at = own_at >= from ? own_at : n;
       if constexpr (kCheckpoints) {
         if (A.checkpoints) {
-          const long D = checkpoint_steps(S, A.checkpoint_step);
+          const long D = checkpoint_steps(A.checkpoint_step);
           const long first = lo + from > t_own ? lo + from : t_own;
           const long c = (first + D - 1) / D * D - lo;
           if (c < at) at = static_cast<int>(c);
@@ -842,33 +861,34 @@ __device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>:
       return at;
     };
     int save_at = next_save(0);
-    for (int o = 0; o < n; o += U) {
+    for (int o = 0; o < n; o += kChunk) {
       if (o == save_at) {
         if (o == own_at) st.save(save_start, lane);
         if constexpr (kCheckpoints) {
           if (A.checkpoints) {
-            const int D = checkpoint_steps(S, A.checkpoint_step);
+            const int D = checkpoint_steps(A.checkpoint_step);
             const long c = (lo + o) / D;  // (checkpoint 0 is the fresh start)
             if (c * D == lo + o && lo + o >= t_own && c > 0 && c <= A.checkpoint_cap)
               st.save(A.checkpoints + (static_cast<size_t>(item) * A.checkpoint_cap + (c - 1)) * kStateStride, lane);
           }
         }
-        save_at = next_save(o + U);
+        save_at = next_save(o + kChunk);
       }
       uint32_t *rg = ring + buf * W + soff;
       const int tabs = static_cast<int>(lo) + o;
-      st.chunk(tref + o, lane, rg, fl * U, ng, tracked, tabs, top);
-      if (++fl == F || (last_tile && o + U >= n)) {
+      st.chunk(tref + o, lane, rg, fl * kChunk, ng, tracked, tabs, top);
+      if (++fl == F || (last_tile && o + kChunk >= n)) {
         __syncwarp();
-        for (int r = 0; r < nscan; ++r) {  // entry j = step tflush + j of this lane's stack
-          const int j = stk ? (lane & 15) + 16 * r : lane + 32 * r;
-          if (j < fl * U) {
-            const long t = tflush + j;
-            const long c = t - last_row;
-            if (t >= t_own && c >= 0 && c < N) tr.add(rg, j, c);
-          }
-        }
-        tflush += static_cast<long>(fl) * U;
+        // entry j of the buffer: column fcol + j of this lane's stack
+        const int j0 = (stk ? lane & 15 : lane) * E, hi_col = min(col_hi, fcol + fl * kChunk);
+        const unsigned ncol = static_cast<unsigned>(max(hi_col - col_lo, 0));
+        const typename Entries<E>::T v = *reinterpret_cast<const typename Entries<E>::T *>(rg + j0);
+        const int rel = fcol + j0;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          tr.add(reinterpret_cast<const uint32_t *>(&v)[e], rg + j0 + e, rel + e,
+                 static_cast<unsigned>(rel + e - col_lo) < ncol);
+        fcol += fl * kChunk;
         fl = 0;
         buf ^= 1;
       }
@@ -876,6 +896,7 @@ __device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>:
     __syncwarp();
     if (lane == 0) src.release(k);
   }
+  tr.rebase(0);
   if (save_final) st.save(save_final, lane);
   return true;
 }
@@ -1015,7 +1036,7 @@ template <int PREC>
 __device__ __forceinline__ TileStream stream_of(const SdtwArgs &A, Shared *sh, int stream, int S, long p_lo, long p_hi,
                                                 int n_active) {
   char *slots = reinterpret_cast<char *>(sh) + kSharedHeader + A.warps * ring_words(PREC) * 4;
-  const int TS = tile_width(S, A.tile_cols);
+  const int TS = tile_width(A.tile_cols);
   TileStream ts;
   ts.sh = &sh->streams[stream];
   ts.abort = &sh->abort;
@@ -1152,8 +1173,8 @@ __global__ void __launch_bounds__(cta_threads<PREC>(), 1) sdtw_kernel(SdtwArgs A
     }
     long t_start, t_own, t_end;
     seg_bounds(S, nseg, seg, A.N, &t_start, &t_own, &t_end);
-    const long p_lo = t_start + cut_steps(S, t_start, t_end, cut_lo, cost);
-    const long p_hi = t_start + cut_steps(S, t_start, t_end, cut_hi, cost);
+    const long p_lo = t_start + cut_steps(t_start, t_end, cut_lo, cost);
+    const long p_hi = t_start + cut_steps(t_start, t_end, cut_hi, cost);
     if (waits) {
       // the CTA placed before this one ran its part of the bundle first (a step takes well under 1 us)
       if (threadIdx.x == 0)
@@ -1240,7 +1261,7 @@ __device__ void recompute_segments(const SdtwArgs &A, int item, uint32_t *ring, 
   const bool stk = it.stacked != 0;
   const uint32_t *ref = static_cast<const uint32_t *>(FORM == kFormI16Large ? A.ref_large : A.ref_img);
   const size_t base = static_cast<size_t>(item) * A.nseg_cap;
-  const int TS = tile_width(S, A.tile_cols);
+  const int TS = tile_width(A.tile_cols);
   const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
   constexpr size_t kWords = state_rows_per_s<FORM>() * 16 * 32;
   typename FormOf<FORM, S>::Strip st;
@@ -1410,9 +1431,13 @@ __global__ void __launch_bounds__(kFixWarps * 32) fixup_kernel(SdtwArgs A) {
 // starts carried through the sweep, 1.9 ms this way.)
 struct TrackAt {
   long want;  // the end column on the lanes of the query's stack, -1 on the others
-  int start = kUnknownStart;
-  __device__ __forceinline__ void add(const uint32_t *rg, int j, long c) {
-    if (c == want) start = static_cast<int>(rg[2 * flush_words(kPrecF32Span) + j]);
+  int want_rel = kNoOffset, start = kUnknownStart;
+  __device__ __forceinline__ void rebase(long to) {
+    const long d = want - to;
+    want_rel = d > kNoOffset && d < 0x7fffffff ? static_cast<int>(d) : kNoOffset;
+  }
+  __device__ __forceinline__ void add(uint32_t, const uint32_t *entry, int rel, bool in) {
+    if (in && rel == want_rel) start = static_cast<int>(entry[2 * flush_words(kPrecF32Span)]);
   }
 };
 
@@ -1424,10 +1449,9 @@ __device__ void trace_query(const SdtwArgs &A, int item, int q, bool lower, uint
   const long end = A.out_col[q];
   int start = -1;
   if (end >= 0) {
-    constexpr int U = Geo<S>::U;
-    const int TS = tile_width(S, 4096), D = checkpoint_steps(S, A.checkpoint_step);
+    const int TS = tile_width(4096), D = checkpoint_steps(A.checkpoint_step);
     const int rows = stk ? 16 * S : 32 * S;
-    const long t_last = end + (stk && !lower ? 16L : 32L) * S - 1, t_end = (t_last + U) / U * U;
+    const long t_last = end + (stk && !lower ? 16L : 32L) * S - 1, t_end = (t_last + kChunk) / kChunk * kChunk;
     const long back = t_last - 2 * rows - 32;
     typename FormOf<FORM, S>::Strip st;
     st.load(A.img + static_cast<size_t>(item) * kImgStride, lane);
