@@ -86,12 +86,11 @@ def dram_rate(traffic, cells: float, gcups: float) -> dict:
 def alu_peak_gcups(sms: int, clock_mhz: float, form: str = "int16") -> float:
     """Peak cell rate of the sweep at the given SM clock, from pipe rates.
 
-    int16: one packed cell pair takes 4 instructions, 2 on the half-rate
-    min/DPX pipe (|q - r| by viaddmax_relu, vimin3) and 2 on the other
-    half-rate integer pipe (vsub2, and vadd2 on rows that do not saturate;
-    the saturating rows' viaddmin is charged to the first pipe and is left
-    out of this minimum): 2 warp-instructions/clk/SM per pipe and 4
-    issued/clk/SM both give 64 cells/clk/SM. FP32: 3 instructions per cell
+    int16: one packed cell pair takes 4 instructions (|q - r| by an f16x2
+    subtraction and a mask, vimin3, add; the saturating rows' viaddmin is
+    left out of this minimum): 4 warp-instructions issued/clk/SM give 64
+    cells/clk/SM, and the half-rate min pipe takes one of the four.
+    FP32: 3 instructions per cell
     (the distance fma, 3-input min, add) at one warp-instruction per clock
     per scheduler:
     128 / 3 = 42.7 cells/clk/SM.
@@ -761,8 +760,8 @@ def main():
                      "unit": "GCUPS", "frac": ach16 / peak, "traffic": profiled_traffic("int16"),
                      "traffic_unit": "bytes per batch (DRAM read+write, ncu at the default launch shape, "
                                      "profiles/sdtw_sweep_sars_uneven_8192.md)",
-                     "peak_basis": f"{sms} SMs x 64 cells/clk/SM (4 instructions per packed cell pair, 2 on "
-                                   f"each half-rate integer pipe) x {max_mhz:.0f} MHz max SM clock",
+                     "peak_basis": f"{sms} SMs x 64 cells/clk/SM (4 instructions per packed cell pair, 4 "
+                                   f"issued per clock) x {max_mhz:.0f} MHz max SM clock",
                      "frac_at_sampled_clock": (ach16 / alu_peak_gcups(sms, clocks["sm_mhz"], "int16"))
                      if clocks.get("sm_mhz") else None,
                      "peak_probe": probe16, "frac_of_probe": ach16 / probe16,

@@ -443,7 +443,7 @@ int haru_autotune(haru_ctx *ctx, int precision, const float *events, const uint3
                   uint32_t flags, haru_config *chosen);
 
 /* Measured ceiling of the cell update: the per-cell instructions of the
- * given form (int16: vsub2, viaddmax_relu, vimin3, viaddmin per two cells;
+ * given form (int16: f16x2 sub, and, vimin3, add per two cells, one row in eight viaddmin;
  * FP32: sub, 3-input min, fma per cell) issued on independent chains over
  * every SM, with none of the wavefront's data movement. *cells_per_s is the
  * best of three runs at the clock the GPU ran them. Errors: HARU_EINVAL,

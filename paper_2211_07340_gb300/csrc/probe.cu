@@ -12,6 +12,11 @@ namespace {
 constexpr int kChains = 8;
 constexpr int kLevels = 4;
 
+__device__ __forceinline__ uint32_t half_diff(uint32_t q, uint32_t r) {
+  uint32_t d;
+  asm volatile("sub.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(q), "r"(r));
+  return d;
+}
 __device__ __forceinline__ float fmin3p(float a, float b, float c) {
   float d;
   asm volatile("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -41,9 +46,9 @@ __global__ void probe_kernel(uint32_t *out, int iters) {
       for (int i = 0; i < kChains; ++i) {
         const int j = (i + 1) % kChains, k = (i + 3) % kChains;
         if (PREC == HARU_INT16) {
-          const uint32_t d = __viaddmax_s16x2_relu(x[i], a[k], __vsub2(x[j], x[i]));
+          const uint32_t d = half_diff(x[i], x[j]) & 0x07ff07ffu;
           const uint32_t m = __vimin3_u16x2(a[i], a[j], a[k]);
-          an[i] = i == 0 ? __viaddmin_u16x2(d, m, x[k]) : __vadd2(m, d);  // one row in eight saturates
+          an[i] = i == 0 ? __viaddmin_u16x2(d, m, x[k]) : m + d;  // one row in eight saturates
           xn[i] = d;
         } else {
           const float t = __fsub_rn(g[i], g[j]);

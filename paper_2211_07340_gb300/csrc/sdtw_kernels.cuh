@@ -1428,7 +1428,7 @@ __global__ void __launch_bounds__(kFixWarps * 32) fixup_kernel(SdtwArgs A) {
 // cell's is unknown only if its alignment began before the checkpoint: then
 // the strip runs again from an earlier one, at last from the fresh start.
 // (512 uneven FP32 queries on 59,796 columns: the whole call 4.1 ms with the
-// starts carried through the sweep, 1.9 ms this way.)
+// starts carried through the sweep, 1.6 ms this way.)
 struct TrackAt {
   long want;  // the end column on the lanes of the query's stack, -1 on the others
   int want_rel = kNoOffset, start = kUnknownStart;
