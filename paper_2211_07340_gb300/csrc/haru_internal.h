@@ -214,6 +214,15 @@ __host__ __device__ inline int checkpoint_steps(int step) {
   return (step + kChunk - 1) / kChunk * kChunk;
 }
 
+// The end column a trace of start columns runs to, given a query's result:
+// -1 (no trace) for none, for one that is not a column of the reference, and
+// for every query of a batch that gave up on a device wait: units that never
+// ran leave whatever their minima held before, and a trace reads the reference
+// up to its end column.
+__host__ __device__ constexpr long trace_end(int64_t col, long N, int gave_up) {
+  return gave_up || col < 0 || col >= N ? -1 : static_cast<long>(col);
+}
+
 // Steps from t_start to where a bundle cut at `at` of `cost` on the schedule's
 // line stops (whole chunks; the same operands give the same cut on both sides).
 __host__ __device__ inline long cut_steps(long t_start, long t_end, long long at, long long cost) {

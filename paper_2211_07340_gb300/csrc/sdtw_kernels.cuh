@@ -1446,7 +1446,7 @@ __device__ void trace_query(const SdtwArgs &A, int item, int q, bool lower, uint
   const bool stk = A.items[item].stacked != 0;
   const uint32_t *ref = static_cast<const uint32_t *>(A.ref_img);
   const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
-  const long end = A.out_col[q];
+  const long end = trace_end(A.out_col[q], A.N, A.ints[kIntAbort]);
   int start = -1;
   if (end >= 0) {
     const int TS = tile_width(4096), D = checkpoint_steps(A.checkpoint_step);
