@@ -114,6 +114,11 @@ __device__ __forceinline__ float fmin3f(float a, float b, float c) {
   return d;
 }
 
+// This lane's place in its stack: it holds rows place * S .. place * S + S - 1
+// of the stack and lags the warp's step by place * S columns. Both stacks of a
+// stacked strip start at column 0 on step 0.
+__device__ __forceinline__ int stack_place(int lane, bool stk) { return stk ? lane & 15 : lane; }
+
 // x == m ? a : b as a compare and a select (never a branch).
 __device__ __forceinline__ int sel_eq(float x, float m, int a, int b) {
   int d;
@@ -131,7 +136,7 @@ __device__ __forceinline__ uint32_t imad(uint32_t a, uint32_t b, uint32_t c) {
 }
 
 // This lane's reference sample of step u of a chunk, read A at a time. The
-// lane's window starts at column t0 - lane * S, a multiple of A (4 when the
+// lane's window starts at column t0 - place * S, a multiple of A (4 when the
 // strip height S is a multiple of 4, 2 when it is even, else 1; the chunk's
 // first step t0 is a multiple of kChunk, which A divides), so every vector load
 // is aligned.
@@ -210,7 +215,7 @@ struct StateI16 {
   // or above CAP until its first column: infinity under min(CAP, .). No
   // cell is masked; every value is the plain DP's modulo min(CAP, .), which
   // is all the tracked (capped) last row and the segment check look at.
-  __device__ __forceinline__ void fresh(long, int, uint32_t ng) {
+  __device__ __forceinline__ void fresh(long, int place) {
 #pragma unroll
     for (int k = 0; k < S; ++k) {
       G[0][k] = kCap2;
@@ -218,19 +223,19 @@ struct StateI16 {
     }
 #pragma unroll
     for (int k = 0; k < kChunk; ++k) Rr[k] = 0u;
-    gprev = ng ? kCap2 : 0u;
+    gprev = place ? kCap2 : 0u;
   }
   // Exact state before step t: G[1] = step t-1, G[0] = step t-2, and the
   // reference samples the cells used at step t-1 (from the global image).
-  __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, uint32_t ng) {
+  __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, int place) {
 #pragma unroll
     for (int k = 0; k < S; ++k) {
       G[1][k] = __ldcg(st + k * 32 + lane);
       G[0][k] = __ldcg(st + (S + k) * 32 + lane);
-      Rr[(1 + k) % kChunk] = gref[t - 1 - static_cast<long>(lane) * S - k];
+      Rr[(1 + k) % kChunk] = gref[t - 1 - static_cast<long>(place) * S - k];
     }
     const uint32_t g = __shfl_up_sync(kFull, G[0][S - 1], 1);
-    gprev = ng ? g : 0u;
+    gprev = place ? g : 0u;
   }
   __device__ __forceinline__ void save(uint32_t *st, int lane) const {
 #pragma unroll
@@ -262,7 +267,7 @@ struct StateI16 {
       // previous value, 0, is in the minimum), so only full-height strips
       // put the zero in.
       if constexpr (S == kMaxS) gup = imad(gup, ng, 0u);
-      Rr[p] = win.get(ref, u);  // row 0's reference: column t - lane * S
+      Rr[p] = win.get(ref, u);  // row 0's reference: column t - place * S
       uint32_t d[S], m[S];
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) d[k] = dist(k, Rr[(p + k) % kChunk]);
@@ -295,7 +300,7 @@ struct StripI16 : StateI16<S> {
     for (int k = 0; k < S; ++k) Q[k] = img[k * 32 + lane];
   }
   __device__ __forceinline__ void chunk(const uint32_t *ref, int, uint32_t *ring, int e0, uint32_t ng, bool tracked,
-                                        int, int) {
+                                        int) {
     this->template steps<kCapRunHalf>(ref, ring, e0, ng, tracked, [this](int k, uint32_t r) {
       return half_diff(Q[k], r) & 0x07ff07ffu;  // the low 11 bits: |q - r|; pad rows (2^15 - r = 2^15): 0
     });
@@ -319,7 +324,7 @@ struct StripI16Large : StateI16<S> {
     }
   }
   __device__ __forceinline__ void chunk(const uint32_t *ref, int, uint32_t *ring, int e0, uint32_t ng, bool tracked,
-                                        int, int) {
+                                        int) {
     this->template steps<kCapRunLarge>(ref, ring, e0, ng, tracked, [this](int k, uint32_t r) {
       return __viaddmax_s16x2_relu(r, NQ[k], __vsub2(Q[k], r));  // |q - r| per half
     });
@@ -397,7 +402,7 @@ struct StripF32 {
   // step back. The top row turns 0 at step 0, each pad row below at its own
   // first column, and a real row stays at kBig or above until its first
   // column whatever reference samples its lane reads before the start.
-  __device__ __forceinline__ void fresh(long, int, uint32_t ng) {
+  __device__ __forceinline__ void fresh(long, int place) {
     const float kBig = 1.0e30f;
 #pragma unroll
     for (int k = 0; k < S; ++k) {
@@ -406,17 +411,17 @@ struct StripF32 {
     }
 #pragma unroll
     for (int k = 0; k < kChunk; ++k) Rr[k] = 0.0f;
-    gprev = ng ? kBig : 0.0f;
+    gprev = place ? kBig : 0.0f;
   }
-  __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, uint32_t ng) {
+  __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, int place) {
 #pragma unroll
     for (int k = 0; k < S; ++k) {
       G[1][k] = __uint_as_float(__ldcg(st + k * 32 + lane));
       G[0][k] = __uint_as_float(__ldcg(st + (S + k) * 32 + lane));
-      Rr[(1 + k) % kChunk] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
+      Rr[(1 + k) % kChunk] = ref_value(gref[t - 1 - static_cast<long>(place) * S - k]);
     }
     const float g = __shfl_up_sync(kFull, G[0][S - 1], 1);
-    gprev = ng ? g : 0.0f;
+    gprev = place ? g : 0.0f;
   }
   __device__ __forceinline__ void save(uint32_t *st, int lane) const {
 #pragma unroll
@@ -427,7 +432,7 @@ struct StripF32 {
   }
 
   __device__ __forceinline__ void chunk(const uint32_t *ref, int lane, uint32_t *ring, int e0, uint32_t ng,
-                                        bool tracked, int, int) {
+                                        bool tracked, int) {
     LaneWindow<S> win;
     RingStore out;
 #pragma unroll
@@ -440,7 +445,7 @@ struct StripF32 {
       // the stack (weight 0, value 0) keeps it for strips of fewer than
       // kMaxS rows per lane, as in the int16 strip.
       if constexpr (S == kMaxS) gup = ng ? gup : 0.0f;
-      Rr[p] = ref_value(win.get(ref, u));  // row 0's reference: column t - lane * S
+      Rr[p] = ref_value(win.get(ref, u));  // row 0's reference: column t - place * S
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) {
         const float r = Rr[(p + k) % kChunk];
@@ -523,53 +528,53 @@ struct StripF32Span {
   // As in StripF32: every row starts at kBig and the free-start zero reaches
   // each row at its first column (a stack's top row takes the injected row
   // above it, 0 with the current column, every step), so each pad row passes
-  // down its own column from then on. Before step t_start row i = lane * S +
-  // k held column t_start - 1 - i (t_start - 2 - i one step earlier); those
+  // down its own column from then on. Before step t_start row i = place * S +
+  // k of a stack held column t_start - 1 - i (t_start - 2 - i one step earlier); those
   // starts belong to values at kBig, which no finite cost takes.
-  __device__ __forceinline__ void fresh(long t_start, int lane, uint32_t ng) {
+  __device__ __forceinline__ void fresh(long t_start, int place) {
     const float kBig = 1.0e30f;
 #pragma unroll
     for (int k = 0; k < S; ++k) {
       G[0][k] = kBig;
       G[1][k] = kBig;
-      const int i = lane * S + k;
+      const int i = place * S + k;
       P[1][k] = static_cast<int>(t_start) - 1 - i;
       P[0][k] = static_cast<int>(t_start) - 2 - i;
     }
 #pragma unroll
     for (int k = 0; k < kChunk; ++k) Rr[k] = 0.0f;
-    gprev = ng ? kBig : 0.0f;
-    pprev = static_cast<int>(t_start) - 1 - lane * S;  // the row above row 0 at step t_start - 2
+    gprev = place ? kBig : 0.0f;
+    pprev = static_cast<int>(t_start) - 1 - place * S;  // the row above row 0 at step t_start - 2
   }
   // States hold G (2S rows of 32 words) then P (2S rows).
-  __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, uint32_t ng) {
+  __device__ __forceinline__ void restore(const uint32_t *st, const uint32_t *gref, long t, int lane, int place) {
 #pragma unroll
     for (int k = 0; k < S; ++k) {
       G[1][k] = __uint_as_float(__ldcg(st + k * 32 + lane));
       G[0][k] = __uint_as_float(__ldcg(st + (S + k) * 32 + lane));
       P[1][k] = static_cast<int>(__ldcg(st + (2 * S + k) * 32 + lane));
       P[0][k] = static_cast<int>(__ldcg(st + (3 * S + k) * 32 + lane));
-      Rr[(1 + k) % kChunk] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
+      Rr[(1 + k) % kChunk] = ref_value(gref[t - 1 - static_cast<long>(place) * S - k]);
     }
     const float g = __shfl_up_sync(kFull, G[0][S - 1], 1);
     const int pg = __shfl_up_sync(kFull, P[0][S - 1], 1);
-    gprev = ng ? g : 0.0f;
-    pprev = ng ? pg : static_cast<int>(t) - 1 - lane * S;
+    gprev = place ? g : 0.0f;
+    pprev = place ? pg : static_cast<int>(t) - 1;
   }
   // A cost form's exact state before step t: every start column before it is
   // kUnknownStart; the free-start rows pass known ones down from step t on.
   __device__ __forceinline__ void restore_costs(const uint32_t *st, const uint32_t *gref, long t, int lane,
-                                                uint32_t ng) {
+                                                int place) {
 #pragma unroll
     for (int k = 0; k < S; ++k) {
       G[1][k] = __uint_as_float(__ldcg(st + k * 32 + lane));
       G[0][k] = __uint_as_float(__ldcg(st + (S + k) * 32 + lane));
       P[1][k] = kUnknownStart;
       P[0][k] = kUnknownStart;
-      Rr[(1 + k) % kChunk] = ref_value(gref[t - 1 - static_cast<long>(lane) * S - k]);
+      Rr[(1 + k) % kChunk] = ref_value(gref[t - 1 - static_cast<long>(place) * S - k]);
     }
     const float g = __shfl_up_sync(kFull, G[0][S - 1], 1);
-    gprev = ng ? g : 0.0f;
+    gprev = place ? g : 0.0f;
     pprev = kUnknownStart;
   }
   __device__ __forceinline__ void save(uint32_t *st, int lane) const {
@@ -582,11 +587,10 @@ struct StripF32Span {
     }
   }
 
-  // t0: the absolute step of the chunk's first step; top: the first row of
-  // this lane's stack (0, or 16 * S in the lower stack). The ring's start
-  // columns sit 128 words after the costs.
+  // t0: the absolute step of the chunk's first step. The ring's start columns
+  // sit two flush buffers after the costs.
   __device__ __forceinline__ void chunk(const uint32_t *ref, int lane, uint32_t *ring, int e0, uint32_t ng,
-                                        bool tracked, int t0, int top) {
+                                        bool tracked, int t0) {
     LaneWindow<S> win;
 #pragma unroll
     for (int u = 0; u < kChunk; ++u) {
@@ -596,8 +600,8 @@ struct StripF32Span {
       float gup = __shfl_up_sync(kFull, G[a][S - 1], 1);
       int pup = __shfl_up_sync(kFull, P[a][S - 1], 1);
       gup = ng ? gup : 0.0f;             // a stack's first lane: the free-start row, 0 ...
-      pup = ng ? pup : t0 + u - top;      // ... whose row processed column t - top at step t - 1
-      Rr[p] = ref_value(win.get(ref, u));  // row 0's reference: column t - lane * S
+      pup = ng ? pup : t0 + u;            // ... whose row processed column t at step t - 1
+      Rr[p] = ref_value(win.get(ref, u));  // row 0's reference: column t - place * S
 #pragma unroll
       for (int k = S - 1; k >= 0; --k) {
         const float r = Rr[(p + k) % kChunk];
@@ -816,12 +820,11 @@ __device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>:
   static_assert(kHalf > 0 && kChunk % 4 == 0, "whole chunks, vector stores");
   constexpr int E = W / 32;  // entries of a lane's scan
   const int F = stk ? kHalf : kWhole;
-  // ng: 0 on a lane that starts a stack from the free-start row
-  const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
+  const int place = stack_place(lane, stk);
+  const uint32_t ng = place != 0 ? 1u : 0u;  // 0 on a lane that starts a stack from the free-start row
   const bool tracked = lane == 31 || (stk && lane == 15);
   const int soff = stk && lane >= 16 ? W / 2 : 0;
-  const int top = stk && lane >= 16 ? 16 * S : 0;  // first row of this lane's stack
-  const long last_row = (stk && lane < 16 ? 16L : 32L) * S - 1;
+  const long last_row = (stk ? 16L : 32L) * S - 1;  // of either stack
   const long k_first = t_start / TS;
   const int K = static_cast<int>((t_end + TS - 1) / TS - k_first);
   int fl = 0, buf = 0;
@@ -844,9 +847,9 @@ __device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>:
     const int col_lo = static_cast<int>(min(max(first_col - base, -far), far));
     const int col_hi = static_cast<int>(min(max(N - base, -far), far));
     // this lane's reference window of the chunk at o: columns from
-    // lo + o - lane * S, found at (column - tk0 + kRefFront) in the slot;
-    // lane * S <= 31 * kMaxS <= kRefFront keeps it inside the slot
-    const uint32_t *tref = tile + (kRefFront + (lo - tk0) - static_cast<long>(lane) * S);
+    // lo + o - place * S, found at (column - tk0 + kRefFront) in the slot;
+    // place * S <= 31 * kMaxS <= kRefFront keeps it inside the slot
+    const uint32_t *tref = tile + (kRefFront + (lo - tk0) - static_cast<long>(place) * S);
     // the next step of this tile before which a state is stored
     auto next_save = [&](int from) {
       int at = own_at >= from ? own_at : n;
@@ -876,11 +879,11 @@ __device__ bool run_steps(const SdtwArgs &A, int item, typename FormOf<FORM, S>:
       }
       uint32_t *rg = ring + buf * W + soff;
       const int tabs = static_cast<int>(lo) + o;
-      st.chunk(tref + o, lane, rg, fl * kChunk, ng, tracked, tabs, top);
+      st.chunk(tref + o, lane, rg, fl * kChunk, ng, tracked, tabs);
       if (++fl == F || (last_tile && o + kChunk >= n)) {
         __syncwarp();
         // entry j of the buffer: column fcol + j of this lane's stack
-        const int j0 = (stk ? lane & 15 : lane) * E, hi_col = min(col_hi, fcol + fl * kChunk);
+        const int j0 = place * E, hi_col = min(col_hi, fcol + fl * kChunk);
         const unsigned ncol = static_cast<unsigned>(max(hi_col - col_lo, 0));
         const typename Entries<E>::T v = *reinterpret_cast<const typename Entries<E>::T *>(rg + j0);
         const int rel = fcol + j0;
@@ -932,16 +935,16 @@ __device__ void sweep_unit(const SdtwArgs &A, TileStream &ts, int nseg, int seg,
   const bool stk = A.items[item].stacked != 0;
   // (start-column units are never cut)
   const bool whole = FORM == kFormF32Span || FORM == kFormWideSpan || p_lo == t_start;
-  const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
+  const int place = stack_place(lane, stk);
   const size_t unit = static_cast<size_t>(item) * A.nseg_cap + seg;
   constexpr size_t kWords = state_rows_per_s<FORM>() * 16 * 32;
   uint32_t *ss = nullptr, *sf = nullptr;
   if (seg > 0) ss = A.states + (unit * 2 + 0) * kWords;
   if (seg + 1 < nseg || p_hi < t_end) sf = A.states + (unit * 2 + 1) * kWords;
   if (whole)
-    st.fresh(t_start, lane, ng);
+    st.fresh(t_start, place);
   else
-    st.restore(A.states + (unit * 2 + 1) * kWords, reinterpret_cast<const uint32_t *>(ts.src), p_lo, lane, ng);
+    st.restore(A.states + (unit * 2 + 1) * kWords, reinterpret_cast<const uint32_t *>(ts.src), p_lo, lane, place);
   const bool ok = run_steps<FORM, S>(A, item, st, tr, ts, ts.tile_cols, p_lo, t_own, p_hi, ss, sf, ring, lane, stk);
   tr.reduce(stk ? 16 : 32);
   if (ok && lane == 0) {
@@ -1262,7 +1265,7 @@ __device__ void recompute_segments(const SdtwArgs &A, int item, uint32_t *ring, 
   const uint32_t *ref = static_cast<const uint32_t *>(FORM == kFormI16Large ? A.ref_large : A.ref_img);
   const size_t base = static_cast<size_t>(item) * A.nseg_cap;
   const int TS = tile_width(A.tile_cols);
-  const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
+  const int place = stack_place(lane, stk);
   constexpr size_t kWords = state_rows_per_s<FORM>() * 16 * 32;
   typename FormOf<FORM, S>::Strip st;
   st.load(A.img + static_cast<size_t>(item) * kImgStride, lane);
@@ -1273,7 +1276,7 @@ __device__ void recompute_segments(const SdtwArgs &A, int item, uint32_t *ring, 
     if (!bad) continue;
     long t_start, t_own, t_end;
     seg_bounds(S, nseg, s, A.N, &t_start, &t_own, &t_end);
-    st.restore(A.states + ((base + s - 1) * 2 + 1) * kWords, ref, t_own, lane, ng);
+    st.restore(A.states + ((base + s - 1) * 2 + 1) * kWords, ref, t_own, lane, place);
     typename FormOf<FORM, S>::Track tr;
     GlobalTiles src{ref, TS, t_own / TS};
     uint32_t *sf = s + 1 < nseg ? A.states + ((base + s) * 2 + 1) * kWords : nullptr;
@@ -1445,13 +1448,13 @@ template <int FORM, int S>
 __device__ void trace_query(const SdtwArgs &A, int item, int q, bool lower, uint32_t *ring, int lane) {
   const bool stk = A.items[item].stacked != 0;
   const uint32_t *ref = static_cast<const uint32_t *>(A.ref_img);
-  const uint32_t ng = (stk ? (lane & 15) : lane) != 0 ? 1u : 0u;
+  const int place = stack_place(lane, stk);
   const long end = trace_end(A.out_col[q], A.N, A.ints[kIntAbort]);
   int start = -1;
   if (end >= 0) {
     const int TS = tile_width(4096), D = checkpoint_steps(A.checkpoint_step);
     const int rows = stk ? 16 * S : 32 * S;
-    const long t_last = end + (stk && !lower ? 16L : 32L) * S - 1, t_end = (t_last + kChunk) / kChunk * kChunk;
+    const long t_last = end + rows - 1, t_end = (t_last + kChunk) / kChunk * kChunk;
     const long back = t_last - 2 * rows - 32;
     typename FormOf<FORM, S>::Strip st;
     st.load(A.img + static_cast<size_t>(item) * kImgStride, lane);
@@ -1460,10 +1463,10 @@ __device__ void trace_query(const SdtwArgs &A, int item, int q, bool lower, uint
     for (;;) {
       const long t0 = c * D;
       if (c == 0)
-        st.fresh(0, lane, ng);
+        st.fresh(0, place);
       else
         st.restore_costs(A.checkpoints + (static_cast<size_t>(item) * A.checkpoint_cap + (c - 1)) * kStateStride, ref,
-                         t0, lane, ng);
+                         t0, lane, place);
       TrackAt tr;
       tr.want = !stk || (lane >= 16) == lower ? end : -1;
       GlobalTiles src{ref, TS, t0 / TS};
