@@ -88,7 +88,7 @@ struct RefView {
 // z-scored over their own m events, so |z| <= sqrt(m - 1) < 22.7 for m <= 512
 // (the largest deviation of m values with population sigma 1); 22.7 * 2^k + 1
 // covers the roundings. With a 2^6 scale and a reference within 9 sigma that
-// bound clears every raw batch, and the large-code sweep is not launched.
+// bound clears every raw batch, and the sweep with both cells is not needed.
 inline int large_codes_possible(const RefView &r, int raw) {
   const double bound = raw ? 22.7 * static_cast<double>(1 << r.scale_log2) + 1.0 : static_cast<double>(kQmax);
   return bound > static_cast<double>(kHalfSpan - r.max_code) && kQmax > kHalfSpan - r.max_code ? 1 : 0;

@@ -85,9 +85,14 @@ static_assert(kRefFront >= 31 * kMaxS && kRefFront % 16 == 0, "front pad: the la
 // HARU_INT16 and HARU_INT16_ACC32: the FP32 and wide forms that also carry
 // each alignment's start column (haru_sdtw_batch_span).
 constexpr int kPrecF32Span = 3, kPrecWideSpan = 4;
-// and the int16 form for groups whose codes are too large for the half-code
-// cell (kHalfSpan).
-constexpr int kPrecI16Large = 5;
+// and the int16 form of a batch in which some codes may be too large for the
+// half-code cell (kHalfSpan): its sweep holds both int16 cells and picks one
+// for each bundle or group. 8,192 uneven queries, one of them or 5% with large
+// codes, take 11.2 and 12.4 ms (none: 11.2); with a sweep of its own for the
+// bundles that hold one, run before the half-code sweep on the same schedule,
+// 17.2 and 23.1; with the cell picked for each warp, 11.3 and 22.0 (the code
+// of two strips does not fit the instruction cache).
+constexpr int kPrecI16Mixed = 5;
 __host__ __device__ constexpr bool prec_span(int p) { return p == kPrecF32Span || p == kPrecWideSpan; }
 // Tracking-ring words per warp: costs (and start columns, +128, for the span forms).
 // Words of one flush buffer of a warp's last-row tracking ring: a whole
@@ -96,7 +101,7 @@ __host__ __device__ constexpr bool prec_span(int p) { return p == kPrecF32Span |
 // columns keep two more for the starts. Measured per form on GB300: 64 words
 // for the int16 strips, 128 for the FP32-unit ones (fewer scans; the int16
 // kernel ran 0.5% slower with 128, FP32 2.9% faster).
-__host__ __device__ constexpr int flush_words(int p) { return p == HARU_INT16 || p == kPrecI16Large ? 64 : 128; }
+__host__ __device__ constexpr int flush_words(int p) { return p == HARU_INT16 || p == kPrecI16Mixed ? 64 : 128; }
 __host__ __device__ constexpr int ring_words(int p) { return (prec_span(p) ? 4 : 2) * flush_words(p); }
 // Words of one saved strip state: costs, and start columns for the span forms.
 __host__ __device__ constexpr int state_words(int p) { return prec_span(p) ? 2 * kStateStride : kStateStride; }
@@ -165,10 +170,10 @@ inline cudaError_t opt_in_smem(K kernel, SmemOptIn &rec, size_t bytes) {
 
 // Layout of the small integer block every batch uses: the status word, the
 // planner's group and item counts, the fix-up count, the sweep kernel's work
-// queue counter, the most segments any item was cut into, the queue counter
-// of the large-code int16 sweep, and whether a sweep gave up on a wait.
+// queue counter, the most segments any item was cut into, and whether a sweep
+// gave up on a wait.
 constexpr int kIntStatus = 0, kIntGroups = 1, kIntItems = 2, kIntFixups = 3, kIntQueue = 4, kIntMaxSeg = 5,
-              kIntQueueLarge = 6, kIntAbort = 7, kIntWords = 8;
+              kIntAbort = 6, kIntWords = 7;
 
 // Steps per unrolled chunk of every strip height. The costs alternate between
 // two registers and a lane reads its reference samples up to four at a time,
@@ -234,9 +239,9 @@ __host__ __device__ inline long cut_steps(long t_start, long t_end, long long at
 struct SdtwArgs {
   const void *ref_img;     // INT16: uint32 (h | h << 16), h the half code; integer forms in FP32: (r | r << 16);
                            // FP32: float. Column 0 of N + kRefPad words, kRefFront zero words before it
-  const void *ref_large;   // INT16: uint32 (r | r << 16), for the large-code groups
+  const void *ref_large;   // INT16: uint32 (r | r << 16), for items with large codes
   int half_max;            // INT16: largest query |code| the half-code cell takes (kHalfSpan - the reference's)
-  int large_possible;      // INT16: a group may hold larger codes (its sweep is launched too)
+  int large_possible;      // INT16: an item may hold larger codes (the sweep with both cells is launched)
   long N;                  // reference length (columns)
   const uint32_t *img;     // item images, kImgStride words each
   const Item *items;

@@ -97,23 +97,26 @@ cudaError_t load_sdtw(int precision) {
 // The sweep kernel of the precision (scheduled, or from the queue), then its
 // segment fix-up kernel (which also writes the outputs), stream-ordered;
 // ev_fix (if given) is recorded between the two. An int16 batch that may
-// hold large codes runs the large-code sweep first.
+// hold large codes runs the sweep with both int16 cells.
 cudaError_t launch_sdtw(int precision, const SdtwArgs &a, int grid, int fix_items, cudaStream_t s,
                         cudaEvent_t ev_fix) {
   cudaError_t e;
-#define HARU_SDTW_FIX(P)                                                        \
-  if (e != cudaSuccess) return e;                                               \
-  if (ev_fix && (e = record_event(ev_fix, s)) != cudaSuccess) return e;         \
-  return sdtw_fixup_##P(a, fix_items, s);
-#define HARU_SDTW_BOTH(P)                                                       \
-  e = a.solo ? sdtw_sweep_##P(a, grid, s) : sdtw_queue_##P(a, grid, s);         \
-  HARU_SDTW_FIX(P)
+#define HARU_SDTW_FIX(P)                                                          \
+  {                                                                               \
+    if (e != cudaSuccess) return e;                                               \
+    if (ev_fix && (e = record_event(ev_fix, s)) != cudaSuccess) return e;         \
+    return sdtw_fixup_##P(a, fix_items, s);                                       \
+  }
+#define HARU_SDTW_BOTH(P)                                                         \
+  {                                                                               \
+    e = a.solo ? sdtw_sweep_##P(a, grid, s) : sdtw_queue_##P(a, grid, s);         \
+    HARU_SDTW_FIX(P)                                                              \
+  }
   switch (precision) {
     case HARU_INT16:
-      if (a.large_possible &&
-          (e = a.solo ? sdtw_sweep_5(a, grid, s) : sdtw_queue_5(a, grid, s)) != cudaSuccess)
-        return e;
-      HARU_SDTW_BOTH(1)
+      if (!a.large_possible) HARU_SDTW_BOTH(1)
+      e = a.solo ? sdtw_sweep_5(a, grid, s) : sdtw_queue_5(a, grid, s);
+      HARU_SDTW_FIX(1)
     case HARU_INT16_ACC32: HARU_SDTW_BOTH(2)
     case kPrecF32Span:
       e = sdtw_queue_3(a, grid, s);

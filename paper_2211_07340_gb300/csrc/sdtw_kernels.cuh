@@ -959,7 +959,7 @@ __device__ void sweep_unit(const SdtwArgs &A, TileStream &ts, int nseg, int seg,
 
 template <int PREC, int S>
 __device__ __forceinline__ void sweep_any(const SdtwArgs &A, TileStream &ts, int nseg, int seg, long p_lo,
-                                          long p_hi, int item, uint32_t *ring, int lane) {
+                                          long p_hi, int item, bool large, uint32_t *ring, int lane) {
   if constexpr (PREC == HARU_FP32) {
     sweep_unit<kFormF32, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   } else if constexpr (PREC == HARU_INT16_ACC32) {
@@ -968,8 +968,11 @@ __device__ __forceinline__ void sweep_any(const SdtwArgs &A, TileStream &ts, int
     sweep_unit<kFormF32Span, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   } else if constexpr (PREC == kPrecWideSpan) {
     sweep_unit<kFormWideSpan, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
-  } else if constexpr (PREC == kPrecI16Large) {
-    sweep_unit<kFormI16Large, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
+  } else if constexpr (PREC == kPrecI16Mixed) {
+    if (large)
+      sweep_unit<kFormI16Large, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
+    else
+      sweep_unit<kFormI16, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   } else {
     sweep_unit<kFormI16, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
   }
@@ -1004,12 +1007,13 @@ __device__ __forceinline__ bool wait_part(const SdtwArgs &A, int cta, unsigned l
 // for the tallest), fed by one longest-first queue of groups.
 template <int PREC, int S = 1>
 __device__ __forceinline__ void dispatch_sweep(int s, const SdtwArgs &A, TileStream &ts, int nseg, int seg,
-                                               long p_lo, long p_hi, int item, uint32_t *ring, int lane) {
+                                               long p_lo, long p_hi, int item, bool large, uint32_t *ring,
+                                               int lane) {
   if constexpr (S <= kMaxS) {
     if (s == S)
-      sweep_any<PREC, S>(A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
+      sweep_any<PREC, S>(A, ts, nseg, seg, p_lo, p_hi, item, large, ring, lane);
     else
-      dispatch_sweep<PREC, S + 1>(s, A, ts, nseg, seg, p_lo, p_hi, item, ring, lane);
+      dispatch_sweep<PREC, S + 1>(s, A, ts, nseg, seg, p_lo, p_hi, item, large, ring, lane);
   }
 }
 
@@ -1017,8 +1021,6 @@ __device__ __forceinline__ void dispatch_sweep(int s, const SdtwArgs &A, TileStr
 // fit in 168 registers a thread; the start-column strips (~240) up to 8.
 template <int PREC>
 __host__ __device__ constexpr int cta_threads() { return prec_span(PREC) ? 256 : 384; }
-template <int PREC>
-__host__ __device__ constexpr bool pairs() { return PREC == HARU_INT16 || PREC == kPrecI16Large; }
 
 // The CTA's shared state and this warp's tile slots; layout: Shared |
 // per-warp tracking rings | two tile slots per stream.
@@ -1037,14 +1039,14 @@ __device__ __forceinline__ void init_shared(Shared *sh) {
 }
 template <int PREC>
 __device__ __forceinline__ TileStream stream_of(const SdtwArgs &A, Shared *sh, int stream, int S, long p_lo, long p_hi,
-                                                int n_active) {
+                                                int n_active, bool large) {
   char *slots = reinterpret_cast<char *>(sh) + kSharedHeader + A.warps * ring_words(PREC) * 4;
   const int TS = tile_width(A.tile_cols);
   TileStream ts;
   ts.sh = &sh->streams[stream];
   ts.abort = &sh->abort;
   ts.slots = slots + static_cast<size_t>(stream) * 2 * (A.tile_cols + kRefFront) * 4;
-  ts.src = reinterpret_cast<const char *>(PREC == kPrecI16Large ? A.ref_large : A.ref_img);
+  ts.src = reinterpret_cast<const char *>(PREC == kPrecI16Mixed && large ? A.ref_large : A.ref_img);
   ts.tile_cols = TS;
   ts.k_first = static_cast<int>(p_lo / TS);
   ts.K = static_cast<int>((p_hi + TS - 1) / TS - p_lo / TS);
@@ -1075,34 +1077,25 @@ __global__ void __launch_bounds__(cta_threads<PREC>(), 1) queue_kernel(SdtwArgs 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   init_shared(sh);
   const int count = A.ints[kIntGroups];
-  int *queue = A.ints + (PREC == kPrecI16Large ? kIntQueueLarge : kIntQueue);
   for (;;) {
-    if (threadIdx.x == 0) sh->group = atomicAdd(queue, 1);
+    if (threadIdx.x == 0) sh->group = atomicAdd(A.ints + kIntQueue, 1);
     __syncthreads();
     const int gi = sh->group;
     if (gi >= count || sh->abort) break;
     const Group grp = A.groups[gi];
-    if constexpr (pairs<PREC>()) {
-      // A group with a code too large for the half-code cell belongs to the
-      // large-code sweep, every other one to this form's.
-      bool large = false;
-      if (A.large_possible)
-        large = __any_sync(kFull, A.items[grp.first + min(lane, grp.count - 1)].qmax > A.half_max);
-      if (large != (PREC == kPrecI16Large)) {
-        __syncthreads();  // every thread has read sh->group
-        continue;
-      }
-    }
+    bool large = false;  // the group holds a code too large for the half-code cell
+    if constexpr (PREC == kPrecI16Mixed)
+      large = __any_sync(kFull, A.items[grp.first + min(lane, grp.count - 1)].qmax > A.half_max);
     long t_start, t_own, t_end;
     seg_bounds(grp.S, grp.nseg, grp.seg, A.N, &t_start, &t_own, &t_end);
-    TileStream ts = stream_of<PREC>(A, sh, 0, grp.S, t_start, t_end, grp.count);
+    TileStream ts = stream_of<PREC>(A, sh, 0, grp.S, t_start, t_end, grp.count, large);
     if (threadIdx.x == 0) {
       ts.issue(0);
       if (ts.K > 1) ts.issue(1);
     }
     __syncthreads();
     if (warp < grp.count)
-      dispatch_sweep<PREC>(grp.S, A, ts, grp.nseg, grp.seg, t_start, t_end, grp.first + warp,
+      dispatch_sweep<PREC>(grp.S, A, ts, grp.nseg, grp.seg, t_start, t_end, grp.first + warp, large,
                            rings + warp * ring_words(PREC), lane);
     __syncthreads();
     if (threadIdx.x == 0) ts.sh->tile_base += ts.K;
@@ -1145,7 +1138,7 @@ __global__ void __launch_bounds__(cta_threads<PREC>(), 1) sdtw_kernel(SdtwArgs A
   // This CTA's place on the line, in the order the CTAs started, and the
   // bundles first .. first + n - 1 that its stretch touches.
   const Schedule &sched = sh->sched;
-  if (threadIdx.x == 0) sh->group = atomicAdd(A.ints + (PREC == kPrecI16Large ? kIntQueueLarge : kIntQueue), 1);
+  if (threadIdx.x == 0) sh->group = atomicAdd(A.ints + kIntQueue, 1);
   for (int i = threadIdx.x; i < static_cast<int>(sizeof(Schedule) / 4); i += blockDim.x)
     reinterpret_cast<int *>(&sh->sched)[i] = reinterpret_cast<const int *>(A.sched)[i];
   init_shared(sh);
@@ -1166,14 +1159,9 @@ __global__ void __launch_bounds__(cta_threads<PREC>(), 1) sdtw_kernel(SdtwArgs A
     const int members = i + 1 < row.bundles ? sched.members : row.last;
     const int u0 = i * sched.members, u = u0 + min(warp, members - 1);  // this warp's unit
     const int item = row.base + u % row.items, seg = u / row.items, nseg = row.nseg;
-    if constexpr (pairs<PREC>()) {
-      // A bundle with a code too large for the half-code cell belongs to the
-      // large-code sweep, every other one to this form's.
-      bool large = false;
-      if (A.large_possible)
-        large = __any_sync(kFull, A.items[row.base + (u0 + min(lane, members - 1)) % row.items].qmax > A.half_max);
-      if (large != (PREC == kPrecI16Large)) continue;
-    }
+    bool large = false;  // the bundle holds a code too large for the half-code cell
+    if constexpr (PREC == kPrecI16Mixed)
+      large = __any_sync(kFull, A.items[row.base + (u0 + min(lane, members - 1)) % row.items].qmax > A.half_max);
     long t_start, t_own, t_end;
     seg_bounds(S, nseg, seg, A.N, &t_start, &t_own, &t_end);
     const long p_lo = t_start + cut_steps(t_start, t_end, cut_lo, cost);
@@ -1188,13 +1176,13 @@ __global__ void __launch_bounds__(cta_threads<PREC>(), 1) sdtw_kernel(SdtwArgs A
     // (after a wait that gave up, this CTA's streams are not used again)
     const bool runs = warp < members && p_lo < p_hi && !__any_sync(kFull, *static_cast<volatile int *>(&sh->abort));
     if (runs) {
-      TileStream ts = stream_of<PREC>(A, sh, warp, S, p_lo, p_hi, 1);
+      TileStream ts = stream_of<PREC>(A, sh, warp, S, p_lo, p_hi, 1, large);
       if (lane == 0) {
         ts.issue(0);
         if (ts.K > 1) ts.issue(1);
       }
       __syncwarp();
-      dispatch_sweep<PREC>(S, A, ts, nseg, seg, p_lo, p_hi, item, rings + warp * ring_words(PREC), lane);
+      dispatch_sweep<PREC>(S, A, ts, nseg, seg, p_lo, p_hi, item, large, rings + warp * ring_words(PREC), lane);
       __syncwarp();
       if (lane == 0) ts.sh->tile_base += ts.K;
     }
@@ -1561,7 +1549,7 @@ int occupancy_prec(int tile_cols, int warps) {
 
 // Define the entry points of a kernel for kernel precision P (0 FP32, 1
 // INT16, 2 int16 inputs with wide accumulation, 3 FP32 with start columns, 4
-// wide with start columns, 5 INT16 groups with large codes): the scheduled
+// wide with start columns, 5 INT16 with both cells): the scheduled
 // sweep, the queue's sweep, the segment fix-up, the trace. One per
 // translation unit, so the kernels compile in parallel.
 #define HARU_SDTW_SWEEP_INSTANCE(P)                                                                        \
