@@ -166,7 +166,14 @@ int haru_create(haru_ctx **out, int device, const haru_config *cfg) {
     if (cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking) != cudaSuccess) { rc = HARU_ECUDA; break; }
     size_t ci = 0;
     if (grow(&ctx->ws.ints, &ci, (size_t)haru::kIntWords) != cudaSuccess) { rc = HARU_ENOMEM; break; }
+    // (haru_last_status and haru_last_stats before the first batch)
+    if (cudaMemsetAsync(ctx->ws.ints, 0, haru::kIntWords * sizeof(int), ctx->stream) != cudaSuccess ||
+        cudaStreamSynchronize(ctx->stream) != cudaSuccess) {
+      rc = HARU_ECUDA;
+      break;
+    }
     if (cudaMalloc(&ctx->stats, 2 * sizeof(double)) != cudaSuccess) { rc = HARU_ENOMEM; break; }
+    if (cudaMalloc(&ctx->ref_words, 2 * sizeof(int)) != cudaSuccess) { rc = HARU_ENOMEM; break; }
     if (cudaMallocHost(&ctx->stage, haru::kStageBytes) != cudaSuccess) { rc = HARU_ENOMEM; break; }
     bool ev_ok = true;
     for (auto &e : ctx->ev) ev_ok = ev_ok && cudaEventCreate(&e) == cudaSuccess;
@@ -202,9 +209,9 @@ void haru_destroy(haru_ctx *ctx) {
     ctx->server = nullptr;
   }
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-  void *ptrs[] = {ctx->ref_z,     ctx->stats,       ctx->partials,    ctx->d_events,   ctx->d_offsets,
-                  ctx->d_cost,    ctx->d_col,       ctx->d_start,     ctx->d_samples,  ctx->d_soff,
-                  ctx->sig_strided, ctx->sig_events, ctx->sig_counts, ctx->sig_off};
+  void *ptrs[] = {ctx->ref_z,     ctx->stats,       ctx->ref_words,   ctx->partials,   ctx->d_events,
+                  ctx->d_offsets, ctx->d_cost,      ctx->d_col,       ctx->d_start,    ctx->d_samples,
+                  ctx->d_soff,    ctx->sig_strided, ctx->sig_events,  ctx->sig_counts, ctx->sig_off};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (ctx->stage) cudaFreeHost(ctx->stage);
@@ -241,19 +248,18 @@ static int ref_install(haru_ctx *ctx, const float *x_dev, size_t n, int normaliz
   uint32_t *i16 = i16b + haru::kRefFront, *ih = ihb + haru::kRefFront;
   float *i32 = i32b + haru::kRefFront;
   const size_t nb = (n + 4095) / 4096;
-  // status, and the largest |code| in the words after it
-  int st[2] = {0, 0};
+  int st[2] = {0, 0};  // ref_words: status, largest |code|
   e = grow(&ctx->partials, &ctx->partials_cap, nb);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws.ints, 0, sizeof(st), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ref_words, 0, sizeof(st), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(i16b, 0, all * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(ihb, 0, all * sizeof(uint32_t), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(i32b, 0, all * sizeof(float), s);
   if (e == cudaSuccess && normalize)
-    e = haru::launch_zscore_stats(x_dev, n, ctx->partials, ctx->stats, ctx->ws.ints, s);
+    e = haru::launch_zscore_stats(x_dev, n, ctx->partials, ctx->stats, ctx->ref_words, s);
   if (e == cudaSuccess)
-    e = haru::launch_ref_finish(x_dev, n, ctx->stats, normalize, scale_log2, z, i16, ih, i32, ctx->ws.ints,
-                                ctx->ws.ints + 1, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(st, ctx->ws.ints, sizeof(st), cudaMemcpyDeviceToHost, s);
+    e = haru::launch_ref_finish(x_dev, n, ctx->stats, normalize, scale_log2, z, i16, ih, i32, ctx->ref_words,
+                                ctx->ref_words + 1, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(st, ctx->ref_words, sizeof(st), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess || st[0] != HARU_OK) {  // the previous reference stays in place
     const int rc = e != cudaSuccess ? cuda_fail(ctx, e) : st[0];
@@ -322,10 +328,10 @@ int haru_ref_build(haru_ctx *ctx, const uint8_t *bases, size_t n_bases, const fl
   cudaStream_t s = ctx->stream;
   e = cudaMemcpyAsync(db, bases, n_bases, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dm, kmer_levels, nmodel * sizeof(float), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws.ints, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = haru::launch_ref_levels(db, n_bases, dm, k, x, ctx->ws.ints, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ref_words, 0, sizeof(int), s);
+  if (e == cudaSuccess) e = haru::launch_ref_levels(db, n_bases, dm, k, x, ctx->ref_words, s);
   int st = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&st, ctx->ws.ints, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&st, ctx->ref_words, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess)
     rc = cuda_fail(ctx, e);

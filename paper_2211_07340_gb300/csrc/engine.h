@@ -191,6 +191,10 @@ struct haru_ctx {
   int max_code = 0;             // largest |q|
   float *img32 = nullptr;       // N + kRefPad
   double *stats = nullptr;      // mean, sigma
+  // Status and largest code of the reference being prepared: apart from the
+  // batches' words (ws.ints), which a batch still queued on a caller's stream
+  // may be using.
+  int *ref_words = nullptr;
   double *partials = nullptr;
   size_t partials_cap = 0;
 
