@@ -436,8 +436,8 @@ int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float *events, c
  * best of those, every stack_short rule (auto, always, never: 32-lane strips
  * or stacked 16-lane strips of twice the rows per lane for queries of <= 256
  * events), keep the fastest (minimum of two timed runs each) in the context's
- * configuration for later batches, and copy the resulting configuration to *chosen (may be
- * NULL). The strip height is fixed by each query's length. Results of the
+ * configuration for later batches (with ctas_per_sm = 0 where that is the cost
+ * model), and copy the resulting configuration to *chosen (may be NULL). The strip height is fixed by each query's length. Results of the
  * trial runs are discarded. Errors: as haru_sdtw_batch. */
 int haru_autotune(haru_ctx *ctx, int precision, const float *events, const uint32_t *offsets, uint32_t nq,
                   uint32_t flags, haru_config *chosen);

@@ -134,6 +134,8 @@ extern "C" int haru_autotune(haru_ctx *ctx, int precision, const float *events, 
   ctx->cfg.warps_per_cta = best.warps;
   ctx->cfg.tile_cols = best.tile;
   ctx->cfg.units_target = best.units_target;
+  // (the planner's own schedule ran without the context's CTA count, which would select the queue)
+  ctx->cfg.ctas_per_sm = best.ctas_per_sm;
   ctx->cfg.stack_short = best.stack_short;
   if (chosen) *chosen = ctx->cfg;
   return HARU_OK;
