@@ -197,6 +197,7 @@ cudaError_t ws_reserve_upto(Workspace &ws, int precision, uint32_t max_nq, const
     most.ctas = std::max(most.ctas, w.ctas);
     most.qstats = std::max(most.qstats, w.qstats);
     most.states = std::max(most.states, w.states);
+    most.checkpoints = std::max(most.checkpoints, w.checkpoints);
   }
   return ws_alloc(ws, most);
 }
