@@ -194,7 +194,7 @@ int haru_sdtw_batch(haru_ctx *ctx, int precision, const float *events, const uin
  * columns are computed as in haru_sdtw_batch and the starts are then carried
  * only along the columns before each end, from exact states saved on the way
  * (about 1.2x the time of haru_sdtw_batch and up to 512 MB more device
- * memory, 32 KB per query in batches of over 16,384); on shorter ones they
+ * memory, 32 KB per query in batches of over 16,384, 16 KB from 2^22 on); on shorter ones they
  * are carried through the whole sweep, a reference segment being kept only if
  * both its costs and its start columns match. */
 int haru_sdtw_batch_span(haru_ctx *ctx, int precision, const float *events, const uint32_t *offsets, uint32_t nq,

@@ -24,6 +24,20 @@ void ws_free(Workspace &ws) {
   ws = Workspace();
 }
 
+// Checkpoints per item: up to 128 (a trace runs half the distance between two
+// of them on average beside two strip heights), fewer in batches whose
+// states would pass 512 MB, at least 8; at least 256 steps apart. From
+// kFewCheckpoints items on 4 do: 8 take an item to 52 KB, a batch of 5.4 M
+// queries to the whole memory, 4 to 36 (1.1 M x 100..120 events on 20,000
+// columns: 473 ms with 8, 590 with 4).
+constexpr size_t kFewCheckpoints = 1u << 22;
+int checkpoint_cap(size_t max_items, long N) {
+  const size_t fit = (static_cast<size_t>(512) << 20) / (max_items * kStateStride * sizeof(uint32_t));
+  const size_t least = max_items < kFewCheckpoints ? 8 : 4;
+  const long most = std::min<long>(std::min<size_t>(std::max(fit, least), 128), (N + 32 * kMaxS) / 256);
+  return static_cast<int>(std::max<long>(most, 1));
+}
+
 namespace {
 
 // Tile of a warp's own stream: two slots of (kSoloTile + kRefFront) words and
@@ -74,14 +88,8 @@ int cost_form(int precision) {
   return precision == kPrecF32Span ? HARU_FP32 : (precision == kPrecWideSpan ? HARU_INT16_ACC32 : precision);
 }
 
-// Checkpoints per item: up to 128 (a trace runs half the distance between two
-// of them on average beside two strip heights), fewer in batches whose
-// states would pass 512 MB, at least 8; at least 256 steps apart.
-int checkpoint_cap(size_t max_items, long N) {
-  const size_t fit = (static_cast<size_t>(512) << 20) / (max_items * kStateStride * sizeof(uint32_t));
-  const long most = std::min<long>(std::min<size_t>(std::max<size_t>(fit, 8), 128), (N + 32 * kMaxS) / 256);
-  return static_cast<int>(std::max<long>(most, 1));
-}
+constexpr size_t kTwoSegments = 16;
+
 int checkpoint_step(int cap, long N) { return static_cast<int>((N + 32 * kMaxS + cap) / cap); }
 
 WsNeeds ws_needs(int precision, uint32_t nq, const LaunchCfg &lc) {
@@ -100,9 +108,13 @@ WsNeeds ws_needs(int precision, uint32_t nq, const LaunchCfg &lc) {
     const size_t units = static_cast<size_t>(stack_units(precision, lc));
     w.nseg_cap = static_cast<int>(std::min<size_t>(64, 2 * ((units + items_min - 1) / items_min)));
   } else {
-    // the cost model spreads a batch over at most about two units per resident warp
+    // The cost model spreads a batch over at most about two units per resident
+    // warp. From kTwoSegments items per resident warp on, a third segment buys
+    // no balance (60,000 x 100..500 FP32 events on 6,000 columns: 15.2 ms with
+    // two and with three) and its states cost 8 KB of an item's 28.
     const size_t resident = static_cast<size_t>(lc.sms) * sh.per_sm * sh.warps;
     w.nseg_cap = static_cast<int>(std::min<size_t>(kMaxSeg, 2 + (2 * resident + items_min - 1) / items_min));
+    if (items_min >= kTwoSegments * resident) w.nseg_cap = 2;
   }
   w.units = w.max_items * static_cast<size_t>(w.nseg_cap);
   w.ctas = static_cast<size_t>(lc.sms) * sh.per_sm;

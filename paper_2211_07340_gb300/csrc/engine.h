@@ -120,6 +120,8 @@ struct Workspace {
   int nseg_cap = 1;
 };
 
+// Checkpoints per item of a traced start-column batch (batch.cu).
+int checkpoint_cap(size_t max_items, long N);
 // Size `ws` for a batch of nq queries (allocates only when it must grow).
 cudaError_t ws_reserve(Workspace &ws, int precision, uint32_t nq, const LaunchCfg &lc);
 // Size `ws` for every batch of 1..max_nq queries at once, so that later

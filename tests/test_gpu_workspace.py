@@ -52,3 +52,33 @@ def test_reserve_upto_covers_every_smaller_batch(tmp_path, n):
   }
   return 0;""" % n)
     assert out.split() == ["0"] * 5
+
+
+# (precision, device bytes a query at most: what a batch of this size took before the static schedule, whose third
+# segment must not cost a caller at the memory's end the batch)
+@pytest.mark.parametrize("prec,most", [("HARU_FP32", 22_800), ("HARU_INT16", 11_500)])
+def test_memory_of_very_large_batches(tmp_path, prec, most):
+    nq = 1 << 20
+    out = run(tmp_path, """
+  LaunchCfg lc;
+  lc.sms = 152;
+  lc.N = 59796;
+  Workspace ws;
+  size_t before, after, all;
+  cudaFree(nullptr);
+  cudaMemGetInfo(&before, &all);
+  if (ws_reserve(ws, %s, %du, lc) != cudaSuccess) return 1;
+  cudaMemGetInfo(&after, &all);
+  std::printf("%%zu", before - after);
+  ws_free(ws);
+  return 0;""" % (prec, nq))
+    assert int(out) <= nq * most
+
+
+def test_checkpoints_of_very_large_batches(tmp_path):
+    """Beside 20.3 KB of other buffers an item (above) 4 checkpoints of 4 KB stay below the 39,100 bytes a start-column
+    query took before there were any."""
+    out = run(tmp_path, """
+  std::printf("%d %d", checkpoint_cap((1u << 22) - 1, 59796), checkpoint_cap(1u << 22, 59796));
+  return 0;""")
+    assert out.split() == ["8", "4"]
