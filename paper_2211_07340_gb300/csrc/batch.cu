@@ -248,7 +248,7 @@ cudaError_t ws_enqueue(Workspace &ws, int precision, const RefView &ref, const f
   pa.ints = ws.ints;
   // (a caller that ran kernels reporting into the status word first has zeroed the counters itself)
   pa.zero = zero_counters;
-  if ((e = launch_prep(pa, d_events, raw ? ws.qstats : nullptr, s)) != cudaSuccess) return e;
+  if ((e = launch_prep(pa, d_events, raw ? ws.qstats : nullptr, lc.sms, s)) != cudaSuccess) return e;
 
   PackArgs ka;
   ka.events = d_events;

@@ -306,8 +306,9 @@ struct PackArgs {
 
 // Kernel launchers (stream-ordered, no synchronisation).
 // The plan and, on raw events (qstats != nullptr), the mean and population
-// sigma (FP64, sequential order) of each query of 1..512 events.
-cudaError_t launch_prep(const PlanArgs &a, const float *events, double *qstats, cudaStream_t s);
+// sigma (FP64, sequential order) of each query of 1..512 events. sms: of the
+// device.
+cudaError_t launch_prep(const PlanArgs &a, const float *events, double *qstats, int sms, cudaStream_t s);
 cudaError_t launch_pack(const PackArgs &a, uint32_t max_items, cudaStream_t s);
 cudaError_t launch_sdtw(int precision, const SdtwArgs &a, int grid, int fix_items, cudaStream_t s,
                         cudaEvent_t ev_fix = nullptr);

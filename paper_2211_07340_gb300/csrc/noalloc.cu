@@ -118,7 +118,7 @@ extern "C" int haru_sdtw_batch_noalloc(haru_ctx *ctx, int precision, const float
   pa.groups = groups;
   pa.ints = status;
   pa.zero = 1;
-  if ((e = launch_prep(pa, events, (flags & HARU_RAW) ? qstats : nullptr, s)) != cudaSuccess)
+  if ((e = launch_prep(pa, events, (flags & HARU_RAW) ? qstats : nullptr, sms, s)) != cudaSuccess)
     return ctx_cuda_fail(ctx, e);
   PackArgs ka;
   ka.events = events;

@@ -511,7 +511,7 @@ struct StatArgs {
   const float *events;
   const uint32_t *offsets;
   uint32_t nq;
-  int per_block;  // queries, 32 or 64
+  int per_block;  // queries: 8, 32 or 64
   double *qstats;
 };
 
@@ -725,12 +725,14 @@ __global__ void pack_kernel(PackArgs a) {
 
 }  // namespace
 
-cudaError_t launch_prep(const PlanArgs &a, const float *events, double *qstats, cudaStream_t s) {
+cudaError_t launch_prep(const PlanArgs &a, const float *events, double *qstats, int sms, cudaStream_t s) {
   StatArgs st{events, a.offsets, a.nq, kStatQueries, qstats};
-  // As few queries to a block as run at once: the chains share the
-  // double-precision unit with the squares of their block's queries.
+  // As few queries to a block as leave a block to an SM: the chains share the
+  // SM's double-precision unit with the squares of their block's queries.
+  // Eight SMs (of 152) stay free of them, one of which runs the planner's block.
+  const uint32_t blocks_at_once = static_cast<uint32_t>(sms > 16 ? sms - 8 : 8);
   for (int k : {32, 8})
-    if (a.nq <= static_cast<uint32_t>(k) * 144u) st.per_block = k;
+    if (a.nq <= static_cast<uint32_t>(k) * blocks_at_once) st.per_block = k;
   const unsigned blocks = qstats ? (a.nq + st.per_block - 1) / st.per_block : 0;
   prep_kernel<<<1 + blocks, 1024, 0, s>>>(a, st);
   return cudaGetLastError();
