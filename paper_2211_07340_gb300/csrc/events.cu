@@ -49,8 +49,8 @@ static_assert(kEvTpos > 4 * kEvMaxW, "a tile longer than its halos");
 // as many ints as the query needs (trim + max_events).
 constexpr size_t kSmX = 0;                                                    // int16 samples, up to 7 in front
 constexpr size_t kSmT = kSmX + (HARU_MAX_READ_SAMPLES + 8) * sizeof(int16_t);  // 2 x (kEvTpos + 2 kEvPad) float t^2
-constexpr size_t kSmLp = kSmT + 2 * (kEvTpos + 2 * kEvPad) * sizeof(float);   // long-peak bits, one word on each side
-constexpr size_t kSmBounds = kSmLp + (kEvTpos / 32 + 2 + 2) / 4 * 4 * sizeof(unsigned);
+constexpr size_t kSmLp = kSmT + 2 * (kEvTpos + 2 * kEvPad) * sizeof(float);   // long-peak bits, one word behind them
+constexpr size_t kSmBounds = kSmLp + (kEvTpos / 32 + 1 + 3) / 4 * 4 * sizeof(unsigned);
 size_t detect_smem_bytes(int need) { return kSmBounds + static_cast<size_t>(need) * sizeof(int); }
 
 struct EvArgs {
@@ -305,7 +305,7 @@ __device__ __forceinline__ unsigned peaks_of(const int16_t *x, const float *tf, 
 __global__ void __launch_bounds__(kEvThreads, 3) detect_kernel(EvArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
   float *t1 = reinterpret_cast<float *>(sm + kSmT) + kEvPad, *t2 = t1 + kEvTpos + 2 * kEvPad;
-  unsigned *lp = reinterpret_cast<unsigned *>(sm + kSmLp) + 1;  // long-peak bit of statistic j: word j / 32
+  unsigned *lp = reinterpret_cast<unsigned *>(sm + kSmLp);  // long-peak bit of statistic j: word j / 32
   int *bounds = reinterpret_cast<int *>(sm + kSmBounds);
   __shared__ int warp_tot[kEvThreads / 32], warp_min[kEvThreads / 32], warp_max[kEvThreads / 32];
   __shared__ int s_nb;
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kEvThreads, 3) detect_kernel(EvArgs a) {
     t1[tid - kEvPad] = t2[tid - kEvPad] = -1.0f;
     t1[kEvTpos + tid] = t2[kEvTpos + tid] = -1.0f;
   }
-  if (tid == 0) lp[-1] = lp[kEvTpos / 32] = 0u;
+  if (tid == 0) lp[kEvTpos / 32] = 0u;
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < kEvThreads / 32; ++w) {
@@ -410,12 +410,11 @@ __global__ void __launch_bounds__(kEvThreads, 3) detect_kernel(EvArgs a) {
 #pragma unroll
       for (int u = 0; u < kEvPer; ++u) {
         if (!((cand >> u) & 1u)) continue;
-        // no long peak at j - w1 .. j + w1
-        const int from = j0 + u - w1, at = from >> 5, sh = from & 31;  // (from >= -kEvMaxW: word -1)
+        // no long peak at j - w1 .. j + w1 (j >= H: from the statistic w2 on)
+        const int from = j0 + u - w1, at = from >> 5, sh = from & 31;
         const unsigned long long two = lp[at] | (static_cast<unsigned long long>(lp[at + 1]) << 32);
-        unsigned long long near = (two >> sh) & ((1ull << min(2 * w1 + 1, 64 - sh)) - 1ull);
-        if (2 * w1 + 1 > 64 - sh) near |= lp[at + 2] & ((1u << (2 * w1 + 1 - (64 - sh))) - 1u);
-        if (near == 0ull) flags |= 1u << u;
+        static_assert(2 * kEvMaxW + 1 <= 64 - 31, "the window's bits lie within two words");
+        if (((two >> sh) & ((1ull << (2 * w1 + 1)) - 1ull)) == 0ull) flags |= 1u << u;
       }
     }
     const int cnt = __popc(flags);
