@@ -56,10 +56,10 @@ constexpr int kSoloTile = 1536;
 struct StepClocks {
   float full[kMaxS], stacked, two, one;
 };
-const StepClocks kStepI16 = {{18.5f, 18.5f, 22.3f, 26.1f, 32.6f, 36.8f, 41.8f, 46.4f, 51.6f, 56.5f, 61.1f, 66.9f,
-                              71.7f, 74.0f, 79.5f, 84.7f}, 2.0f, 5.0f, 23.0f};
-const StepClocks kStepF32 = {{16.8f, 15.4f, 18.5f, 21.0f, 25.7f, 31.6f, 36.0f, 39.3f, 44.7f, 48.7f, 53.6f, 56.7f,
-                              62.5f, 66.2f, 70.7f, 75.8f}, 1.4f, 4.0f, 13.5f};
+const StepClocks kStepI16 = {{18.2f, 18.1f, 22.2f, 25.7f, 33.7f, 35.6f, 43.4f, 45.2f, 50.6f, 56.1f, 62.2f, 65.2f,
+                              70.1f, 75.9f, 81.1f, 84.6f}, 0.8f, 5.0f, 23.0f};
+const StepClocks kStepF32 = {{16.8f, 15.3f, 18.2f, 20.8f, 26.2f, 30.5f, 36.6f, 38.6f, 45.1f, 48.1f, 53.8f, 56.6f,
+                              61.5f, 65.1f, 70.2f, 74.7f}, 0.4f, 4.0f, 13.5f};
 const StepClocks &step_clocks(int precision) {
   return precision == HARU_INT16 ? kStepI16 : kStepF32;
 }
