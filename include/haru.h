@@ -85,7 +85,8 @@ typedef struct {
 
 typedef struct {
   /* launch shape of batches with an explicit units_target or ctas_per_sm, and of start-column batches (the
-   * default, units_target = 0 and ctas_per_sm = 0, spreads a batch by the planner's cost model instead) */
+   * default, units_target = 0 and ctas_per_sm = 0, spreads a batch by the planner's cost model instead, on
+   * references of 512 columns and more) */
   int warps_per_cta;        /* warps (queries or query pairs) sharing one reference tile stream: 2, 4, 8
                                or 12 (start-column batches run at most 8); other values = 8 */
   int tile_cols;            /* reference columns per shared-memory tile, 2048..16384; 0 = auto */

@@ -164,7 +164,12 @@ cudaError_t ws_alloc(Workspace &ws, const WsNeeds &w) {
 // unit target or CTA count, and the start-column forms (two strip heights of
 // whose code do not fit the cache together: 512 uneven queries took 5.4 ms,
 // 4.1 from the queue), run the configured shape: groups from a queue, each
-// sharing one stream of configured tiles.
+// sharing one stream of configured tiles. So do references of fewer than
+// kScheduleColumns: a sweep as short as a strip is high leaves nothing to cut,
+// and the schedule's own cost shows (20 x 30..200 FP32 z-values on 300
+// columns: 58 us scheduled, 39 from the queue; on 600 columns 8..3,000
+// queries of one length still gain 5% from the schedule, uneven ones lose 3%).
+constexpr long kScheduleColumns = 512;
 BatchShape batch_shape(int precision, uint32_t nq, const LaunchCfg &lc) {
   BatchShape sh;
   const long seg_room = std::min<long>(64, lc.N / 8192);
@@ -180,7 +185,7 @@ BatchShape batch_shape(int precision, uint32_t nq, const LaunchCfg &lc) {
   sh.solo = false;
   sh.per_sm = lc.ctas_per_sm > 0 ? lc.ctas_per_sm : 0;
   if (sh.per_sm == 0) sh.per_sm = sdtw_max_ctas_per_sm(precision, sh.tile, sh.warps);
-  if (lc.units_target == 0 && lc.ctas_per_sm == 0 && !prec_span(precision)) {
+  if (lc.units_target == 0 && lc.ctas_per_sm == 0 && !prec_span(precision) && lc.N >= kScheduleColumns) {
     sh.solo = true;
     sh.warps = kMaxWarps;
     sh.tile = kSoloTile;
