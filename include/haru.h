@@ -93,7 +93,9 @@ typedef struct {
   int ctas_per_sm;          /* persistent CTAs per SM; 0 = as many as fit */
   uint32_t wait_limit;      /* longest single device wait, microseconds, before HARU_ETIMEDOUT; 0 = 2 s;
                                values below 1000 act as 1000 (a timed-out CTA's drain of its copies in
-                               flight shares the limit and must outlast a tile copy) */
+                               flight shares the limit and must outlast a tile copy). The wait for
+                               another CTA's part of a sweep that the two share may take 1 us longer per
+                               reference column: the part may rightly run that long */
   /* serving */
   float threshold;          /* accept iff cost <= threshold (z units; int16 compares floor(threshold * 2^k)) */
   int serve_precision;      /* HARU_FP32 or HARU_INT16 */
@@ -194,7 +196,7 @@ int haru_sdtw_batch(haru_ctx *ctx, int precision, const float *events, const uin
  * HARU_ON_DEVICE. On references of 2,048 columns and more the costs and end
  * columns are computed as in haru_sdtw_batch and the starts are then carried
  * only along the columns before each end, from exact states saved on the way
- * (about 1.2x the time of haru_sdtw_batch and up to 512 MB more device
+ * (about 1.3x the time of haru_sdtw_batch and up to 512 MB more device
  * memory, 32 KB per query in batches of over 16,384, 16 KB from 2^22 on); on shorter ones they
  * are carried through the whole sweep, a reference segment being kept only if
  * both its costs and its start columns match. */

@@ -121,8 +121,9 @@ struct Group {
 // The static schedule of a batch planned by the cost model. Units (item x
 // segment, segment-major) of each strip height form bundles of `members`, run
 // by a CTA's warps side by side; the few items beyond the last full bundle
-// (`rest`) are cut into segments of their own so that theirs are full too. The bundles' estimated times, tallest strips
-// first, lie end to end on one line, and CTA p runs the line's stretch
+// (`rest`) are cut into segments of their own so that theirs are full too. The
+// bundles' estimated times, tallest strips first, lie end to end on one line,
+// and CTA p runs the line's stretch
 // [p * share, (p + 1) * share). No bundle is longer than a share, so at most
 // one crosses each border: the CTA before the border runs the bundle's first
 // steps before anything else, the one after it the remaining steps from the

@@ -4,7 +4,8 @@
 // Layout of one warp's work. A query of M events is padded at the top to
 // 32 * S rows (S = floor(M / 32) + 1, at most 16, so that a strip lower than
 // 16 rows per lane has at least one pad row); lane l holds rows l*S .. l*S + S - 1 in
-// registers. Row i processes reference column t - i at step t, so every row
+// registers (a stacked strip is two such strips of 16 * S rows, in lanes 0..15
+// and 16..31, each with its own lane 0). Row i processes reference column t - i at step t, so every row
 // is one processing element of the paper's PE chain and the whole strip is
 // one oblique column: the S cells of a lane in one step are independent
 // (instruction-level parallelism S), a cell reads
@@ -21,10 +22,12 @@
 // above is absorbed there, and only full-height strips (16 rows per lane,
 // no pad row) have lane 0 replace that value by the zero.
 //
-// INT16 form: two queries share a warp, one per 16-bit half (DPX
-// __viaddmax_s16x2_relu for |q - r|, __vimin3_u16x2, and __viaddmin_u16x2 on
-// the rows that saturate at CAP); pad rows hold 0. FP32 form: one query per warp, 3-input min.f32,
-// gamma = |d| + min3 with d = fma(r, w, q): w = -1 on real rows, 0 on pad rows (and q = 0 there).
+// INT16 form: two queries share a warp, one per 16-bit half: |q - r| by an
+// fp16x2 subtraction of half codes and a mask, __vimin3_u16x2, and an add, or
+// __viaddmin_u16x2 on the rows that saturate at CAP (codes too large for
+// halves: __vsub2 and __viaddmax_s16x2_relu); pad rows hold 0. FP32 form: one
+// query per warp, 3-input min.f32, gamma = |d| + min3 with d = fma(r, w, q):
+// w = -1 on real rows, 0 on pad rows (and q = 0 there).
 //
 // Segments. The steps of one query are cut into segments that run as
 // independent work units. Segment s > 0 starts V steps early from a fresh
@@ -41,17 +44,18 @@
 // on from it on the other one, so balance costs no further warm-up.
 //
 // The reference streams through shared memory, one stream per warp (a CTA's
-// warps run any units of one strip height), or, with an explicit unit
-// target, one per CTA (same S, same segment). Tiles of T_S columns, each with the kRefFront columns before it (the lanes lag the warp's step by
-// up to 31 * S columns), are fetched by cp.async.bulk (TMA) into a two-slot
-// ring guarded by mbarriers. The warp that releases a slot last issues the
+// warps run any units of one strip height), or, in the queue, one per CTA
+// (same S, same segment). Tiles of T_S columns, each with the kRefFront
+// columns before it (the lanes lag the warp's step by up to 31 * S columns),
+// are fetched by cp.async.bulk (TMA) into a two-slot ring guarded by mbarriers. The warp that releases a slot last issues the
 // copy of the tile two ahead.
 //
 // The last-row minimum and its first column (Algorithm 1's final scan,
 // Algorithm 2's per-column compare) are tracked through a small per-warp
-// shared ring: lane 31 stores its bottom-row cost every step, and every
-// <= 32 steps each lane scans one stored value; a warp reduction keeps the
-// smallest cost, then the smallest column.
+// shared ring: lane 31 (and lane 15 of a stacked strip) stores its bottom-row
+// cost of every step, and each time a flush buffer is full every lane scans
+// its two (int16) or four entries; a warp reduction keeps the smallest cost,
+// then the smallest column.
 //
 // Every wait is bounded by a global-timer deadline; on expiry the kernel
 // records HARU_ETIMEDOUT, waits (bounded) for its own copies in flight and
@@ -1004,7 +1008,7 @@ __device__ __forceinline__ bool wait_part(const SdtwArgs &A, int cta, unsigned l
 }
 
 // One kernel covers every strip height S = 1..16 (registers are allocated
-// for the tallest), fed by one longest-first queue of groups.
+// for the tallest).
 template <int PREC, int S = 1>
 __device__ __forceinline__ void dispatch_sweep(int s, const SdtwArgs &A, TileStream &ts, int nseg, int seg,
                                                long p_lo, long p_hi, int item, bool large, uint32_t *ring,
