@@ -297,11 +297,12 @@ __device__ __forceinline__ unsigned peaks_of(const int16_t *x, const float *tf, 
 }
 
 // Three CTAs per SM (80 registers a thread; with four and 64 it spilled and
-// ran the same). Each thread keeps kEvPer consecutive statistics of a tile from the window
-// sums to the boundaries; instruction bound (64 MB of samples in 8,192 reads
-// are 10 us of HBM time): 8,192 reads of 140..640 levels took 790 us with
-// 64-bit sums, products and divisions at every position and a neighbour loop
-// per candidate, 225 us this way.
+// ran the same). Each thread keeps kEvPer consecutive statistics of a tile
+// from the window sums to the boundaries. It issues in two cycles of three and
+// waits for fixed latencies, barriers and shared memory in the rest (64 MB of
+// samples in 8,192 reads are 10 us of HBM time): 8,192 reads of 140..640 levels
+// took 790 us with 64-bit sums, products and divisions at every position and a
+// neighbour loop per candidate, 213 us this way.
 __global__ void __launch_bounds__(kEvThreads, 3) detect_kernel(EvArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
   float *t1 = reinterpret_cast<float *>(sm + kSmT) + kEvPad, *t2 = t1 + kEvTpos + 2 * kEvPad;
